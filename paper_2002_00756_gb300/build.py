@@ -18,8 +18,8 @@ ROOT = os.path.dirname(HERE)
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
-SOURCES = ["mgsolve.cu", "mesh.cpp"]
-HEADERS = ["kernels.cuh", "krylov.cuh", "mesh.h"]
+SOURCES = ["mgsolve.cu", "sweep_f32.cu", "sweep_p64.cu", "sweep_bf16.cu", "mesh.cpp"]
+HEADERS = ["kernels.cuh", "krylov.cuh", "sweep32.cuh", "sweep64.cuh", "sweep_launch.cuh", "sweep_tma.cuh", "mesh.h"]
 
 
 def _nvcc() -> str:

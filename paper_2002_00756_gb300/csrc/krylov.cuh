@@ -106,24 +106,15 @@ __global__ void k_scale_volume(int ncol, int nlev, const double* __restrict__ ar
 // a_up(kf-1, c) dz[kf-1] (vertical).  Valid only for a flux-symmetric operator, V_i a_if = V_j a_jf:
 // the other cell's product must agree to 1e-10 relative, every coupling must be finite and
 // >= 0, and none may cross the surface or the lid.  A failed check sets *bad; with write the
-// kernels store the face form in every precision the handle holds (NULL arrays are skipped).
-struct CoefTargets {
-    double* Th64;
-    float* Th32;
-    __nv_bfloat16* Th16;
-    double* Tv64;
-    float* Tv32;
-    __nv_bfloat16* Tv16;
-};
-
+// kernels store the face form.
 __device__ __forceinline__ bool coef_close(double u, double v) {
     return fabs(u - v) <= 1e-10 * fmax(fabs(u), fabs(v));
 }
 
 __global__ void k_coef_faces(int ncol, int nlev, const int32_t* __restrict__ faceL, const int32_t* __restrict__ faceR,
                              const int32_t* __restrict__ faceSide, const int32_t* __restrict__ nbrSide,
-                             const double* __restrict__ area, const double* __restrict__ a, bool write, CoefTargets t,
-                             unsigned int* bad) {
+                             const double* __restrict__ area, const double* __restrict__ a, bool write,
+                             double* __restrict__ Th, unsigned int* bad) {
     const int f = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y, nf = 2 * ncol;
     if (f >= nf || k >= nlev) return;
     const size_t N = (size_t)nlev * ncol, o = (size_t)k * ncol;
@@ -131,14 +122,11 @@ __global__ void k_coef_faces(int ncol, int nlev, const int32_t* __restrict__ fac
     const double tl = a[s * N + o + L] * area[L], tr = a[sr * N + o + R] * area[R];
     if (!(tl >= 0.0) || !(tr >= 0.0) || !isfinite(tl) || !isfinite(tr) || !coef_close(tl, tr)) atomicOr(bad, 1u);
     if (!write) return;
-    const size_t e = (size_t)k * nf + f;
-    if (t.Th64) t.Th64[e] = tl;
-    if (t.Th32) t.Th32[e] = (float)tl;
-    if (t.Th16) t.Th16[e] = __float2bfloat16_rn((float)tl);
+    Th[(size_t)k * nf + f] = tl;
 }
 
 __global__ void k_coef_vertical(int ncol, int nlev, const double* __restrict__ dz, const double* __restrict__ a,
-                                bool write, CoefTargets t, unsigned int* bad) {
+                                bool write, double* __restrict__ Tv, unsigned int* bad) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x, kf = blockIdx.y;
     if (c >= ncol || kf > nlev) return;
     const size_t N = (size_t)nlev * ncol;
@@ -154,10 +142,7 @@ __global__ void k_coef_vertical(int ncol, int nlev, const double* __restrict__ d
         if (!(up >= 0.0) || !(dn >= 0.0) || !isfinite(tv) || !isfinite(ta) || !coef_close(tv, ta)) atomicOr(bad, 1u);
     }
     if (!write) return;
-    const size_t e = (size_t)kf * ncol + c;
-    if (t.Tv64) t.Tv64[e] = tv;
-    if (t.Tv32) t.Tv32[e] = (float)tv;
-    if (t.Tv16) t.Tv16[e] = __float2bfloat16_rn((float)tv);
+    Tv[(size_t)kf * ncol + c] = tv;
 }
 
 // a6[s][e] = a[s][e] (s < 6) and a6[6][e] = 1 + their sum: the FP64 operator of the GCR apply

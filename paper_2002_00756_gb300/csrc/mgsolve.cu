@@ -21,50 +21,12 @@
 #include "kernels.cuh"
 #include "krylov.cuh"
 #include "mesh.h"
-
-// tuning knobs of the sweep kernel (FP32 prefetch depths, threads per block)
-#ifndef MG_SWEEP_DEEP32
-#define MG_SWEEP_DEEP32 4
-#endif
-#ifndef MG_SWEEP_SHAL32
-#define MG_SWEEP_SHAL32 4
-#endif
-// residual + restriction on levels with n % 16 == 0: levels per thread, levels loaded ahead
-#ifndef MG_RESTRICT_KCHUNK
-#define MG_RESTRICT_KCHUNK 8
-#endif
-#ifndef MG_RESTRICT_KCHUNK_BIG
-#define MG_RESTRICT_KCHUNK_BIG 24
-#endif
-#ifndef MG_RESTRICT_BIG_NCOL
-#define MG_RESTRICT_BIG_NCOL 100000
-#endif
-#ifndef MG_RESTRICT_ASYNC
-#define MG_RESTRICT_ASYNC 1          // FP32 levels: own-column streams through a copy ring
-#endif
-#ifndef MG_RESTRICT_ASYNC_NCOL
-#define MG_RESTRICT_ASYNC_NCOL 40000 // smaller levels: the register ring alone is as fast
-#endif
-#ifndef MG_RESTRICT_DEEP
-#define MG_RESTRICT_DEEP 4
-#endif
-#ifndef MG_RESTRICT_ASHAL
-#define MG_RESTRICT_ASHAL 2
-#endif
-#ifndef MG_RESTRICT_SHAL
-#define MG_RESTRICT_SHAL 2
-#endif
-#ifndef MG_SWEEP_SHAL_PRO
-#define MG_SWEEP_SHAL_PRO 2
-#endif
-#ifndef MG_SWEEP_SHAL_ZERO
-#define MG_SWEEP_SHAL_ZERO 2
-#endif
-#ifndef MG_SWEEP_BLOCK
-#define MG_SWEEP_BLOCK 128
-#endif
+#include "sweep64.cuh"
+#include "sweep_tma.cuh"
 
 using mg::Lvl;
+using mg::Lvl32;
+using mg::Lvl64;
 typedef __nv_bfloat16 bf16;
 
 namespace {
@@ -74,15 +36,28 @@ struct DevLevel {
     int32_t* nbr = nullptr;
     int32_t* fof = nullptr;
     double* rA64 = nullptr;
-    float* rA32 = nullptr;
     double* Th64 = nullptr;
     double* Tv64 = nullptr;
+    int32_t* hd = nullptr;       // [4][ncol] rim cells of the padded FP32 fields (sweep32.cuh)
+    int32_t* par = nullptr;      // [5][ncol] coarse parents of the neighbours and of the column
+    // FP64 level data (sweep64.cuh; also mg_smooth and mg_residual_restrict)
+    double *te64 = nullptr, *tn64 = nullptr, *tbw64 = nullptr, *tbs64 = nullptr, *tv64 = nullptr;
+    double *e64 = nullptr, *ip64 = nullptr;
+    double* wA64 = nullptr;      // area x scale
+    // FP32 level data (sweep32.cuh): couplings in FP32 or BF16, reciprocal pivots, 1 / area; the
+    // FP64 elimination of MG_FP32_P64's finest level; restriction weights onto the next level
+    // [4][ncol_next] (the 9-cell stencil's as well); tensor maps, iterate in x32[0] / x32[1]
+    float *te32 = nullptr, *tn32 = nullptr, *tv32 = nullptr;
+    bf16 *te16 = nullptr, *tn16 = nullptr, *tv16 = nullptr;
+    float* ip32 = nullptr;
+    double *ipd = nullptr, *md = nullptr, *ed = nullptr;
+    float* rA32 = nullptr;
+    double* w64 = nullptr;
+    float* w32 = nullptr;
+    std::vector<mg::SweepMaps> maps;
+    // 9-cell stencil in FP32: the face form
     float* Th32 = nullptr;
     float* Tv32 = nullptr;
-    bf16* Th16 = nullptr;
-    bf16* Tv16 = nullptr;
-    double* w64 = nullptr;  // restriction weights onto the next level, [4][ncol_next]
-    float* w32 = nullptr;
     // workspace: two iterates, the level's rhs and the result handed to the finer level
     double* x64[2] = {nullptr, nullptr};
     double* b64 = nullptr;
@@ -91,9 +66,8 @@ struct DevLevel {
     float* b32 = nullptr;
     float* r32 = nullptr;
     // launch shapes chosen by mg_autotune (0 / -1: the built-in choice)
-    int sweep_bd = 0;          // threads per sweep block, a multiple of 64
+    int sweep_bd = 0;          // FP32 sweep: 64: register chunks, 128: tensor-copy tiles
     int restrict_kc = 0;       // levels per thread of the residual + restriction
-    int restrict_async = -1;   // 1: copy-ring restriction (FP32 levels, n % 16 = 0), 0: register ring
     // 9-cell stencil: fluxes two levels apart [nlev][ncol] and three scratch fields (the
     // residual and the two Thomas factors of a sweep)
     double* T2_64 = nullptr;
@@ -112,9 +86,9 @@ struct mg_handle {
     std::vector<DevLevel> lv;
     double* rdz64 = nullptr;
     float* rdz32 = nullptr;
+    double scale = 1.0;         // power of two in the FP64 volume weights, 1 / (largest finest area x depth)
     double* a6 = nullptr;       // finest level: six premultiplied FP64 couplings and 1 + their sum, per cell
     bool nine = false;          // 9-cell stencil (mg_setup_9pt)
-    bool pivot64 = false;       // MG_FP32_P64: FP64 elimination in the finest level's FP32 sweeps
     double* area0 = nullptr;    // finest level: column areas and layer depths (cell volumes, adjoint solve)
     double* dz = nullptr;
     double* adj = nullptr;      // [N] the scaled right-hand side of the adjoint solve
@@ -124,6 +98,7 @@ struct mg_handle {
     int32_t* faceSide0 = nullptr;
     int32_t* nbrSide0 = nullptr;
     unsigned int* flag = nullptr;
+    unsigned int* timeout = nullptr;   // device: a bounded wait of a sweep ran into its limit
     // pressure solver K_H(A_H, P_H, eps_H) of the Schur-complement step (Sec. 4.1, Table 1)
     mg_pressure_solver ps{MG_PS_MG, 1e-2, 0.8, 10, 200};
     double* bv[8] = {};             // BiCGStab vectors r^, r, p, v, s, t, p^, s^ (allocated on demand)
@@ -246,16 +221,6 @@ mg_status upload(mg_handle* h, P** p, const std::vector<S>& src) {
     return MG_OK;
 }
 
-template <>
-mg_status upload<bf16, double>(mg_handle* h, bf16** p, const std::vector<double>& src) {
-    mg_status st = dalloc(h, p, src.size());
-    if (st != MG_OK) return st;
-    std::vector<bf16> tmp(src.size());
-    for (size_t i = 0; i < src.size(); ++i) tmp[i] = __float2bfloat16_rn((float)src[i]);
-    CK(cudaMemcpy(*p, tmp.data(), tmp.size() * sizeof(bf16), cudaMemcpyHostToDevice));
-    return MG_OK;
-}
-
 // An NVTX range over the scope (shows the library's calls and GCR iterations on a profiler's
 // timeline; costs nothing without a tool attached)
 struct NvtxRange {
@@ -323,24 +288,36 @@ struct View<float, float> {
     static const float* t2(const DevLevel& d) { return d.T2_32; }
     static float* scratch(DevLevel& d, int i) { return d.s32[i]; }
 };
-template <>
-struct View<float, bf16> {
-    static Lvl<float, bf16> lvl(const mg_handle* h, int l) {
-        const DevLevel& d = h->lv[l];
-        return {d.n, d.ncol, h->nlev, d.nbr, d.fof, d.Th16, d.Tv16, d.rA32, h->rdz32};
+
+Lvl64 lvl64(const mg_handle* h, int l) {
+    const DevLevel& d = h->lv[l];
+    return {d.n, d.ncol, h->nlev, d.nbr, d.par, d.te64, d.tn64, d.tbw64, d.tbs64, d.tv64, d.e64, d.ip64, d.wA64, h->dz};
+}
+
+template <typename C, typename P>
+Lvl32<C, P> lvl32(const mg_handle* h, int l) {
+    const DevLevel& d = h->lv[l];
+    Lvl32<C, P> L{d.n, d.ncol, h->nlev, mg::pad_row(d.n), mg::padded(d.n), d.hd};
+    if constexpr (sizeof(C) == 4) {
+        L.te = d.te32;
+        L.tn = d.tn32;
+        L.tv = d.tv32;
+    } else {
+        L.te = d.te16;
+        L.tn = d.tn16;
+        L.tv = d.tv16;
     }
-    static float* x(DevLevel& d, int i) { return d.x32[i]; }
-    static float* b(DevLevel& d) { return d.b32; }
-    static float* r(DevLevel& d) { return d.r32; }
-    static const float* w(const DevLevel& d) { return d.w32; }
-};
-
-constexpr size_t SWEEP_SMEM_MAX = 200 * 1024;
-
-inline int sweep_block(int ncol) {
-    if (ncol >= 128 * 300) return MG_SWEEP_BLOCK;
-    if (ncol >= 64 * 300) return 64;
-    return 32;
+    if constexpr (sizeof(P) == 4) {
+        L.ip = d.ip32;
+        L.m = L.e = nullptr;
+    } else {
+        L.ip = d.ipd;
+        L.m = d.md;
+        L.e = d.ed;
+    }
+    L.rA = d.rA32;
+    L.rdz = h->rdz32;
+    return L;
 }
 
 // ---- launchers ----
@@ -356,159 +333,112 @@ mg_status launch_apply(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, Y*
     return MG_OK;
 }
 
-// prefetch depths of the sweep's register rings (levels in flight per thread)
-template <typename T>
-struct SweepPF {
-    static constexpr int deep = sizeof(T) == 8 ? 4 : MG_SWEEP_DEEP32;
-    static constexpr int shal = sizeof(T) == 8 ? 2 : MG_SWEEP_SHAL32;
-};
+// FP32 levels of this many cells run their sweeps on tensor-copy tiles: below, a tile per block leaves
+// SMs idle and the register sweep is as fast.
+constexpr double TMA_CELLS = 8e5;
 
-// FP32 levels of 30, 50 or 70 levels use the register-stash sweep (k_sweep_rs) where it was
-// measured faster at C192L70: every sweep from a zero iterate (the first of each level; finest
-// level 107 us against 110, levels 1-3 27 / 14 / 11 us against 36 / 20 / 19), and the plain
-// sweeps of levels of at most MG_SWEEP_RS_PLAIN_NCOL columns (the coarsest, 13 us against 15).
-// On larger levels its eleven staged words per step make the plain sweep slower (167 us against
-// 121 on the finest level), and the sweep with fused prolongation slower on every level.
-#ifndef MG_SWEEP_REG
-#define MG_SWEEP_REG 1
-#endif
-#ifndef MG_SWEEP_RS_PLAIN_NCOL
-#define MG_SWEEP_RS_PLAIN_NCOL 4000
-#endif
+inline bool aligned(const void* p, size_t bytes) { return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) == 0; }
 
-// The register-stash sweep (k_sweep_rs) for an FP32 level of NLEV levels, bd threads per block
-template <int NLEV, int MODE, typename B, typename O, bool BCOPY>
-mg_status launch_sweep_rs(const Lvl<float, float>& L, const float* x, const float* xc, int ncol_c, const B* b,
-                          float* bcopy, O* xo, float omega, int bd, cudaStream_t s) {
-    constexpr bool PRO = (MODE == mg::XM_PROLONG || MODE == mg::XM_PROLONG0);
-    constexpr bool RAW = (MODE == mg::XM_PLAIN || MODE == mg::XM_PROLONG);
-    // ring depth: the shared memory of the resident blocks (3 at 70 levels, else 4)
-    constexpr int DEEP = mg::SweepRsBlocks<NLEV>::value == 3 ? ((PRO && RAW) ? 8 : 12) : ((PRO && RAW) ? 6 : 8);
-    constexpr int NW = 5 + (RAW ? 5 : 0) + (PRO ? 5 : 0) + (sizeof(B) == 8 ? 0 : 1);
-    const size_t smem = (size_t)DEEP * bd * (sizeof(B) == 8 ? 8 : 0) + (size_t)DEEP * NW * bd * 4 + NLEV * 4;
-    auto kern = mg::k_sweep_rs<NLEV, MODE, B, O, BCOPY, DEEP>;
-    if (smem > 48 * 1024) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int grid = (L.ncol + bd / 2 - 1) / (bd / 2);
-    kern<<<grid, bd, smem, s>>>(L, x, xc, ncol_c, b, bcopy, xo, omega);
+inline int sweep_mode(const void* x, const void* xc) {
+    return xc ? (x ? mg::XM_PROLONG : mg::XM_PROLONG0) : (x ? mg::XM_PLAIN : mg::XM_ZERO);
+}
+
+// levels per thread of the residual + restriction: long chunks (fewer prologues) where the level
+// fills the GPU several times over; the small levels need every thread (one level per thread at C48L30:
+// 6.5 us a launch against 13 with eight)
+inline int restrict_chunk(const mg_handle* h, int lev) {
+    const DevLevel& d = h->lv[lev];
+    if (d.restrict_kc > 0) return d.restrict_kc;
+    return d.ncol >= 100000 ? 24 : (double)h->nlev * d.ncol >= 2e6 ? 2 : 1;
+}
+
+// One FP64 block-Jacobi sweep on level `lev`.  The iterate it starts from is x (NULL: zero) plus,
+// with xc, the prolongation of xc.  b: weighted, or with `raw` the caller's, whose weighted form is
+// stored in bcopy when that is given.  (h is NULL where no launch may be recorded.)
+template <bool RAW, bool COPY, int K>
+cudaError_t sweep64_go(const Lvl64& L, int mode, const double* x, const double* xc, int ncol_c, const double* b,
+                       double* bcopy, double* xo, double om, cudaStream_t s) {
+    const dim3 g((L.ncol + 31) / 32), t(32 * ((L.nlev + K - 1) / K));
+    switch (mode) {
+        case mg::XM_ZERO: mg::k_sweep64<mg::XM_ZERO, RAW, COPY, K><<<g, t, 0, s>>>(L, x, xc, ncol_c, b, bcopy, xo, om); break;
+        case mg::XM_PLAIN: mg::k_sweep64<mg::XM_PLAIN, RAW, COPY, K><<<g, t, 0, s>>>(L, x, xc, ncol_c, b, bcopy, xo, om); break;
+        case mg::XM_PROLONG: mg::k_sweep64<mg::XM_PROLONG, RAW, COPY, K><<<g, t, 0, s>>>(L, x, xc, ncol_c, b, bcopy, xo, om); break;
+        default: mg::k_sweep64<mg::XM_PROLONG0, RAW, COPY, K><<<g, t, 0, s>>>(L, x, xc, ncol_c, b, bcopy, xo, om); break;
+    }
+    return cudaGetLastError();
+}
+
+mg_status launch_sweep64(mg_handle* h, int lev, const Lvl64& L, const double* x, const double* xc, int ncol_c,
+                         const double* b, bool raw, double* bcopy, double* xo, double om, cudaStream_t s) {
+    const int mode = sweep_mode(x, xc);
+    Prof pr(h, MG_K_SWEEP, lev, 8.0 * L.nlev * L.ncol * (4 + (mode != mg::XM_ZERO ? 2 : 0) + (x ? 1 : 0) +
+                                                         (xc ? 0.25 : 0.0) + (bcopy ? 1 : 0)), s, mode);
+    auto shape = [&](auto r, auto c) -> cudaError_t {
+        constexpr bool R = decltype(r)::value, B = decltype(c)::value;
+        if (L.nlev > 80) return sweep64_go<R, B, 16>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
+        if ((double)L.nlev * L.ncol < 2e6) return sweep64_go<R, B, 5>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
+        return sweep64_go<R, B, 10>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
+    };
+    if (raw && bcopy) CK(shape(std::true_type(), std::true_type()));
+    else if (raw) CK(shape(std::true_type(), std::false_type()));
+    else CK(shape(std::false_type(), std::false_type()));
+    return MG_OK;
+}
+
+// FP64 residual and restriction of level lev onto lev + 1 (weighted right-hand sides; RAW: the caller's
+// unweighted arrays, mg_residual_restrict).
+template <bool RAW>
+mg_status launch_restrict64(mg_handle* h, int lev, const double* x, const double* b, double* bc, cudaStream_t s) {
+    const Lvl64 L = lvl64(h, lev);
+    const int ncol_c = h->lv[lev + 1].ncol, kc = restrict_chunk(h, lev);
+    const double* wAc = h->lv[lev + 1].wA64;
+    Prof pr(h, MG_K_RESTRICT, lev, 8.0 * L.nlev * L.ncol * (1.25 + (x ? 3.5 : 0.0)), s);
+    const bool vec = aligned(b, 16) && aligned(x, 16);
+    const dim3 grid((ncol_c + 127) / 128, (L.nlev + kc - 1) / kc);
+    if (!x) mg::k_restrict64<true, RAW, false><<<grid, 128, 0, s>>>(L, x, b, wAc, bc, ncol_c, kc);
+    else if (vec) mg::k_restrict64<false, RAW, true><<<grid, 128, 0, s>>>(L, x, b, wAc, bc, ncol_c, kc);
+    else mg::k_restrict64<false, RAW, false><<<grid, 128, 0, s>>>(L, x, b, wAc, bc, ncol_c, kc);
     CK(cudaGetLastError());
     return MG_OK;
 }
 
-template <typename T, typename C, int MODE, typename X, typename B, typename O, bool BCOPY, typename P>
-mg_status launch_sweep_shared(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, const T* xc, int ncol_c,
-                              const B* b, T* bcopy, O* xo, double omega, cudaStream_t s);
-
-template <typename T, typename C, int MODE, typename X, typename B, typename O, bool BCOPY>
-mg_status launch_sweep(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, const T* xc, int ncol_c,
-                       const B* b, T* bcopy, O* xo, double omega, cudaStream_t s) {
-    const double nc = (double)L.nlev * L.ncol;
-    double per = sizeof(B) + 3 * sizeof(C) + sizeof(O);
-    if (MODE == mg::XM_PLAIN || MODE == mg::XM_PROLONG) per += sizeof(X);
-    if (MODE == mg::XM_PROLONG || MODE == mg::XM_PROLONG0) per += 0.25 * sizeof(T);
-    if (BCOPY) per += sizeof(T);
-    Prof pr(h, MG_K_SWEEP, lev, nc * per, s, MODE);
-    if constexpr (std::is_same<T, float>::value && std::is_same<C, float>::value) {
-        // MG_FP32_P64: the finest level eliminates with FP64 pivots
-        if (h && h->pivot64 && lev == 0)
-            return launch_sweep_shared<T, C, MODE, X, B, O, BCOPY, double>(h, lev, L, x, xc, ncol_c, b, bcopy, xo,
-                                                                          omega, s);
-    }
-    if constexpr (MG_SWEEP_REG && std::is_same<T, float>::value && std::is_same<C, float>::value &&
-                  std::is_same<X, float>::value && (MODE == mg::XM_ZERO || MODE == mg::XM_PLAIN)) {
-        const int bdr = (h && h->lv[lev].sweep_bd > 0) ? h->lv[lev].sweep_bd : MG_SWEEP_BLOCK;
-        const bool use = MODE == mg::XM_ZERO || L.ncol <= MG_SWEEP_RS_PLAIN_NCOL;
-        if (use) switch (L.nlev) {
-            case 70: return launch_sweep_rs<70, MODE, B, O, BCOPY>(L, x, xc, ncol_c, b, bcopy, xo, (float)omega, bdr, s);
-            case 50: return launch_sweep_rs<50, MODE, B, O, BCOPY>(L, x, xc, ncol_c, b, bcopy, xo, (float)omega, bdr, s);
-            case 30: return launch_sweep_rs<30, MODE, B, O, BCOPY>(L, x, xc, ncol_c, b, bcopy, xo, (float)omega, bdr, s);
-            default: break;
-        }
-    }
-    return launch_sweep_shared<T, C, MODE, X, B, O, BCOPY, T>(h, lev, L, x, xc, ncol_c, b, bcopy, xo, omega, s);
-}
-
-// the shared-memory-stash sweep (k_sweep), elimination in P
-template <typename T, typename C, int MODE, typename X, typename B, typename O, bool BCOPY, typename P>
-mg_status launch_sweep_shared(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, const T* xc, int ncol_c,
-                              const B* b, T* bcopy, O* xo, double omega, cudaStream_t s) {
-    // two threads per column; per thread the shared memory holds the asynchronous-copy
-    // ring (DEEP slots of b, the next iterate and, unless BF16, three coefficients) and the
-    // stash (2 values per step of half a column); it must fit the budget
-    constexpr int DEEP = SweepPF<T>::deep;
-    const int hsteps = (L.nlev + 1) / 2;
-    // (BF16 coefficients travel as 4-byte pairs)
-    const size_t per_thread =
-        DEEP * (sizeof(B) + sizeof(T) + (sizeof(C) >= 4 ? 3 * sizeof(C) : (MG_SWEEP_BF16_PAIRS ? 12 : 0))) +
-        2 * (size_t)hsteps * sizeof(T);
-    const size_t per_block = (size_t)L.nlev * sizeof(T);   // the 1/dz table
-    // (h is NULL for the allocation-free smoothing: built-in shapes)
-    int bd = (h && h->lv[lev].sweep_bd > 0) ? h->lv[lev].sweep_bd : sweep_block(2 * L.ncol);
-#if MG_SWEEP_WARP_HALVES
-    constexpr int BQ = 64;   // the halves of a column lie in different warps
-#else
-    constexpr int BQ = 32;
-#endif
-    const int cap = (int)((SWEEP_SMEM_MAX - per_block) / per_thread) / BQ * BQ;
-    if (cap < BQ) return MG_ERR_UNSUPPORTED;
-    if (bd < BQ) bd = BQ;
-    if (bd > cap) bd = cap;
-    const size_t smem = per_thread * bd + per_block;
-    // ring lengths per iterate source (measured at C192L70): a prolongation sweep with a fine
-    // iterate carries eight neighbour values per step and needs the shorter ring to fit the
-    // register budget; the zero-start sweep is fastest with the shorter ring as well
-    constexpr int SHAL = MODE == mg::XM_PROLONG ? MG_SWEEP_SHAL_PRO
-                         : MODE == mg::XM_ZERO    ? (sizeof(T) == 8 ? 2 : MG_SWEEP_SHAL_ZERO)
-                                                  : SweepPF<T>::shal;
-    auto kern = mg::k_sweep<T, C, MODE, X, B, O, BCOPY, DEEP, SHAL, P>;
-    if (smem > 48 * 1024) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int cols = bd / 2;
-    const int grid = (L.ncol + cols - 1) / cols;
-    kern<<<grid, bd, smem, s>>>(L, x, xc, ncol_c, b, bcopy, xo, (T)omega);
-    CK(cudaGetLastError());
-    return MG_OK;
-}
-
-template <typename T, typename C, bool XZERO, typename X, typename B, typename O>
-mg_status launch_restrict(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, const B* b, const T* w, O* bc,
-                          int ncol_c, cudaStream_t s) {
-    const double nc = (double)L.nlev * L.ncol;
-    Prof pr(h, MG_K_RESTRICT, lev, nc * (sizeof(B) + 3 * sizeof(C) + (XZERO ? 0 : sizeof(X)) + 0.25 * sizeof(O) +
-                                          sizeof(T) / (double)L.nlev), s);
-    if (L.n % 16 == 0) {
-        // one thread per fine column, 4 warps per block
-        const int warps = 6 * (L.n / 2) * (L.n / 16);
-        // levels per thread: on a level large enough to fill the GPU several times over, long
-        // chunks (fewer prologues); smaller levels need the threads of short chunks
-        const int kc = (h && h->lv[lev].restrict_kc > 0) ? h->lv[lev].restrict_kc
-                       : L.ncol >= MG_RESTRICT_BIG_NCOL ? MG_RESTRICT_KCHUNK_BIG
-                                                        : MG_RESTRICT_KCHUNK;
-        const dim3 grid((warps + 3) / 4, (L.nlev + kc - 1) / kc);
-        constexpr bool ASYNC = MG_RESTRICT_ASYNC && !XZERO && std::is_same<T, float>::value &&
-                               std::is_same<C, float>::value && std::is_same<X, float>::value &&
-                               std::is_same<B, float>::value && std::is_same<O, float>::value;
-        bool async_done = false;
-        if constexpr (ASYNC) {
-            const int ra = h ? h->lv[lev].restrict_async : -1;
-            if (ra >= 0 ? ra == 1 : L.ncol >= MG_RESTRICT_ASYNC_NCOL) {
-                mg::k_resid_restrict16a<MG_RESTRICT_DEEP, MG_RESTRICT_ASHAL><<<grid, 128, 0, s>>>(L, x, b, w, bc,
-                                                                                                 ncol_c, kc);
-                async_done = true;
-            }
-        }
-        if (!async_done)
-            mg::k_resid_restrict16<T, C, XZERO, X, B, O, MG_RESTRICT_SHAL><<<grid, 128, 0, s>>>(L, x, b, w, bc,
-                                                                                               ncol_c, kc);
+// The same of the FP32 V-cycle (fields padded).  raw: b is the caller's FP64 array, its FP32 copy goes
+// to bcopy.  xo: padded FP32, or FP64 with out64.
+template <typename C, typename P>
+mg_status launch_sweep32(mg_handle* h, int lev, const float* x, const float* xc, const void* b, bool raw, float* bcopy,
+                         void* xo, bool out64, double om, cudaStream_t s) {
+    const Lvl32<C, P> L = lvl32<C, P>(h, lev);
+    const DevLevel& d = h->lv[lev];
+    const int mode = sweep_mode(x, xc);
+    double per = (raw ? 12.0 : 4.0) + sizeof(C) + (sizeof(P) == 8 ? 24.0 : 4.0) + (out64 ? 8.0 : 4.0);
+    if (mode != mg::XM_ZERO) per += 2.0 * sizeof(C);
+    if (x) per += 4.0;
+    if (xc) per += 1.0;
+    Prof pr(h, MG_K_SWEEP, lev, (double)L.nlev * L.ncol * per, s, mode);
+    const mg::SweepMaps* maps = nullptr;
+    const bool tiles = d.sweep_bd > 0 ? d.sweep_bd == 128 : (double)L.nlev * L.ncol >= TMA_CELLS;
+    if (tiles && d.maps.size() == 2 && mode != mg::XM_PROLONG0) maps = &d.maps[x == d.x32[1]];
+    const mg::SweepCall32<C, P> q{L, mode, x, xc, b, raw, bcopy, xo, out64, om, maps, h->nsm, h->timeout};
+    CK((mg::sweep32_run<C, P>(q, s)));
+    if (L.n == 1 && !out64) {   // (a C1 column has several edges on one axis)
+        mg::k_fill_rims<float><<<dim3(1, L.nlev), 32, 0, s>>>(L.n, L.ncol, L.hd, static_cast<float*>(xo));
         CK(cudaGetLastError());
-        return MG_OK;
     }
-    const int bd = ncol_c >= 128 * 300 ? 128 : (ncol_c >= 64 * 300 ? 64 : 32);
-    // chunk of levels per thread: enough threads to fill the GPU, few re-loads of the
-    // 32 connectivity entries of the 4 children
-    const int kc = (h && h->lv[lev].restrict_kc > 0) ? h->lv[lev].restrict_kc
-                   : ncol_c >= 128 * 300 ? 3 * APPLY_KCHUNK
-                                         : APPLY_KCHUNK;
-    const dim3 grid((ncol_c + bd - 1) / bd, (L.nlev + kc - 1) / kc);
-    mg::k_resid_restrict<T, C, XZERO, X, B, O><<<grid, bd, 0, s>>>(L, x, b, w, bc, ncol_c, kc);
+    return MG_OK;
+}
+
+template <typename C>
+mg_status launch_restrict32(mg_handle* h, int lev, const float* x, const float* b, float* bc, cudaStream_t s) {
+    const Lvl32<C, float> L = lvl32<C, float>(h, lev);
+    const DevLevel& d = h->lv[lev];
+    const int ncol_c = h->lv[lev + 1].ncol, kc = restrict_chunk(h, lev);
+    Prof pr(h, MG_K_RESTRICT, lev, (double)L.nlev * L.ncol * (5.0 + (x ? 4.0 + 3.0 * sizeof(C) : 0.0)), s);
+    const dim3 grid((ncol_c + 127) / 128, (L.nlev + kc - 1) / kc);
+    const bool tree = L.n % 16 == 0;
+    if (!x && tree) mg::k_restrict32<C, true, true><<<grid, 128, 0, s>>>(L, x, b, d.w32, bc, ncol_c, kc);
+    else if (!x) mg::k_restrict32<C, true, false><<<grid, 128, 0, s>>>(L, x, b, d.w32, bc, ncol_c, kc);
+    else if (tree) mg::k_restrict32<C, false, true><<<grid, 128, 0, s>>>(L, x, b, d.w32, bc, ncol_c, kc);
+    else mg::k_restrict32<C, false, false><<<grid, 128, 0, s>>>(L, x, b, d.w32, bc, ncol_c, kc);
     CK(cudaGetLastError());
     return MG_OK;
 }
@@ -531,26 +461,6 @@ mg_status launch_convert(mg_handle* h, int lev, size_t n, const A* a, B* b, cuda
     return MG_OK;
 }
 
-// One sweep with the iterate source chosen at run time.
-//   cur == nullptr and xc == nullptr : zero iterate
-//   xc != nullptr                    : iterate = (cur or 0) + Prolongate(xc)
-template <typename T, typename C, typename B, typename O>
-mg_status sweep_any(mg_handle* h, int lev, const Lvl<T, C>& L, const T* cur, const T* xc, int ncol_c, const B* b,
-                    T* bcopy, O* xo, double om, cudaStream_t s) {
-    if (bcopy) {
-        if (xc) return MG_ERR_ARG;
-        if (cur) return launch_sweep<T, C, mg::XM_PLAIN, T, B, O, true>(h, lev, L, cur, xc, ncol_c, b, bcopy, xo, om, s);
-        return launch_sweep<T, C, mg::XM_ZERO, T, B, O, true>(h, lev, L, cur, xc, ncol_c, b, bcopy, xo, om, s);
-    }
-    if (xc) {
-        if (cur)
-            return launch_sweep<T, C, mg::XM_PROLONG, T, B, O, false>(h, lev, L, cur, xc, ncol_c, b, bcopy, xo, om, s);
-        return launch_sweep<T, C, mg::XM_PROLONG0, T, B, O, false>(h, lev, L, cur, xc, ncol_c, b, bcopy, xo, om, s);
-    }
-    if (cur) return launch_sweep<T, C, mg::XM_PLAIN, T, B, O, false>(h, lev, L, cur, xc, ncol_c, b, bcopy, xo, om, s);
-    return launch_sweep<T, C, mg::XM_ZERO, T, B, O, false>(h, lev, L, cur, xc, ncol_c, b, bcopy, xo, om, s);
-}
-
 // Settings of one cycle: levels used, over-relaxation and sweep counts.  A single-level
 // cycle with n_coarse sweeps is the block-Jacobi iteration P_H^(Jac)(omega, n_coarse) of
 // Sec. 4.1 (line relaxation).
@@ -564,59 +474,109 @@ inline Cycle vcycle_of(const mg_handle* h) {
     return {h->L, h->prm.omega, h->prm.n_pre, h->prm.n_post, h->prm.n_coarse};
 }
 
-// Algorithm 1 on level l with right-hand side `b` (type B: FP64 on the finest level of the
-// FP32 V-cycle, T otherwise); the result goes to `out` (type O).  On every level the
-// iterate starts at zero (x^(l+1) <- 0 of Algorithm 1; the V-cycle is used as a
-// preconditioner, so x^(1) = 0 as well).
-template <typename T, typename C, typename B, typename O>
-mg_status mgv(mg_handle* h, const Cycle& cy, int l, const B* b, O* out, cudaStream_t s) {
+// out = (x or 0) + Prolongate(xc), or without xc the conversion of x, into a level's result
+template <typename T, typename O>
+mg_status launch_emit(mg_handle* h, int lev, const T* x, const T* xc, O* out, cudaStream_t s) {
+    const DevLevel& d = h->lv[lev];
+    Prof pr(h, xc ? MG_K_PROLONG : MG_K_CONVERT, lev,
+            (double)cells(h, lev) * ((xc ? 0.25 * sizeof(T) : 0.0) + (x ? sizeof(T) : 0) + sizeof(O)), s);
+    mg::k_emit<T, O><<<dim3((d.ncol + 127) / 128, h->nlev), 128, 0, s>>>(d.n, d.ncol, d.hd, x, xc, out);
+    CK(cudaGetLastError());
+    return MG_OK;
+}
+
+// The precisions of the V-cycle: workspace and launches of one level.
+struct Cyc64 {
+    typedef double T;
+    static T* x(DevLevel& d, int i) { return d.x64[i]; }
+    static T* b(DevLevel& d) { return d.b64; }
+    static T* r(DevLevel& d) { return d.r64; }
+    static mg_status sweep(mg_handle* h, int l, const T* x, const T* xc, const void* b, bool raw, T* bcopy, void* xo,
+                           bool, double om, cudaStream_t s) {
+        return launch_sweep64(h, l, lvl64(h, l), x, xc, xc ? h->lv[l + 1].ncol : 0, static_cast<const double*>(b), raw,
+                              bcopy, static_cast<double*>(xo), om, s);
+    }
+    static mg_status restrict_(mg_handle* h, int l, const T* x, const T* b, T* bc, cudaStream_t s) {
+        return launch_restrict64<false>(h, l, x, b, bc, s);
+    }
+    static mg_status copy_b(mg_handle* h, const double* b, cudaStream_t s) {
+        const DevLevel& d = h->lv[0];
+        Prof pr(h, MG_K_CONVERT, 0, 16.0 * cells(h, 0), s);
+        mg::k_weight64<<<dim3((d.ncol + 127) / 128, h->nlev), 128, 0, s>>>(d.ncol, b, d.wA64, h->dz, d.b64);
+        CK(cudaGetLastError());
+        return MG_OK;
+    }
+};
+
+template <typename C>
+struct Cyc32 {
+    typedef float T;
+    static T* x(DevLevel& d, int i) { return d.x32[i]; }
+    static T* b(DevLevel& d) { return d.b32; }
+    static T* r(DevLevel& d) { return d.r32; }
+    static mg_status sweep(mg_handle* h, int l, const T* x, const T* xc, const void* b, bool raw, T* bcopy, void* xo,
+                           bool out64, double om, cudaStream_t s) {
+        if constexpr (sizeof(C) == 4) {
+            // MG_FP32_P64: the finest level eliminates with FP64 pivots
+            if (l == 0 && h->lv[0].ipd) return launch_sweep32<C, double>(h, l, x, xc, b, raw, bcopy, xo, out64, om, s);
+        }
+        return launch_sweep32<C, float>(h, l, x, xc, b, raw, bcopy, xo, out64, om, s);
+    }
+    static mg_status restrict_(mg_handle* h, int l, const T* x, const T* b, T* bc, cudaStream_t s) {
+        return launch_restrict32<C>(h, l, x, b, bc, s);
+    }
+    static mg_status copy_b(mg_handle* h, const double* b, cudaStream_t s) {
+        return launch_emit<double, float>(h, 0, b, nullptr, h->lv[0].b32, s);
+    }
+};
+
+// Algorithm 1 on level l; the result goes to `out` (FP64 on the finest level, the cycle's type
+// below).  On every level the iterate starts at zero (x^(l+1) <- 0 of Algorithm 1; the V-cycle is
+// used as a preconditioner, so x^(1) = 0 as well).  The finest level's right-hand side is the
+// caller's FP64 array; its first sweep stores it in the cycle's form for the level's later kernels.
+template <typename Cyc>
+mg_status mgv(mg_handle* h, const Cycle& cy, int l, const void* b, void* out, cudaStream_t s) {
     static const char* const level_range[MG_MAX_LEVELS] = {"V-cycle level 0", "V-cycle level 1", "V-cycle level 2",
                                                            "V-cycle level 3", "V-cycle level 4", "V-cycle level 5",
                                                            "V-cycle level 6", "V-cycle level 7"};
     NvtxRange nvtx_(level_range[l]);   // the level and the levels below it (nested ranges)
-    typedef View<T, C> V;
+    typedef typename Cyc::T T;
     DevLevel& d = h->lv[l];
-    const Lvl<T, C> L = V::lvl(h, l);
-    const bool coarsest = (l == cy.L - 1);
+    const bool coarsest = (l == cy.L - 1), finest = l == 0;
     const double om = cy.omega;
-    const bool conv = !std::is_same<B, T>::value;  // rhs arrives in FP64, iterate in FP32
-    T* ws[2] = {V::x(d, 0), V::x(d, 1)};
-    const T* bT = conv ? (const T*)V::b(d) : (const T*)(const void*)b;
+    const bool wide = finest && sizeof(T) == 4;   // the level's result leaves in FP64
+    T* ws[2] = {Cyc::x(d, 0), Cyc::x(d, 1)};
+    const T* bT = finest ? Cyc::b(d) : static_cast<const T*>(b);
     const int npre = coarsest ? cy.n_coarse : cy.n_pre;
-    if (conv && npre == 0) TRY(launch_convert(h, l, cells(h, l), b, V::b(d), s));
+    if (finest && npre == 0) TRY(Cyc::copy_b(h, static_cast<const double*>(b), s));
     T* cur = nullptr;
     for (int i = 0; i < npre; ++i) {
         const bool final = coarsest && i == npre - 1;
         T* dst = (cur == ws[0]) ? ws[1] : ws[0];
-        T* bcopy = (conv && i == 0) ? V::b(d) : nullptr;
-        if (final) {
-            if (i == 0) TRY((sweep_any<T, C, B, O>(h, l, L, cur, (const T*)nullptr, 0, b, bcopy, out, om, s)));
-            else TRY((sweep_any<T, C, T, O>(h, l, L, cur, (const T*)nullptr, 0, bT, nullptr, out, om, s)));
-            return MG_OK;
-        }
-        if (i == 0) TRY((sweep_any<T, C, B, T>(h, l, L, cur, (const T*)nullptr, 0, b, bcopy, dst, om, s)));
-        else TRY((sweep_any<T, C, T, T>(h, l, L, cur, (const T*)nullptr, 0, bT, nullptr, dst, om, s)));
+        const bool raw = finest && i == 0;
+        // (a raw sweep writes T: a single-sweep FP32 cycle converts its result)
+        const bool direct = final && !(raw && wide);
+        TRY(Cyc::sweep(h, l, cur, nullptr, raw ? b : bT, raw, raw ? Cyc::b(d) : nullptr, direct ? out : dst,
+                       direct && wide, om, s));
+        if (final) return direct ? MG_OK : launch_emit<T, double>(h, l, dst, nullptr, static_cast<double*>(out), s);
         cur = dst;
     }
     // residual and restriction onto level l+1
     DevLevel& dc = h->lv[l + 1];
-    T* bc = V::b(dc);
-    if (cur) TRY((launch_restrict<T, C, false, T, T, T>(h, l, L, cur, bT, V::w(d), bc, dc.ncol, s)));
-    else TRY((launch_restrict<T, C, true, T, T, T>(h, l, L, cur, bT, V::w(d), bc, dc.ncol, s)));
-    T* xc = V::r(dc);
-    TRY((mgv<T, C, T, T>(h, cy, l + 1, bc, xc, s)));
+    T* bc = Cyc::b(dc);
+    TRY(Cyc::restrict_(h, l, cur, bT, bc, s));
+    T* xc = Cyc::r(dc);
+    TRY(mgv<Cyc>(h, cy, l + 1, bc, xc, s));
     // coarse-grid correction fused into the first post-smoothing sweep
     const int npost = cy.n_post;
     if (npost == 0) {
-        if (cur) return launch_prolong<T, false, T, O>(h, l, d.n, d.ncol, dc.ncol, h->nlev, cur, xc, out, s);
-        return launch_prolong<T, true, T, O>(h, l, d.n, d.ncol, dc.ncol, h->nlev, cur, xc, out, s);
+        if (wide) return launch_emit<T, double>(h, l, cur, xc, static_cast<double*>(out), s);
+        return launch_emit<T, T>(h, l, cur, xc, static_cast<T*>(out), s);
     }
     for (int i = 0; i < npost; ++i) {
-        const T* pxc = (i == 0) ? xc : nullptr;
-        const int ncc = (i == 0) ? dc.ncol : 0;
-        if (i == npost - 1) return sweep_any<T, C, T, O>(h, l, L, cur, pxc, ncc, bT, nullptr, out, om, s);
+        const bool last = i == npost - 1;
         T* dst = (cur == ws[0]) ? ws[1] : ws[0];
-        TRY((sweep_any<T, C, T, T>(h, l, L, cur, pxc, ncc, bT, nullptr, dst, om, s)));
+        TRY(Cyc::sweep(h, l, cur, i == 0 ? xc : nullptr, bT, false, nullptr, last ? out : dst, last && wide, om, s));
         cur = dst;
     }
     return MG_OK;
@@ -719,10 +679,10 @@ mg_status run_cycle(mg_handle* h, const Cycle& cy, const double* b, double* x, c
         }
     }
     switch (h->prm.vcycle_precision) {
-        case MG_FP64: return mgv<double, double, double, double>(h, cy, 0, b, x, s);
+        case MG_FP64: return mgv<Cyc64>(h, cy, 0, b, x, s);
         case MG_FP32:
-        case MG_FP32_P64: return mgv<float, float, double, double>(h, cy, 0, b, x, s);
-        case MG_FP32_BF16COEF: return mgv<float, bf16, double, double>(h, cy, 0, b, x, s);
+        case MG_FP32_P64: return mgv<Cyc32<float>>(h, cy, 0, b, x, s);
+        case MG_FP32_BF16COEF: return mgv<Cyc32<bf16>>(h, cy, 0, b, x, s);
         default: return MG_ERR_ARG;
     }
 }
@@ -999,7 +959,10 @@ mg_status gcr_landed(mg_handle* h, GcrRun& g, cudaStream_t s) {
     ++g.it;
     const double rr = h->host_sc[0];
     if (!std::isfinite(rr)) {
-        g.st = MG_ERR_BREAKDOWN;
+        unsigned int late = 0;   // a sweep's copy that did not arrive leaves NaN and this flag
+        CK(cudaMemcpyAsync(&late, h->timeout, sizeof late, cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        g.st = late ? MG_ERR_TIMEOUT : MG_ERR_BREAKDOWN;
         g.active = false;
         return MG_OK;
     }
@@ -1100,6 +1063,98 @@ mg_status schur_impl(mg_handle* h, const double* ru, const double* rp, double* u
     return MG_OK;
 }
 
+// parents of the neighbours E, W, N, S and of the column itself, [5][ncol]
+// the rim cell of the padded fields that repeats each edge column (SLvl::hd), [4][ncol]
+__global__ void k_rims(int n, int ncol, const int32_t* __restrict__ nbr, int32_t* __restrict__ hd) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
+    if (c >= ncol) return;
+    const int np = mg::pad_row(n), step[4] = {1, -1, np, -np};
+    const mg::Pos at(c, n, np);
+    const bool edge = s == 0 ? at.i + 1 == (unsigned)n : s == 1 ? at.i == 0 : s == 2 ? at.j + 1 == (unsigned)n : at.j == 0;
+    int d = -1;
+    if (edge) {
+        const int nb = nbr[(size_t)s * ncol + c];
+        for (int t = 0; t < 4; ++t)   // the neighbour's side that faces this column
+            if (nbr[(size_t)t * ncol + nb] == c) d = (int)mg::Pos(nb, n, np).cp + step[t];
+    }
+    hd[(size_t)s * ncol + c] = d;
+}
+
+__global__ void k_parents(int n, int ncol, const int32_t* __restrict__ nbr, int32_t* __restrict__ par) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
+    if (c < ncol) par[(size_t)s * ncol + c] = mg::parent_col(s < 4 ? nbr[(size_t)s * ncol + c] : c, n);
+}
+
+// Tensor maps of the TMA sweep (sweep_tma.cuh) for an FP32 level of 8 to 80 levels (two blocks'
+// boxes per SM).
+mg_status build_maps(mg_handle* h, int l) {
+    DevLevel& d = h->lv[l];
+    d.maps.clear();
+    if (h->nine || !d.ip32 || h->nlev < 8 || h->nlev > 80) return MG_OK;
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    CK(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found));
+    if (!fn || found != cudaDriverEntryPointSuccess) return MG_ERR_CUDA;
+    const auto encode = reinterpret_cast<decltype(&cuTensorMapEncodeTiled)>(fn);
+    bool ok = true;
+    const int H = (h->nlev + 1) / 2;
+    // a padded field of C_n, boxes of `cols` columns x `rows` levels
+    auto map = [&](CUtensorMap* out, const auto* base, int n, int levels, int cols, int rows) {
+        const cuuint64_t size = sizeof(*base), dims[2] = {(cuuint64_t)mg::padded(n), (cuuint64_t)levels};
+        const cuuint64_t stride[1] = {size * dims[0]};
+        const cuuint32_t boxes[2] = {(cuuint32_t)cols, (cuuint32_t)rows}, one[2] = {1, 1};
+        ok &= encode(out, size == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                     const_cast<void*>(static_cast<const void*>(base)), dims, stride, boxes, one,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    d.maps.resize(2);
+    for (int i = 0; i < 2; ++i) {
+        mg::SweepMaps& m = d.maps[i];
+        const int n = d.n, N = h->nlev;
+        auto coefs = [&](const auto* te, const auto* tn, const auto* tv) {
+            map(&m.te, te, n, N, 32 + 16 / (int)sizeof(*te), H);
+            map(&m.tn, tn, n, N, 32, H);
+            map(&m.tv, tv, n, N + 1, 32, H + 1);
+        };
+        if (d.te32) coefs(d.te32, d.tn32, d.tv32);
+        else coefs(d.te16, d.tn16, d.tv16);
+        map(&m.b, d.b32, n, N, 32, H);
+        map(&m.ip, d.ip32, n, N, 32, H);
+        map(&m.x, d.x32[i], n, N, 40, H + 1);
+        map(&m.xr, d.x32[i], n, N, 32, H);
+        if (l + 1 < h->L) {
+            map(&m.xc, h->lv[l + 1].r32, h->lv[l + 1].n, N, 24, H + 1);
+            map(&m.xca, h->lv[l + 1].r32, h->lv[l + 1].n, N, 24, H);
+        }
+    }
+    return ok ? MG_OK : MG_ERR_CUDA;
+}
+
+// The level data of the sweeps and restrictions from level l's FP64 face form, in every precision the
+// handle holds.
+mg_status pack_level(mg_handle* h, int l, cudaStream_t s) {
+    DevLevel& d = h->lv[l];
+    const dim3 grid((d.ncol + 127) / 128, h->nlev + 1);
+    mg::k_pack64<<<grid, 128, 0, s>>>(d.n, d.ncol, h->nlev, d.fof, d.Th64, d.Tv64, d.wA64, h->dz, h->scale, d.te64, d.tn64,
+                                      d.tbw64, d.tbs64, d.tv64);
+    mg::k_factor64<<<(d.ncol + 63) / 64, 64, 0, s>>>(d.n, d.ncol, h->nlev, d.te64, d.tn64, d.tbw64, d.tbs64, d.tv64,
+                                                     d.wA64, h->dz, d.e64, d.ip64);
+    const dim3 halves((d.ncol + 63) / 64, 2);
+    if (d.te32) {
+        mg::k_pack32<float><<<grid, 128, 0, s>>>(d.n, d.ncol, h->nlev, d.fof, d.Th64, d.Tv64, d.te32, d.tn32, d.tv32);
+        mg::k_factor32<float, float><<<halves, 64, 0, s>>>(lvl32<float, float>(h, l), d.ip32, nullptr, nullptr);
+        if (d.ipd)
+            mg::k_factor32<float, double><<<halves, 64, 0, s>>>(lvl32<float, double>(h, l), d.ipd, d.md, d.ed);
+    }
+    if (d.te16) {
+        mg::k_pack32<bf16><<<grid, 128, 0, s>>>(d.n, d.ncol, h->nlev, d.fof, d.Th64, d.Tv64, d.te16, d.tn16, d.tv16);
+        mg::k_factor32<bf16, float><<<halves, 64, 0, s>>>(lvl32<bf16, float>(h, l), d.ip32, nullptr, nullptr);
+    }
+    CK(cudaGetLastError());
+    return MG_OK;
+}
+
 // Replaces the finest-level operator by the caller's couplings a[s][k][c] (DEVICE, 6 N): the
 // FP64 operator of the GCR apply takes them as they are, the V-cycle's finest level their face
 // form in its precision.  A first pass only checks them (flux symmetry, sign, no flux through
@@ -1107,14 +1162,13 @@ mg_status schur_impl(mg_handle* h, const double* ru, const double* rp, double* u
 mg_status set_coefficients_impl(mg_handle* h, const double* a, cudaStream_t s) {
     const int ncol = h->lv[0].ncol, nlev = h->nlev, nf = 2 * ncol;
     const DevLevel& d = h->lv[0];
-    const mg::CoefTargets t{d.Th64, d.Th32, d.Th16, d.Tv64, d.Tv32, d.Tv16};
     CK(cudaMemsetAsync(h->flag, 0, sizeof(unsigned int), s));
     for (int pass = 0; pass < 2; ++pass) {
         const bool write = pass == 1;
         mg::k_coef_faces<<<dim3((nf + 127) / 128, nlev), 128, 0, s>>>(ncol, nlev, h->faceL0, h->faceR0, h->faceSide0,
-                                                                       h->nbrSide0, h->area0, a, write, t, h->flag);
-        mg::k_coef_vertical<<<dim3((ncol + 127) / 128, nlev + 1), 128, 0, s>>>(ncol, nlev, h->dz, a, write, t,
-                                                                                h->flag);
+                                                                       h->nbrSide0, h->area0, a, write, d.Th64, h->flag);
+        mg::k_coef_vertical<<<dim3((ncol + 127) / 128, nlev + 1), 128, 0, s>>>(ncol, nlev, h->dz, a, write,
+                                                                                d.Tv64, h->flag);
         CK(cudaGetLastError());
         if (!write) {
             unsigned int bad = 0;
@@ -1125,6 +1179,7 @@ mg_status set_coefficients_impl(mg_handle* h, const double* a, cudaStream_t s) {
     }
     mg::k_coef_cells<<<4 * h->nsm, 256, 0, s>>>(cells(h, 0), a, h->a6);
     CK(cudaGetLastError());
+    TRY(pack_level(h, 0, s));
     CK(cudaStreamSynchronize(s));
     return MG_OK;
 }
@@ -1260,14 +1315,18 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
     TRY(upload(h, &h->dz, vg.dz));
     TRY(upload(h, &h->area0, hg[0].area));
     TRY(upload(h, &h->rdz32, rdz));
+    // V = area x depth x scale is at most about 1 on the finest level (a power of two: exact)
+    h->scale = std::exp2(-std::ceil(std::log2(*std::max_element(hg[0].area.begin(), hg[0].area.end()) *
+                                              *std::max_element(vg.dz.begin(), vg.dz.end()))));
     TRY(upload(h, &h->faceL0, hg[0].faceL));
     TRY(upload(h, &h->faceR0, hg[0].faceR));
     TRY(upload(h, &h->faceSide0, hg[0].faceSide));
     TRY(upload(h, &h->nbrSide0, hg[0].nbr_side));
     TRY(dalloc(h, &h->flag, 1));
+    TRY(dalloc(h, &h->timeout, 1));
+    CK(cudaMemset(h->timeout, 0, sizeof(unsigned int)));
     // MG_FP32_P64 stores and computes as MG_FP32; only the finest level's elimination differs
     const int prec = prm->vcycle_precision == MG_FP32_P64 ? MG_FP32 : prm->vcycle_precision;
-    h->pivot64 = prm->vcycle_precision == MG_FP32_P64;
     h->lv.resize(L);
     for (int l = 0; l < L; ++l) {
         DevLevel& d = h->lv[l];
@@ -1282,23 +1341,49 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
         TRY(upload(h, &d.Th64, co[l].Th));
         TRY(upload(h, &d.Tv64, co[l].Tv));
         const size_t Nl = (size_t)nlev * G.ncol;
+        const size_t Np = gamma2 > 0.0 ? Nl : (size_t)nlev * mg::padded(G.n);   // an FP32 field
+        if (prec != MG_FP64) TRY(upload(h, &d.rA32, rA));
+        if (gamma2 > 0.0) {
+            if (prec != MG_FP64) {
+                TRY(upload(h, &d.Th32, co[l].Th));
+                TRY(upload(h, &d.Tv32, co[l].Tv));
+            }
+        } else {
+            std::vector<double> wA(G.ncol);
+            for (int c = 0; c < G.ncol; ++c) wA[c] = G.area[c] * h->scale;
+            TRY(upload(h, &d.wA64, wA));
+            for (double** p : {&d.te64, &d.tn64, &d.e64, &d.ip64}) TRY(dalloc(h, p, Nl));
+            for (double** p : {&d.tbw64, &d.tbs64}) TRY(dalloc(h, p, (size_t)nlev * 6 * G.n));
+            TRY(dalloc(h, &d.tv64, Nl + G.ncol));
+            if (prec == MG_FP32) {
+                for (float** p : {&d.te32, &d.tn32}) TRY(dalloc(h, p, Np));
+                TRY(dalloc(h, &d.tv32, Np + mg::padded(G.n)));
+            } else if (prec == MG_FP32_BF16COEF) {
+                for (bf16** p : {&d.te16, &d.tn16}) TRY(dalloc(h, p, Np));
+                TRY(dalloc(h, &d.tv16, Np + mg::padded(G.n)));
+            }
+            if (prec != MG_FP64) {
+                TRY(dalloc(h, &d.ip32, Np));
+                if (l == 0 && prm->vcycle_precision == MG_FP32_P64)
+                    for (double** p : {&d.ipd, &d.md, &d.ed}) TRY(dalloc(h, p, Np));
+                TRY(dalloc(h, &d.hd, 4 * (size_t)G.ncol));
+                k_rims<<<dim3((G.ncol + 127) / 128, 4), 128>>>(G.n, G.ncol, d.nbr, d.hd);
+            }
+            if (l + 1 < L) {
+                TRY(dalloc(h, &d.par, 5 * (size_t)G.ncol));
+                k_parents<<<dim3((G.ncol + 127) / 128, 5), 128>>>(G.n, G.ncol, d.nbr, d.par);
+            }
+            TRY(pack_level(h, l, nullptr));
+        }
         TRY(dalloc(h, &d.x64[0], Nl));
         TRY(dalloc(h, &d.x64[1], Nl));
         TRY(dalloc(h, &d.b64, Nl));
         TRY(dalloc(h, &d.r64, Nl));
         if (prec != MG_FP64) {
-            TRY(upload(h, &d.rA32, rA));
-            if (prec == MG_FP32) {
-                TRY(upload(h, &d.Th32, co[l].Th));
-                TRY(upload(h, &d.Tv32, co[l].Tv));
-            } else {
-                TRY(upload(h, &d.Th16, co[l].Th));
-                TRY(upload(h, &d.Tv16, co[l].Tv));
-            }
-            TRY(dalloc(h, &d.x32[0], Nl));
-            TRY(dalloc(h, &d.x32[1], Nl));
-            TRY(dalloc(h, &d.b32, Nl));
-            TRY(dalloc(h, &d.r32, Nl));
+            TRY(dalloc(h, &d.x32[0], Np));
+            TRY(dalloc(h, &d.x32[1], Np));
+            TRY(dalloc(h, &d.b32, Np));
+            TRY(dalloc(h, &d.r32, Np));
         }
         if (gamma2 > 0.0) {
             // 9-cell stencil: flux between cells k and k + 2 of every column,
@@ -1326,10 +1411,11 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
             std::vector<double> w(4 * (size_t)Gc.ncol);
             for (int C = 0; C < Gc.ncol; ++C)
                 for (int q = 0; q < 4; ++q) w[(size_t)q * Gc.ncol + C] = G.area[mg::child_col(G.n, C, q)] / Gc.area[C];
-            TRY(upload(h, &d.w64, w));
+            if (gamma2 > 0.0) TRY(upload(h, &d.w64, w));
             if (prec != MG_FP64) TRY(upload(h, &d.w32, w));
         }
     }
+    for (int l = 0; l < L; ++l) TRY(build_maps(h, l));
     {
         // finest level: a_side = Th[k][face] / area, a_up = Tv[k+1] / dz, a_dn = Tv[k] / dz,
         // and the diagonal 1 + sum of the six
@@ -2081,14 +2167,13 @@ mg_status mg_smooth(mg_handle* h, int32_t level, const double* b, const double* 
     DeviceGuard dg(h->device);
     cudaStream_t s = S(stream);
     DevLevel& d = h->lv[level];
-    const Lvl<double, double> L = View<double, double>::lvl(h, level);
+    const Lvl64 L = lvl64(h, level);
     const size_t n = cells(h, level);
     const double* cur = x_in;
     for (int i = 0; i < sweeps; ++i) {
         double* dst = (cur == d.x64[0]) ? d.x64[1] : d.x64[0];
         if (h->nine) TRY((sweep9<double, double, double>(h, level, cur, b, dst, h->prm.omega, s)));
-        else TRY((sweep_any<double, double, double, double>(h, level, L, cur, (const double*)nullptr, 0, b, nullptr,
-                                                            dst, h->prm.omega, s)));
+        else TRY(launch_sweep64(h, level, L, cur, nullptr, 0, b, true, nullptr, dst, h->prm.omega, s));
         cur = dst;
     }
     if (cur == nullptr) CK(cudaMemsetAsync(x_out, 0, n * sizeof(double), s));
@@ -2102,8 +2187,7 @@ mg_status mg_residual_restrict(mg_handle* h, int32_t level, const double* b, con
     if (level + 1 >= h->L || !b || !x || !bc) return MG_ERR_ARG;
     DeviceGuard dg(h->device);
     if (h->nine) return restrict9<double, double, double>(h, level, x, b, bc, S(stream));
-    return launch_restrict<double, double, false, double, double, double>(
-        h, level, View<double, double>::lvl(h, level), x, b, h->lv[level].w64, bc, h->lv[level + 1].ncol, S(stream));
+    return launch_restrict64<true>(h, level, x, b, bc, S(stream));
 }
 
 mg_status mg_prolong_add(mg_handle* h, int32_t level, const double* xc, double* x, void* stream) {
@@ -2173,8 +2257,7 @@ mg_status mg_autotune(mg_handle* h, int32_t* choices, void* stream) {
         h->recs.clear();
         return MG_OK;
     };
-    // sweep blocks: 64 or 128 threads (two warps hold the two halves of 32 columns; the
-    // kernel's launch bounds allow 128)
+    // FP32 sweeps: 64: register chunks, 128: tensor-copy tiles where the level has them
     std::vector<int> best_bd(L, 0);
     std::vector<double> best_t(L, 1e300);
     for (int bd : {64, 128}) {
@@ -2184,17 +2267,16 @@ mg_status mg_autotune(mg_handle* h, int32_t* choices, void* stream) {
             if (sweep_ms[l] < best_t[l]) best_t[l] = sweep_ms[l], best_bd[l] = bd;
     }
     for (int l = 0; l < L; ++l) h->lv[l].sweep_bd = best_bd[l];
-    // residual + restriction: levels per thread, copy ring or register ring
+    // residual + restriction: levels per thread
     std::vector<int> best_kc(L, 0), best_as(L, -1);
     std::fill(best_t.begin(), best_t.end(), 1e300);
-    for (int as : {0, 1})
-        for (int kc : {4, 8, 16, 24, 35, 70}) {
-            for (int l = 0; l < L; ++l) h->lv[l].restrict_kc = kc, h->lv[l].restrict_async = as;
-            TRY(measure());
-            for (int l = 0; l + 1 < L; ++l)
-                if (restr_ms[l] < best_t[l]) best_t[l] = restr_ms[l], best_kc[l] = kc, best_as[l] = as;
-        }
-    for (int l = 0; l < L; ++l) h->lv[l].restrict_kc = best_kc[l], h->lv[l].restrict_async = best_as[l];
+    for (int kc : {4, 8, 16, 24, 35, 70}) {
+        for (int l = 0; l < L; ++l) h->lv[l].restrict_kc = kc;
+        TRY(measure());
+        for (int l = 0; l + 1 < L; ++l)
+            if (restr_ms[l] < best_t[l]) best_t[l] = restr_ms[l], best_kc[l] = kc, best_as[l] = 0;
+    }
+    for (int l = 0; l < L; ++l) h->lv[l].restrict_kc = best_kc[l];
     // the cached GCR graphs hold the old launch shapes
     for (auto& row : h->gexec)
         for (cudaGraphExec_t& g : row)
@@ -2293,7 +2375,7 @@ extern "C" mg_status mg_smooth_noalloc(mg_handle* h, int32_t level, const double
     double* scratch = nullptr;
     TRY(scratch_address(h->device, &scratch));
     cudaStream_t s = S(stream);
-    const Lvl<double, double> L = View<double, double>::lvl(h, level);
+    const Lvl64 L = lvl64(h, level);
     if (sweeps == 0) {
         if (!x_in) CK(cudaMemsetAsync(x_out, 0, n * sizeof(double), s));
         else if (x_in != x_out) CK(cudaMemcpyAsync(x_out, x_in, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -2309,8 +2391,7 @@ extern "C" mg_status mg_smooth_noalloc(mg_handle* h, int32_t level, const double
     const double* cur = x_in;
     for (int i = 0; i < sweeps; ++i) {
         double* dst = to_out ? x_out : scratch;
-        TRY((sweep_any<double, double, double, double>(nullptr, level, L, cur, (const double*)nullptr, 0, b,
-                                                       nullptr, dst, h->prm.omega, s)));
+        TRY(launch_sweep64(nullptr, level, L, cur, nullptr, 0, b, true, nullptr, dst, h->prm.omega, s));
         cur = dst;
         to_out = !to_out;
     }

@@ -1,0 +1,85 @@
+// Launcher of the FP32 column sweep (sweep32.cuh, sweep_tma.cuh).
+#pragma once
+
+#include <algorithm>
+#include <type_traits>
+
+#include "sweep_tma.cuh"
+
+namespace mg {
+namespace {
+
+// Levels per chunk of the register sweep: 10 where the level fills the GPU, 5 below 2M cells (twice
+// the threads); columns of more than 80 levels take 8, so that a block has at most 16 warps.
+constexpr int BIG_K = 10, SMALL_K = 5, TALL_K = 8;
+constexpr double SMALL_CELLS = 2e6;
+
+template <typename C, typename P, int MODE, typename B, typename O, bool BRAW, int K>
+cudaError_t go(const SweepCall32<C, P>& q, cudaStream_t s) {
+    const int G = ((q.L.nlev + 1) / 2 + K - 1) / K;
+    k_sweep32<C, P, MODE, B, O, BRAW, K><<<(q.L.ncol + 31) / 32, 64 * G, 0, s>>>(
+        q.L, q.x, q.xc, static_cast<const B*>(q.b), q.bcopy, static_cast<O*>(q.xo), (float)q.omega);
+    return cudaGetLastError();
+}
+
+template <typename C, typename P, int MODE, typename B, typename O, bool BRAW>
+cudaError_t shape(const SweepCall32<C, P>& q, cudaStream_t s) {
+    if (q.L.nlev > 80) return go<C, P, MODE, B, O, BRAW, TALL_K>(q, s);
+    if ((double)q.L.nlev * q.L.ncol < SMALL_CELLS) return go<C, P, MODE, B, O, BRAW, SMALL_K>(q, s);
+    return go<C, P, MODE, B, O, BRAW, BIG_K>(q, s);
+}
+
+template <typename C, typename P, int MODE, typename O, bool BRAW, int K, bool FULL>
+cudaError_t go_tma(const SweepCall32<C, P>& q, cudaStream_t s) {
+    const TmaLayout<C, P, MODE, BRAW, K> Y(q.L.nlev);
+    auto kern = k_sweep_tma<C, P, MODE, O, BRAW, K, FULL>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Y.total);
+    if (e != cudaSuccess) return e;
+    const int threads = 64 * tma_chunks(q.L.nlev, K);
+    // tiles: up to 32 columns of a row, a multiple of 16 bytes of the couplings wide (tensor coordinates)
+    constexpr int Q = 16 / (int)sizeof(C);
+    const int tr = (q.L.n + TMA_COLS - 1) / TMA_COLS, tw = ((q.L.n + tr - 1) / tr + Q - 1) / Q * Q;
+    const int per_sm = std::max(1, std::min({227 * 1024 / (Y.total + 1024), tma_blocks(MODE, BRAW, sizeof(P)) * tma_threads(K) / threads, 8}));
+    const int grid = std::min(6 * q.L.n * tr, per_sm * q.nsm);
+    kern<<<grid, threads, Y.total, s>>>(*q.maps, q.L, static_cast<const double*>(BRAW ? q.b : nullptr), q.bcopy,
+                                        static_cast<O*>(q.xo), (float)q.omega, tr, tw, q.timeout);
+    return cudaGetLastError();
+}
+
+// tiles where the level has them, else register chunks
+template <typename C, typename P, int MODE, typename O, bool BRAW>
+cudaError_t form(const SweepCall32<C, P>& q, cudaStream_t s) {
+    if constexpr (MODE != XM_PROLONG0) {
+        if (q.maps) {
+            if (q.L.nlev > tma_max_levels(7)) return go_tma<C, P, MODE, O, BRAW, 8, false>(q, s);
+            if (q.L.nlev == tma_chunks(q.L.nlev, 7) * 14) return go_tma<C, P, MODE, O, BRAW, 7, true>(q, s);
+            return go_tma<C, P, MODE, O, BRAW, 7, false>(q, s);
+        }
+    }
+    return shape<C, P, MODE, typename std::conditional<BRAW, double, float>::type, O, BRAW>(q, s);
+}
+
+template <typename C, typename P, int MODE>
+cudaError_t outs(const SweepCall32<C, P>& q, cudaStream_t s) {
+    if (q.out64) return form<C, P, MODE, double, false>(q, s);
+    return form<C, P, MODE, float, false>(q, s);
+}
+
+}  // namespace
+
+template <typename C, typename P>
+cudaError_t sweep32_run(const SweepCall32<C, P>& q, cudaStream_t s) {
+    if (q.raw) {
+        if (q.mode != XM_ZERO || !q.bcopy || q.out64) return cudaErrorInvalidValue;
+        return form<C, P, XM_ZERO, float, true>(q, s);
+    }
+    switch (q.mode) {
+        case XM_ZERO: return outs<C, P, XM_ZERO>(q, s);
+        case XM_PLAIN: return outs<C, P, XM_PLAIN>(q, s);
+        case XM_PROLONG: return outs<C, P, XM_PROLONG>(q, s);
+        case XM_PROLONG0: return outs<C, P, XM_PROLONG0>(q, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace mg
