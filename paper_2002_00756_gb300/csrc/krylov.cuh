@@ -11,11 +11,6 @@
 
 #include "kernels.cuh"
 
-// fused GCR apply in diagonal form (1) or difference form (0)
-#ifndef MG_APPLY_DIAG
-#define MG_APPLY_DIAG 1
-#endif
-
 namespace mg {
 
 constexpr int RED_THREADS = 256;
@@ -656,26 +651,49 @@ __global__ void k_mx_cells(MixedDev M, const double* __restrict__ uh, const doub
     else yp[o] = __ldg(p + o) - div_cell<true>(M, k, c, uh, uv);
 }
 
-// Pressure-system GCR pass 1: w = H z (FP64, Eq. helmholtz_operator) for the levels
-// [k0, k0 + kchunk) of one column per thread, fused with the GCR sums of the new direction J.
-// The finest level keeps its six couplings per cell premultiplied in FP64 (a6[side][k][c],
-// sides E, W, N, S, up, down), so H z costs 6 differences and 6 fused multiply-adds: FP64
-// issue, not memory, bounds this kernel on GB300.
+// Pressure-system GCR pass 1: w = H z (FP64, Eq. helmholtz_operator) fused with the GCR sums of the
+// new direction J.  The finest level keeps its six couplings and the diagonal 1 + sum_f a_f per cell
+// premultiplied in FP64 (a6[side][k][c], sides E, W, N, S, up, down, then the diagonal), so H z costs 7
+// and the sums J + 2 FP64 operations per cell: the FP64 pipe (two lanes per clock and SM), not memory,
+// bounds this kernel.
+//
+// The units of work, 32 columns x kchunk levels, are dealt out over a grid that is resident at once,
+// and a warp keeps its sums over all its units: one reduction per warp (it runs on the FP64 pipe as
+// well) instead of one per 24 levels, and no last wave of blocks on a part of the chip.  At C192L70
+// 254 / 281 / 307 / 336 / 365 us for J = 0..4 (one unit per thread, blocks in waves: 280 / 314 / 343 / 381
+// / 417; the FP64 pipe's bound: 223 / 248 / 273 / 298 / 322); C48L30 20-33 us instead of 35-49.  Two, four
+// and five blocks per SM: 256-369, 256-385, 258-391.
+constexpr int APPLY_BLOCKS = 3;   // resident blocks per SM
+
+// Levels per unit: the fewest rounds x (levels + about one level's worth of prologue); more than 18
+// levels in a row cost more in cache reuse than they save.
+inline int apply_chunk(int groups, int nlev, int warps) {
+    int best = 1;
+    double t = 1e300;
+    for (int kc = 1; kc <= 18 && kc <= nlev; ++kc) {
+        const long long units = (long long)groups * ((nlev + kc - 1) / kc);
+        const double tk = (double)((units + warps - 1) / warps) * (kc + 1);
+        if (tk <= t) t = tk, best = kc;
+    }
+    return best;
+}
+
 template <int J>
-__global__ void __launch_bounds__(RED_THREADS) k_apply_gcr(Lvl<double, double> L, const double* __restrict__ a6,
-                                                           const double* __restrict__ z, double* __restrict__ w,
-                                                           const double* __restrict__ Wb, size_t ld,
-                                                           const double* __restrict__ r, int kchunk,
-                                                           double* partials, unsigned int* ticket, GcrScal* S) {
+__global__ void __launch_bounds__(RED_THREADS, APPLY_BLOCKS) k_apply_gcr(
+    Lvl<double, double> L, const double* __restrict__ a6, const double* __restrict__ z, double* __restrict__ w,
+    const double* __restrict__ Wb, size_t ld, const double* __restrict__ r, int kchunk, int nchunk, double* partials,
+    unsigned int* ticket, GcrScal* S) {
     double v[J + 2], t[J + 2];
 #pragma unroll
     for (int i = 0; i < J + 2; ++i) v[i] = 0.0;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < L.ncol) {
-        const size_t ncol = L.ncol, N = (size_t)L.nlev * ncol;
-        const int k0 = blockIdx.y * kchunk;
-        const int k1 = min(L.nlev, k0 + kchunk);
-        int nb[4];
+    const unsigned ncol = L.ncol, ngroup = (ncol + 31) >> 5, nunit = ngroup * nchunk;
+    const unsigned lane = threadIdx.x & 31, nwarp = gridDim.x * (RED_THREADS / 32);
+    const size_t N = (size_t)L.nlev * ncol;
+    for (unsigned u = blockIdx.x * (RED_THREADS / 32) + (threadIdx.x >> 5); u < nunit; u += nwarp) {
+        const unsigned ch = u / ngroup, c = (u - ch * ngroup) * 32 + lane;
+        if (c >= ncol) continue;
+        const int k0 = ch * kchunk, k1 = min(L.nlev, k0 + kchunk);
+        unsigned nb[4];
 #pragma unroll
         for (int s = 0; s < 4; ++s) nb[s] = __ldg(L.nbr + s * ncol + c);
         double xm = k0 > 0 ? __ldg(z + (size_t)(k0 - 1) * ncol + c) : 0.0;
@@ -683,9 +701,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_apply_gcr(Lvl<double, double> L
 #pragma unroll 2
         for (int k = k0; k < k1; ++k) {
             const size_t o = (size_t)k * ncol, e = o + c;
-            const double xp = (k + 1 < L.nlev) ? __ldg(z + o + ncol + c) : 0.0;
-#if MG_APPLY_DIAG
-            // diagonal form: (1 + sum_f a_f) x_i - sum_f a_f x_j, 7 FP64 operations
+            const double xp = (k + 1 < L.nlev) ? __ldg(z + e + ncol) : 0.0;
             double we = __ldg(a6 + 6 * N + e) * x0;
             we = fma(-__ldg(a6 + e), __ldg(z + o + nb[0]), we);
             we = fma(-__ldg(a6 + N + e), __ldg(z + o + nb[1]), we);
@@ -693,15 +709,6 @@ __global__ void __launch_bounds__(RED_THREADS) k_apply_gcr(Lvl<double, double> L
             we = fma(-__ldg(a6 + 3 * N + e), __ldg(z + o + nb[3]), we);
             we = fma(-__ldg(a6 + 4 * N + e), xp, we);
             we = fma(-__ldg(a6 + 5 * N + e), xm, we);
-#else
-            double we = x0;
-            we = fma(__ldg(a6 + e), x0 - __ldg(z + o + nb[0]), we);
-            we = fma(__ldg(a6 + N + e), x0 - __ldg(z + o + nb[1]), we);
-            we = fma(__ldg(a6 + 2 * N + e), x0 - __ldg(z + o + nb[2]), we);
-            we = fma(__ldg(a6 + 3 * N + e), x0 - __ldg(z + o + nb[3]), we);
-            we = fma(__ldg(a6 + 4 * N + e), x0 - xp, we);
-            we = fma(__ldg(a6 + 5 * N + e), x0 - xm, we);
-#endif
             w[e] = we;
             gcr_accumulate<J>(v, we, __ldg(r + e), Wb, ld, e);
             xm = x0;

@@ -806,9 +806,6 @@ mg_status dispatch_j(int j, A&&... a) {
     }
 }
 
-// column-chunk of the fused apply: long enough to amortise the per-thread reduction
-constexpr int GCR_APPLY_KCHUNK = 24;
-
 template <int J>
 struct RunSums {
     static mg_status run(mg_handle* h, size_t n, const double* w, cudaStream_t s) {
@@ -825,11 +822,13 @@ struct RunApplyGcr {
     static mg_status run(mg_handle* h, const double* z, double* w, cudaStream_t s) {
         const Lvl<double, double> L = View<double, double>::lvl(h, 0);
         const double nc = (double)L.nlev * L.ncol;
-        // z, the couplings (6, and the diagonal in diagonal form), w, r, w_i
-        Prof pr(h, MG_K_APPLY, 0, nc * 8.0 * (1 + 6 + MG_APPLY_DIAG + 1 + 1 + J), s, J);
-        const int kc = GCR_APPLY_KCHUNK;
-        dim3 grid((L.ncol + mg::RED_THREADS - 1) / mg::RED_THREADS, (L.nlev + kc - 1) / kc);
-        mg::k_apply_gcr<J><<<grid, mg::RED_THREADS, 0, s>>>(L, h->a6, z, w, h->W, h->glen, h->r, kc, h->partials,
+        // z, the couplings (6 and the diagonal), w, r, w_i
+        Prof pr(h, MG_K_APPLY, 0, nc * 8.0 * (1 + 7 + 1 + 1 + J), s, J);
+        const int groups = (L.ncol + 31) / 32, per_block = mg::RED_THREADS / 32;
+        const int kc = mg::apply_chunk(groups, L.nlev, mg::APPLY_BLOCKS * h->nsm * per_block), nk = (L.nlev + kc - 1) / kc;
+        const int grid = std::min(mg::APPLY_BLOCKS * h->nsm, (int)(((long long)groups * nk + per_block - 1) / per_block));
+        mg::k_apply_gcr<J><<<grid, mg::RED_THREADS, 0, s>>>(L, h->a6, z, w, h->W, h->glen, h->r, kc, nk,
+                                                            h->partials,
                                                             h->tickets + TK_SUMS, h->gs);
         CK(cudaGetLastError());
         return MG_OK;
@@ -1534,10 +1533,8 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
     TRY(dalloc(h, &h->adj, N0));
     TRY(dalloc(h, &h->gs, 1));
     {
-        const size_t apply_blocks = (size_t)((ncol0 + mg::RED_THREADS - 1) / mg::RED_THREADS) *
-                                    ((nlev + GCR_APPLY_KCHUNK - 1) / GCR_APPLY_KCHUNK);
-        const size_t blocks = apply_blocks > (size_t)h->red_grid ? apply_blocks : (size_t)h->red_grid;
-        h->npartials = blocks * (2 * mg::MAXR + 2);
+        // (every reduction's grid is at most red_grid blocks)
+        h->npartials = (size_t)h->red_grid * (2 * mg::MAXR + 2);
         TRY(dalloc(h, &h->partials, h->npartials));
     }
     TRY(dalloc(h, &h->tickets, TK_COUNT));

@@ -67,6 +67,24 @@ def test_both_forms_of_the_sweep_agree_bit_for_bit(mg, n, nlev, precision):
     h.destroy()
 
 
+@pytest.mark.parametrize("n,nlev,levels", [(2, 1, 1), (5, 3, 1), (10, 19, 2), (44, 71, 2)])
+def test_recurred_residual_is_the_true_one(mg, n, nlev, levels):
+    """The fused apply's units (32 columns by up to 18 levels; one level, a ragged last group of
+    columns, a ragged last run of levels) add up: the solve's own residual norm is that of b - A x.
+    They drift apart by a few eps ||A|| ||x|| per iteration, ||A|| ~ 1e3 here: 1e-10 of ||b|| at most."""
+    cfg = syn.small_config(n, nlev, levels=levels, seed=syn.BASE_SEED + 760 + n)
+    inp = syn.make_inputs(cfg)
+    h = mg.mg_setup_config(cfg, inp)
+    b = torch.from_numpy(inp["rhs"]).cuda()
+    x, y = torch.empty_like(b), torch.empty_like(b)
+    for tol in (1e-3, 1e-7):
+        info = mg.pressure_solve(h, b, x, tol)
+        mg.helmholtz_apply(h, x, y)
+        true = float((b - y).norm() / b.norm())
+        assert info.converged and abs(true - info.rel_res) <= 1e-10, (info, true)
+    h.destroy()
+
+
 def test_smoothing_of_misaligned_vectors(mg):
     """Vectors that start on an odd double (8-byte alignment only) give what aligned ones give."""
     cfg = syn.small_config(20, 9, levels=3, seed=syn.BASE_SEED + 720)
