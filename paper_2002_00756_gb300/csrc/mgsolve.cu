@@ -333,9 +333,12 @@ mg_status launch_apply(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, Y*
     return MG_OK;
 }
 
-// FP32 levels of this many cells run their sweeps on tensor-copy tiles: below, a tile per block leaves
-// SMs idle and the register sweep is as fast.
-constexpr double TMA_CELLS = 8e5;
+// FP32 levels that run their sweeps on tensor-copy tiles rather than register chunks.  A V-cycle on its own /
+// eight side by side [us each] with the chunks and with the tiles on levels of these cells:
+//   columns of more than 40 levels, whose chunks fill an SM with one block, 250k: C32L50 74.0/28.2 and 72.7/25.5,
+//   C32L70 94/35 and 88/32, C48L41 89/52 and 86/41 (C48L50 92.9/55 and 94.9/50; C24L70, 242k: 92.9 and 93.7);
+//   up to 40 levels, 700k: C64L30 81/47 and 80/42 (C56L30, 564k: 71 and 78; C48L37 77/34 and 81/36).
+inline bool tma_level(int nlev, int ncol) { return (double)nlev * ncol >= (nlev > 40 ? 2.5e5 : 7e5); }
 
 inline bool aligned(const void* p, size_t bytes) { return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) == 0; }
 
@@ -416,7 +419,7 @@ mg_status launch_sweep32(mg_handle* h, int lev, const float* x, const float* xc,
     if (xc) per += 1.0;
     Prof pr(h, MG_K_SWEEP, lev, (double)L.nlev * L.ncol * per, s, mode);
     const mg::SweepMaps* maps = nullptr;
-    const bool tiles = d.sweep_bd > 0 ? d.sweep_bd == 128 : (double)L.nlev * L.ncol >= TMA_CELLS;
+    const bool tiles = d.sweep_bd > 0 ? d.sweep_bd == 128 : tma_level(L.nlev, L.ncol);
     if (tiles && d.maps.size() == 2 && mode != mg::XM_PROLONG0) maps = &d.maps[x == d.x32[1]];
     const mg::SweepCall32<C, P> q{L, mode, x, xc, b, raw, bcopy, xo, out64, om, maps, h->nsm, h->timeout};
     CK((mg::sweep32_run<C, P>(q, s)));
