@@ -498,91 +498,11 @@ struct MixedDev {
     // coefficient gradient: d(kappa_f / d_f) / d g_i = c_s dt / (2 d_f) for both cells of f
     const double* cdh;              // [nfh]      c_s dt / (2 centre distance)
     const double* cdv;              // [nlev+1]   c_s dt / (2 dzc), 0 on surface and lid
+    // 1 / W_f of interior faces as factors at hand: kd_h divv rel and kd_v / (c_s dt area)
+    const double* rel;              // [nfh]      1 / ((c_s dt)^2 edge length)
+    const double* rcA;              // [ncol]     1 / (c_s dt area)
     double eps;                     // strength of B_w
 };
-
-// (D u)_i, velocities optionally divided by the lumped mass
-template <bool LUMP>
-__device__ __forceinline__ double div_cell(const MixedDev& M, int k, int c, const double* __restrict__ uh,
-                                           const double* __restrict__ uv) {
-    const size_t ncol = M.ncol;
-    double s = 0.0;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        const int f = __ldg(M.fof + d * ncol + c);
-        const double u = __ldg(uh + (size_t)k * M.nfh + f);
-        s += __ldg(M.sdiv + d * ncol + c) * (LUMP ? u * __ldg(M.rmlump_h + f) : u);
-    }
-    double v = 0.0;
-    if (k + 1 < M.nlev) {
-        const size_t o = (size_t)(k + 1) * ncol + c;
-        v += LUMP ? __ldg(uv + o) * __ldg(M.rmlump + o) : __ldg(uv + o);
-    }
-    if (k > 0) {
-        const size_t o = (size_t)k * ncol + c;
-        v -= LUMP ? __ldg(uv + o) * __ldg(M.rmlump + o) : __ldg(uv + o);
-    }
-    return s + __ldg(M.divv + k) * v;
-}
-
-// velocity rows on horizontal faces: yh = M_h uh + kd (p_R - p_L)          [MODE 0]
-// Step 3 on horizontal faces:         yh = (uh - kd (p_R - p_L)) / m_h    [MODE 1, times 1 / m_h]
-// rows of A-hat:                      yh = (W^-1 M_h^T W uh) + kd (p_R - p_L)  [MODE 2]
-template <int MODE>
-__global__ void k_mx_faces_h(MixedDev M, const double* __restrict__ uh, const double* __restrict__ p,
-                             double* __restrict__ yh) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = blockIdx.y;
-    if (f >= M.nfh) return;
-    const size_t o = (size_t)k * M.nfh + f, op = (size_t)k * M.ncol;
-    const double g = __ldg(M.kd_h + o) * (__ldg(p + op + __ldg(M.faceR + f)) - __ldg(p + op + __ldg(M.faceL + f)));
-    if (MODE == 0) {
-        double m = M.ms * __ldg(uh + o);
-        const double* ul = uh + (size_t)k * M.nfh;
-        for (int t = 0; t < M.ncf; ++t)
-            m += __ldg(M.wf + (size_t)t * M.nfh + f) * __ldg(ul + __ldg(M.cf + (size_t)t * M.nfh + f));
-        yh[o] = m + g;
-    } else if (MODE == 2) {
-        const double* ul = uh + (size_t)k * M.nfh;
-        const double* Wl = M.Wf + (size_t)k * M.nfh;
-        double m = 0.0;
-        for (int t = 0; t < M.ncf; ++t) {
-            const int gf = __ldg(M.cf + (size_t)t * M.nfh + f);
-            m += __ldg(M.wfT + (size_t)t * M.nfh + f) * (__ldg(Wl + gf) * __ldg(ul + gf));
-        }
-        yh[o] = (M.ms * __ldg(uh + o) + m / __ldg(Wl + f)) + g;
-    } else {
-        yh[o] = (__ldg(uh + o) - g) * __ldg(M.rmlump_h + f);
-    }
-}
-
-// velocity rows on vertical faces: yv = M-bar uv + kd (p_kf - p_kf-1)   [MODE 0]
-// rows of A-hat: the couplings of M-bar^T (face kf+1's coupling down, face kf-1's up)
-// weighted by W_neighbour / W_kf                                        [MODE 2]
-// Step 3 on vertical faces:         yv = (uv - kd (p_kf - p_kf-1)) / m  [MODE 1]
-template <int MODE>
-__global__ void k_mx_faces_v(MixedDev M, const double* __restrict__ uv, const double* __restrict__ p,
-                             double* __restrict__ yv) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int kf = blockIdx.y;
-    if (c >= M.ncol) return;
-    const size_t ncol = M.ncol, o = (size_t)kf * ncol + c;
-    if (kf == 0 || kf == M.nlev) {
-        yv[o] = __ldg(uv + o);
-        return;
-    }
-    const double g = __ldg(M.kd_v + o) * (__ldg(p + (size_t)kf * ncol + c) - __ldg(p + (size_t)(kf - 1) * ncol + c));
-    if (MODE == 0) {
-        yv[o] = M.mv * __ldg(uv + o) + __ldg(M.w_up + o) * __ldg(uv + o + ncol) + __ldg(M.w_dn + o) * __ldg(uv + o - ncol) + g;
-    } else if (MODE == 2) {
-        const double* Wv = M.Wf + (size_t)M.nlev * M.nfh;
-        const double m = __ldg(M.w_dn + o + ncol) * (__ldg(Wv + o + ncol) * __ldg(uv + o + ncol)) +
-                         __ldg(M.w_up + o - ncol) * (__ldg(Wv + o - ncol) * __ldg(uv + o - ncol));
-        yv[o] = (M.mv * __ldg(uv + o) + m / __ldg(Wv + o)) + g;
-    } else {
-        yv[o] = (__ldg(uv + o) - g) * __ldg(M.rmlump + o);
-    }
-}
 
 // [out_u; out_p] = J S^-1 [in_u; in_p] (MULT false) or S J [in_u; in_p] (MULT true), with
 // S = diag(W, V) (V = area dz, the cell volumes) and J = diag(I, -I)
@@ -593,12 +513,12 @@ __global__ void k_mx_adj_scale(MixedDev M, size_t nu, const double* __restrict__
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nu + np; i += (size_t)gridDim.x * blockDim.x) {
         if (i < nu) {
             const double w = __ldg(M.Wf + i);
-            out_u[i] = MULT ? in_u[i] * w : in_u[i] / w;
+            out_u[i] = MULT ? in_u[i] * w : in_u[i] * recip64(w);
         } else {
             const size_t e = i - nu;
             const int k = (int)(e / M.ncol), c = (int)(e - (size_t)k * M.ncol);
             const double v = __ldg(area + c) * __ldg(dz + k);
-            out_p[e] = MULT ? -(in_p[e] * v) : -(in_p[e] / v);
+            out_p[e] = MULT ? -(in_p[e] * v) : -(in_p[e] * recip64(v));
         }
     }
 }
@@ -636,19 +556,6 @@ __global__ void k_mx_grad_beta(MixedDev M, const double* __restrict__ lam_v, con
     const int nlev = M.nlev;
     gup[o] = (kf >= 1 && kf + 1 <= nlev - 1) ? -M.eps * lam_v[o] * uv[o + ncol] : 0.0;
     gdn[o] = (kf >= 2 && kf <= nlev - 1) ? -M.eps * lam_v[o] * uv[o - ncol] : 0.0;
-}
-
-// pressure rows: yp = p + D u                           [MODE 0]
-// Step 1:        B  = rp - D M-ring^{-1} ru (p := rp)    [MODE 1]
-template <int MODE>
-__global__ void k_mx_cells(MixedDev M, const double* __restrict__ uh, const double* __restrict__ uv,
-                           const double* __restrict__ p, double* __restrict__ yp) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = blockIdx.y;
-    if (c >= M.ncol) return;
-    const size_t o = (size_t)k * M.ncol + c;
-    if (MODE == 0) yp[o] = __ldg(p + o) + div_cell<false>(M, k, c, uh, uv);
-    else yp[o] = __ldg(p + o) - div_cell<true>(M, k, c, uh, uv);
 }
 
 // Pressure-system GCR pass 1: w = H z (FP64, Eq. helmholtz_operator) fused with the GCR sums of the
@@ -716,6 +623,155 @@ __global__ void __launch_bounds__(RED_THREADS, APPLY_BLOCKS) k_apply_gcr(
         }
     }
     if (grid_reduce<J + 2>(v, partials, ticket, t)) gcr_coeffs<J>(t, S);
+}
+
+// Mixed system, the forms of k_mixed:
+//   MX_A         y = A [u; p]: velocity rows M u + kd (p_R - p_L), pressure rows p + D u
+//   MX_HAT       the same with W^-1 M^T W for M (rows of A-hat), from u and wu = W u
+//   MX_RHS       Step 1: B = r_p - D M-ring^{-1} r_u (pressure rows only; p = r_p)
+//   MX_UPDATE    Step 3: u' = M-ring^{-1} (r_u - kd (p_R - p_L)) (velocity rows only)
+//   MX_UPDATE_W  the same, and W u' to wu
+enum { MX_A = 0, MX_HAT = 1, MX_RHS = 2, MX_UPDATE = 3, MX_UPDATE_W = 4 };
+
+// Units of work: 32 horizontal faces, vertical faces or cells by a run of levels, dealt out over a grid
+// that is resident at once (as k_apply_gcr's).  Face numbers, couplings and weights of the columns are
+// read once per unit, not once per level; with J >= 0 the GCR sums of the new direction J are taken in
+// the same pass, while its rows are in registers (a pass over J + 2 vectors and three launches less).
+// The FP64 pipe bounds MX_A and MX_HAT: 29 and 34 operations per cell (18 / 22 of them on its two
+// horizontal faces) and 4 (J + 2) of the sums.  A-hat's weights therefore come from Step 3, which
+// stores W u' beside u' (one product per face instead of six), and its quotient by W from factors
+// that are loaded anyway.
+// C48L30, sums of 0..4 directions included, on average: MX_A 38 us (four launches of a thread per row and
+// level: 56), MX_HAT 54 us (91); the FP64 pipe's bound with J = 2: 32 and 36.  Steps 1 and 3 have few
+// registers and run on five blocks per SM.
+constexpr int mixed_blocks(int mode) { return mode >= MX_RHS ? 5 : APPLY_BLOCKS; }   // resident per SM
+
+template <int MODE, int J>
+__global__ void __launch_bounds__(RED_THREADS, mixed_blocks(MODE)) k_mixed(
+    MixedDev M, const double* __restrict__ u, const double* __restrict__ p, double* __restrict__ yu,
+    double* __restrict__ yp, double* __restrict__ wu, const double* __restrict__ Wb, size_t ld, const double* __restrict__ r, int kchunk,
+    int nchunk, double* partials, unsigned int* ticket, GcrScal* S) {
+    constexpr int NV = J >= 0 ? J + 2 : 1, JJ = J >= 0 ? J : 0;
+    double v[NV], t[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = 0.0;
+    const unsigned ncol = M.ncol, nfh = M.nfh, lane = threadIdx.x & 31, nwarp = gridDim.x * (RED_THREADS / 32);
+    constexpr bool UPD = MODE == MX_UPDATE || MODE == MX_UPDATE_W;
+    const unsigned gh = MODE == MX_RHS ? 0 : (nfh + 31) >> 5, gc = (ncol + 31) >> 5;
+    const unsigned G = MODE == MX_RHS ? gc : UPD ? gh + gc : gh + 2 * gc;
+    const size_t nh = (size_t)M.nlev * nfh, nu = nh + (size_t)(M.nlev + 1) * ncol;
+    const double *uv = u + nh, *wv = MODE == MX_HAT ? wu + nh : uv;
+    // row e of [u; p] comes out as y
+    auto put = [&](double* to, size_t e, double y) {
+        *to = y;
+        if (MODE == MX_UPDATE_W) wu[e] = __ldg(M.Wf + e) * y;
+        if constexpr (J >= 0) gcr_accumulate<JJ>(v, y, __ldg(r + e), Wb, ld, e);
+    };
+    for (unsigned q = blockIdx.x * (RED_THREADS / 32) + (threadIdx.x >> 5); q < G * nchunk; q += nwarp) {
+        const unsigned ch = q / G, g = q - ch * G;
+        const int k0 = ch * kchunk, k1 = min(M.nlev, k0 + kchunk);
+        if (g < gh) {   // horizontal faces
+            const unsigned f = g * 32 + lane;
+            if (f >= nfh) continue;
+            const unsigned fl = __ldg(M.faceL + f), fr = __ldg(M.faceR + f);
+            const bool coupled = !UPD && M.ncf > 0;
+            unsigned cf[6] = {};
+            double wt[6] = {};
+            if (coupled) {
+#pragma unroll
+                for (int i = 0; i < 6; ++i) {
+                    cf[i] = __ldg(M.cf + (size_t)i * nfh + f);
+                    wt[i] = __ldg((MODE == MX_HAT ? M.wfT : M.wf) + (size_t)i * nfh + f);
+                }
+            }
+            const double rm = UPD ? __ldg(M.rmlump_h + f) : 0.0, rel = MODE == MX_HAT ? __ldg(M.rel + f) : 0.0;
+#pragma unroll 2
+            for (int k = k0; k < k1; ++k) {
+                const double *ul = (MODE == MX_HAT ? wu : u) + (size_t)k * nfh, *pl = p + (size_t)k * ncol;
+                const size_t o = (size_t)k * nfh + f;
+                const double kd = __ldg(M.kd_h + o), dp = __ldg(pl + fr) - __ldg(pl + fl), uf = __ldg(u + o);
+                double y;
+                if (UPD) {
+                    y = fma(-kd, dp, uf) * rm;
+                } else {
+                    y = M.ms * uf;
+                    double m = 0.0;
+                    if (coupled) {
+                        if (MODE == MX_A) m = y;
+#pragma unroll
+                        for (int i = 0; i < 6; ++i) m = fma(wt[i], __ldg(ul + cf[i]), m);
+                        if (MODE == MX_A) y = m;
+                    }
+                    y = fma(kd, MODE == MX_HAT ? fma(rel * __ldg(M.divv + k), m, dp) : dp, y);
+                }
+                put(yu + o, o, y);
+            }
+        } else if (MODE != MX_RHS && g < gh + gc) {   // vertical faces; the last run has the lid's as well
+            const unsigned c = (g - gh) * 32 + lane;
+            if (c >= ncol) continue;
+            const int k2 = k1 == M.nlev ? k1 + 1 : k1;
+            const double rcA = MODE == MX_HAT ? __ldg(M.rcA + c) : 0.0;
+            double ub = k0 > 0 ? __ldg(uv + (size_t)(k0 - 1) * ncol + c) : 0.0, u0 = __ldg(uv + (size_t)k0 * ncol + c);
+            double pb = k0 > 0 ? __ldg(p + (size_t)(k0 - 1) * ncol + c) : 0.0;
+#pragma unroll 2
+            for (int k = k0; k < k2; ++k) {
+                const size_t o = (size_t)k * ncol + c;
+                double y = u0, ua = 0.0, pa = 0.0;
+                if (k < M.nlev) {
+                    ua = __ldg(uv + o + ncol);
+                    pa = __ldg(p + o);
+                    if (k > 0) {
+                        const double kd = __ldg(M.kd_v + o), dp = pa - pb;
+                        if (MODE == MX_A)
+                            y = fma(kd, dp, fma(__ldg(M.w_dn + o), ub, fma(__ldg(M.w_up + o), ua, M.mv * u0)));
+                        if (MODE == MX_HAT) {   // the couplings of the faces above and below to this one
+                            const double m = fma(__ldg(M.w_up + o - ncol), __ldg(wv + o - ncol),
+                                                 __ldg(M.w_dn + o + ncol) * __ldg(wv + o + ncol));
+                            y = fma(kd, fma(rcA, m, dp), M.mv * u0);
+                        }
+                        if (UPD) y = fma(-kd, dp, u0) * __ldg(M.rmlump + o);
+                    }
+                }
+                put(yu + nh + o, nh + o, y);
+                ub = u0;
+                u0 = ua;
+                pb = pa;
+            }
+        } else if (!UPD) {   // cells
+            const unsigned c = (MODE == MX_RHS ? g : g - gh - gc) * 32 + lane;
+            if (c >= ncol) continue;
+            unsigned ff[4];
+            double sd[4];
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+                ff[d] = __ldg(M.fof + d * ncol + c);
+                sd[d] = __ldg(M.sdiv + d * ncol + c);
+                if (MODE == MX_RHS) sd[d] *= __ldg(M.rmlump_h + ff[d]);
+            }
+            // flux through the faces below and above (none through surface and lid)
+            auto flux = [&](int k) {
+                if (k <= 0 || k >= M.nlev) return 0.0;
+                const size_t o = (size_t)k * ncol + c;
+                return MODE == MX_RHS ? __ldg(uv + o) * __ldg(M.rmlump + o) : __ldg(uv + o);
+            };
+            double below = flux(k0);
+#pragma unroll 2
+            for (int k = k0; k < k1; ++k) {
+                const double* ul = u + (size_t)k * nfh;
+                const size_t o = (size_t)k * ncol + c;
+                const double above = flux(k + 1);
+                double y = __ldg(p + o);
+#pragma unroll
+                for (int d = 0; d < 4; ++d) y = fma(MODE == MX_RHS ? -sd[d] : sd[d], __ldg(ul + ff[d]), y);
+                y = fma(MODE == MX_RHS ? -__ldg(M.divv + k) : __ldg(M.divv + k), above - below, y);
+                put(yp + o, nu + o, y);
+                below = above;
+            }
+        }
+    }
+    if constexpr (J >= 0) {
+        if (grid_reduce<NV>(v, partials, ticket, t)) gcr_coeffs<JJ>(t, S);
+    }
 }
 
 }  // namespace mg

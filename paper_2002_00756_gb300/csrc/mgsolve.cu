@@ -1010,31 +1010,37 @@ mg_status gcr(mg_handle* h, int sys, size_t n, const double* b, double* x, doubl
 }
 
 // ---- mixed operator and Schur-complement preconditioner ----
-mg_status mixed_apply_impl(mg_handle* h, const double* u, const double* p, double* yu, double* yp, cudaStream_t s) {
+// One form of k_mixed (krylov.cuh), with the GCR sums of direction J unless J < 0; wu: see there.
+template <int MODE, int J>
+mg_status launch_mixed(mg_handle* h, const double* u, const double* p, double* yu, double* yp, double* wu,
+                       cudaStream_t s) {
     const mg::MixedDev& M = h->md;
-    const size_t nh = (size_t)M.nlev * M.nfh;
-    const int bd = 128;
-    Prof pr(h, MG_K_MIXED, 0, 8.0 * (2.0 * h->nu + 3.0 * cells(h, 0)), s);
-    mg::k_mx_faces_h<0><<<dim3((M.nfh + bd - 1) / bd, M.nlev), bd, 0, s>>>(M, u, p, yu);
-    mg::k_mx_faces_v<0><<<dim3((M.ncol + bd - 1) / bd, M.nlev + 1), bd, 0, s>>>(M, u + nh, p, yu + nh);
-    mg::k_mx_cells<0><<<dim3((M.ncol + bd - 1) / bd, M.nlev), bd, 0, s>>>(M, u, u + nh, p, yp);
+    const int gh = (M.nfh + 31) / 32, gc = (M.ncol + 31) / 32, per_block = mg::RED_THREADS / 32;
+    const int G = MODE == mg::MX_RHS ? gc : MODE >= mg::MX_UPDATE ? gh + gc : gh + 2 * gc;
+    const int slots = mg::mixed_blocks(MODE) * h->nsm, kc = mg::apply_chunk(G, M.nlev, slots * per_block);
+    const int nk = (M.nlev + kc - 1) / kc;
+    const int grid = (int)std::min((long long)slots, ((long long)G * nk + per_block - 1) / per_block);
+    mg::k_mixed<MODE, J><<<grid, mg::RED_THREADS, 0, s>>>(M, u, p, yu, yp, wu, h->W, h->glen, h->r, kc, nk,
+                                                          h->partials, h->tickets + TK_SUMS, h->gs);
     CK(cudaGetLastError());
     return MG_OK;
 }
 
-// A-hat [u; p]: the mixed operator with its velocity mass replaced by W^-1 M-bar^T W
-mg_status mixed_apply_hat_impl(mg_handle* h, const double* u, const double* p, double* yu, double* yp,
-                               cudaStream_t s) {
-    const mg::MixedDev& M = h->md;
-    const size_t nh = (size_t)M.nlev * M.nfh;
-    const int bd = 128;
-    Prof pr(h, MG_K_MIXED, 0, 8.0 * (3.0 * h->nu + 3.0 * cells(h, 0)), s, 2);
-    mg::k_mx_faces_h<2><<<dim3((M.nfh + bd - 1) / bd, M.nlev), bd, 0, s>>>(M, u, p, yu);
-    mg::k_mx_faces_v<2><<<dim3((M.ncol + bd - 1) / bd, M.nlev + 1), bd, 0, s>>>(M, u + nh, p, yu + nh);
-    mg::k_mx_cells<0><<<dim3((M.ncol + bd - 1) / bd, M.nlev), bd, 0, s>>>(M, u, u + nh, p, yp);
-    CK(cudaGetLastError());
-    return MG_OK;
-}
+// y = A v (MX_A) or A-hat v (MX_HAT, wu = W v_u) of a concatenated v = [u; p], with the GCR sums of direction j
+template <int MODE>
+struct RunMixed {
+    template <int J>
+    struct K {
+        static mg_status run(mg_handle* h, const double* v, double* y, double* wu, cudaStream_t s) {
+            const size_t nu = (size_t)h->nu;
+            const double n = nu + cells(h, 0);
+            // u, kd (W u) per velocity row and the row, p; of the sums r and the stored directions
+            Prof pr(h, MG_K_MIXED, 0, 8.0 * ((MODE == mg::MX_HAT ? 3.0 : 2.0) * nu + 3.0 * cells(h, 0) + (J + 1) * n), s,
+                    MODE == mg::MX_HAT ? 2 : 0);
+            return launch_mixed<MODE, J>(h, v, v + nu, y, y + nu, wu, s);
+        }
+    };
+};
 
 template <bool MULT>
 mg_status mixed_adj_scale(mg_handle* h, const double* in_u, const double* in_p, double* out_u, double* out_p,
@@ -1046,23 +1052,19 @@ mg_status mixed_adj_scale(mg_handle* h, const double* in_u, const double* in_p, 
     return MG_OK;
 }
 
-mg_status schur_impl(mg_handle* h, const double* ru, const double* rp, double* u, double* p, cudaStream_t s) {
-    const mg::MixedDev& M = h->md;
-    const size_t nh = (size_t)M.nlev * M.nfh;
-    const int bd = 128;
+// wu: takes W u' as well (null: not wanted)
+mg_status schur_impl(mg_handle* h, const double* ru, const double* rp, double* u, double* p, double* wu,
+                     cudaStream_t s) {
     // Step 1: B = r_p - D M-ring^{-1} r_u
-    mg::k_mx_cells<1><<<dim3((M.ncol + bd - 1) / bd, M.nlev), bd, 0, s>>>(M, ru, ru + nh, rp, h->schurB);
-    CK(cudaGetLastError());
+    TRY((launch_mixed<mg::MX_RHS, -1>(h, ru, rp, nullptr, h->schurB, nullptr, s)));
     // Step 2: H Pi' = B by the pressure solver K_H(A_H, P_H, eps_H) (one V-cycle by default);
     // an inexact inner solve (BiCGStab at its iteration limit) is still a usable preconditioner
     double it = 0.0;
     const mg_status st = run_pressure_solver(h, h->schurB, p, s, &it);
     if (st != MG_OK && st != MG_ERR_NOT_CONVERGED) return st;
     // Step 3: u' = M-ring^{-1} (r_u - G Pi')
-    mg::k_mx_faces_h<1><<<dim3((M.nfh + bd - 1) / bd, M.nlev), bd, 0, s>>>(M, ru, p, u);
-    mg::k_mx_faces_v<1><<<dim3((M.ncol + bd - 1) / bd, M.nlev + 1), bd, 0, s>>>(M, ru + nh, p, u + nh);
-    CK(cudaGetLastError());
-    return MG_OK;
+    if (wu) return launch_mixed<mg::MX_UPDATE_W, -1>(h, ru, p, u, nullptr, wu, s);
+    return launch_mixed<mg::MX_UPDATE, -1>(h, ru, p, u, nullptr, nullptr, s);
 }
 
 // parents of the neighbours E, W, N, S and of the column itself, [5][ncol]
@@ -1496,12 +1498,14 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
                 if (found < 0) return MG_ERR_ARG;   // the coupling pattern is symmetric by construction
                 wfT[(size_t)t * nfh + f] = hm.wf[(size_t)found * nfh + gf];
             }
-        std::vector<double> cdh(nfh), cdv(nlev + 1, 0.0);
+        std::vector<double> cdh(nfh), cdv(nlev + 1, 0.0), rel(nfh), rcA(ncol0);
         for (int f = 0; f < nfh; ++f) cdh[f] = c / (2.0 * G.cdist[G.faceSide[f] * ncol0 + G.faceL[f]]);
         for (int kf = 1; kf < nlev; ++kf) cdv[kf] = c / (2.0 * vg.dzc[kf]);
+        for (int f = 0; f < nfh; ++f) rel[f] = 1.0 / (c * c * G.edge_len[G.faceSide[f] * ncol0 + G.faceL[f]]);
+        for (int col = 0; col < ncol0; ++col) rcA[col] = 1.0 / (c * G.area[col]);
         int32_t *fL, *fR, *dcf = nullptr;
         double *dkd_h, *dkd_v, *dsdiv, *dwu, *dwd, *dml, *ddivv, *dwf = nullptr, *dmlh, *dwfT = nullptr, *dWf, *dcdh,
-            *dcdv;
+            *dcdv, *drel, *drcA;
         TRY(upload(h, &fL, G.faceL));
         TRY(upload(h, &fR, G.faceR));
         TRY(upload(h, &dkd_h, kd_h));
@@ -1520,8 +1524,10 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
         TRY(upload(h, &dWf, Wf));
         TRY(upload(h, &dcdh, cdh));
         TRY(upload(h, &dcdv, cdv));
+        TRY(upload(h, &drel, rel));
+        TRY(upload(h, &drcA, rcA));
         h->md = mg::MixedDev{ncol0, nlev, nfh, fL, fR, h->lv[0].fof, dsdiv, dkd_h, dkd_v, dwu, dwd, dml, ddivv,
-                             hm.ncf, dcf, dwf, hm.ms, mv, dmlh, dwfT, dWf, dcdh, dcdv, mixed->eps};
+                             hm.ncf, dcf, dwf, hm.ms, mv, dmlh, dwfT, dWf, dcdh, dcdv, drel, drcA, mixed->eps};
         h->nu = (int64_t)nlev * nfh + (int64_t)NV0;
         TRY(dalloc(h, &h->schurB, N0));
         TRY(dalloc(h, &h->mb, (size_t)h->nu + N0));
@@ -2087,10 +2093,9 @@ mg_status mixed_solve(mg_handle* h, const double* rhs_u, const double* rhs_p, do
     CK(cudaMemcpyAsync(h->mb, rhs_u, nu * sizeof(double), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(h->mb + nu, rhs_p, np * sizeof(double), cudaMemcpyDeviceToDevice, s));
     auto A = [&](const double* v, double* y, int j, cudaStream_t q) {
-        TRY(mixed_apply_impl(h, v, v + nu, y, y + nu, q));
-        return gcr_sums(h, n, y, j, q);
+        return dispatch_j<RunMixed<mg::MX_A>::K>(j, h, v, y, nullptr, q);
     };
-    auto P = [&](const double* r, double* z, cudaStream_t q) { return schur_impl(h, r, r + nu, z, z + nu, q); };
+    auto P = [&](const double* r, double* z, cudaStream_t q) { return schur_impl(h, r, r + nu, z, z + nu, nullptr, q); };
     const mg_status st = gcr(h, 1, n, h->mb, h->mx, tol, info, s, A, P);
     if (st == MG_OK || st == MG_ERR_NOT_CONVERGED || st == MG_ERR_BREAKDOWN) {
         CK(cudaMemcpyAsync(u, h->mx, nu * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -2111,10 +2116,10 @@ mg_status mixed_solve_adjoint(mg_handle* h, const double* g_u, const double* g_p
     // Schur-complement step of A itself (its transpose is S J P J S^-1 as well)
     TRY(mixed_adj_scale<false>(h, g_u, g_p, h->mb, h->mb + nu, s));
     auto A = [&](const double* v, double* y, int j, cudaStream_t q) {
-        TRY(mixed_apply_hat_impl(h, v, v + nu, y, y + nu, q));
-        return gcr_sums(h, n, y, j, q);
+        return dispatch_j<RunMixed<mg::MX_HAT>::K>(j, h, v, y, h->mb, q);
     };
-    auto P = [&](const double* r, double* z, cudaStream_t q) { return schur_impl(h, r, r + nu, z, z + nu, q); };
+    // (mb is free once the iteration has taken its right-hand side: W z_u of the direction under way)
+    auto P = [&](const double* r, double* z, cudaStream_t q) { return schur_impl(h, r, r + nu, z, z + nu, h->mb, q); };
     const mg_status st = gcr(h, 2, n, h->mb, h->mx, tol, info, s, A, P);
     if (st == MG_OK || st == MG_ERR_NOT_CONVERGED || st == MG_ERR_BREAKDOWN) {
         TRY(mixed_adj_scale<true>(h, h->mx, h->mx + nu, lam_u, lam_p, s));
@@ -2148,7 +2153,11 @@ mg_status mixed_apply_transpose(mg_handle* h, const double* u, const double* p, 
     cudaStream_t s = S(stream);
     const size_t nu = (size_t)h->nu;
     TRY(mixed_adj_scale<false>(h, u, p, h->mb, h->mb + nu, s));
-    TRY(mixed_apply_hat_impl(h, h->mb, h->mb + nu, h->mx, h->mx + nu, s));
+    {
+        Prof pr(h, MG_K_MIXED, 0, 8.0 * (3.0 * h->nu + 3.0 * cells(h, 0)), s, 2);
+        // (W times the scaled velocity is u itself)
+        TRY((launch_mixed<mg::MX_HAT, -1>(h, h->mb, h->mb + nu, h->mx, h->mx + nu, const_cast<double*>(u), s)));
+    }
     return mixed_adj_scale<true>(h, h->mx, h->mx + nu, yu, yp, s);
 }
 
@@ -2203,14 +2212,15 @@ mg_status mixed_apply(mg_handle* h, const double* u, const double* p, double* yu
     if (!h || !u || !p || !yu || !yp) return MG_ERR_ARG;
     if (!h->mixed) return MG_ERR_UNSUPPORTED;
     DeviceGuard dg(h->device);
-    return mixed_apply_impl(h, u, p, yu, yp, S(stream));
+    Prof pr(h, MG_K_MIXED, 0, 8.0 * (2.0 * h->nu + 3.0 * cells(h, 0)), S(stream));
+    return launch_mixed<mg::MX_A, -1>(h, u, p, yu, yp, nullptr, S(stream));
 }
 
 mg_status schur_precond(mg_handle* h, const double* ru, const double* rp, double* u, double* p, void* stream) {
     if (!h || !ru || !rp || !u || !p) return MG_ERR_ARG;
     if (!h->mixed) return MG_ERR_UNSUPPORTED;
     DeviceGuard dg(h->device);
-    return schur_impl(h, ru, rp, u, p, S(stream));
+    return schur_impl(h, ru, rp, u, p, nullptr, S(stream));
 }
 
 mg_status mg_autotune(mg_handle* h, int32_t* choices, void* stream) {

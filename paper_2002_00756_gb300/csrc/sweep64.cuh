@@ -351,15 +351,6 @@ __global__ void k_pack64(int n, int ncol, int nlev, const int32_t* __restrict__ 
     if (j == 0) tbs[(size_t)k * 6 * n + p * n + i] = t[__ldg(fof + 3 * ncol + c)] * wt;
 }
 
-// 1 / p: FP32 reciprocal and one cubic step (r = 1 - p y: y + y r + y r^2, relative error r^3 < 2^-66
-// before rounding), 4 FP64 operations instead of a division's dozen; pivots outside FP32's range are
-// divided.
-__device__ __forceinline__ double recip64(double p) {
-    if (!(p > 1e-30 && p < 1e30)) return 1.0 / p;
-    const double y = (double)(1.0f / (float)p), r = fma(-p, y, 1.0);
-    return fma(fma(r, r, r), y, y);
-}
-
 // The factors e, ip of every column; one thread per column.
 __global__ void k_factor64(int n, int ncol, int nlev, const double* __restrict__ te, const double* __restrict__ tn,
                            const double* __restrict__ tbw, const double* __restrict__ tbs,

@@ -85,6 +85,24 @@ def test_recurred_residual_is_the_true_one(mg, n, nlev, levels):
     h.destroy()
 
 
+@pytest.mark.parametrize("n,nlev,levels,rotation", [(10, 19, 1, 0.0), (10, 19, 1, 7.292e-5), (44, 37, 2, 7.292e-5)])
+def test_recurred_mixed_residual_is_the_true_one(mg, n, nlev, levels, rotation):
+    """The fused mixed operator (units of 32 faces or cells by a run of levels) and its sums: the solve's own
+    residual norm is that of b - A x, with ||A|| ~ 2e3 again within 1e-10 of ||b||."""
+    cfg = syn.small_config(n, nlev, levels=levels, seed=syn.BASE_SEED + 780 + n, mixed=True,
+                           consistent_mass=rotation != 0.0, rotation=rotation)
+    inp = syn.make_inputs(cfg)
+    h = mg.mg_setup_config(cfg, inp)
+    b = [torch.from_numpy(inp[k]).cuda().ravel() for k in ("rhs_u", "rhs_p")]
+    x, y = [torch.empty_like(v) for v in b], [torch.empty_like(v) for v in b]
+    for tol in (1e-3, 1e-7):
+        info = mg.mixed_solve(h, *b, *x, tol=tol)
+        mg.mixed_apply(h, *x, *y)
+        true = float(torch.cat([v - w for v, w in zip(b, y)]).norm() / torch.cat(b).norm())
+        assert info.converged and abs(true - info.rel_res) <= 1e-10, (info, true)
+    h.destroy()
+
+
 def test_smoothing_of_misaligned_vectors(mg):
     """Vectors that start on an odd double (8-byte alignment only) give what aligned ones give."""
     cfg = syn.small_config(20, 9, levels=3, seed=syn.BASE_SEED + 720)
