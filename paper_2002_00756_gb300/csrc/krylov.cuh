@@ -35,26 +35,38 @@ __device__ __forceinline__ double warp_sum(double v) {
 // waiting) adds all partials with every thread taking a fixed stride of blocks, then a
 // fixed tree; thread 0 of that block gets the totals in `tot` and the function returns
 // true there.  The order of every addition is fixed, so results are bitwise repeatable.
+//
+// An FP64 instruction of a warp takes the SM's pipe 16 cycles whatever its lanes do, so a block's
+// threads meet in shared memory and one warp per sum adds 8 values a lane before its tree: 12
+// instructions per block and sum, where a shuffle tree in each warp takes 40 and more.  With event
+// overhead (about 4 us), C48L30: orthogonalisation 14.4 -> 12.3 us, fused apply 20.5 .. 30.8 -> 18.4 .. 24.6;
+// C12L30: 12.3 -> 8.2 and 10.2 .. 14.4 -> 10.2 .. 12.3.
 template <int ND>
-__device__ bool grid_reduce(double (&v)[ND], double* partials, unsigned int* ticket, double (&tot)[ND]) {
-    __shared__ double sm[ND][RED_THREADS / 32];
-    __shared__ bool last;
+__device__ __forceinline__ void block_sums(const double (&v)[ND], double (*sm)[RED_THREADS], double* to, size_t stride) {
+    constexpr int W = RED_THREADS / 32;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < ND; ++i) sm[i][threadIdx.x] = v[i];
+    __syncthreads();
+    for (int i = wid; i < ND; i += W) {
+        double s = sm[i][lane];
+#pragma unroll
+        for (int w = 1; w < W; ++w) s += sm[i][w * 32 + lane];
+        s = warp_sum(s);
+        if (lane == 0) {
+            to[i * stride] = s;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+}
+
+template <int ND>
+__device__ bool grid_reduce(const double (&v)[ND], double* partials, unsigned int* ticket, double (&tot)[ND]) {
+    __shared__ double sm[ND][RED_THREADS], total[ND];
+    __shared__ bool last;
     const unsigned nblk = gridDim.x * gridDim.y, bid = blockIdx.y * gridDim.x + blockIdx.x;
-#pragma unroll
-    for (int i = 0; i < ND; ++i) v[i] = warp_sum(v[i]);
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < ND; ++i) sm[i][wid] = v[i];
-    }
-    __syncthreads();
-    if (threadIdx.x < ND) {
-        double s = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) s += sm[threadIdx.x][w];
-        partials[(size_t)bid * ND + threadIdx.x] = s;
-    }
-    __threadfence();
-    __syncthreads();
+    block_sums<ND>(v, sm, partials + bid, nblk);
     if (threadIdx.x == 0) last = (atomicAdd(ticket, 1u) == nblk - 1);
     __syncthreads();
     if (!last) return false;
@@ -64,23 +76,12 @@ __device__ bool grid_reduce(double (&v)[ND], double* partials, unsigned int* tic
     for (int i = 0; i < ND; ++i) a[i] = 0.0;
     for (unsigned b = threadIdx.x; b < nblk; b += RED_THREADS) {
 #pragma unroll
-        for (int i = 0; i < ND; ++i) a[i] += __ldcg(partials + (size_t)b * ND + i);
+        for (int i = 0; i < ND; ++i) a[i] += __ldcg(partials + (size_t)i * nblk + b);
     }
-#pragma unroll
-    for (int i = 0; i < ND; ++i) a[i] = warp_sum(a[i]);
-    __syncthreads();
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < ND; ++i) sm[i][wid] = a[i];
-    }
-    __syncthreads();
+    block_sums<ND>(a, sm, total, 1);
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int i = 0; i < ND; ++i) {
-            double s = 0.0;
-            for (int w = 0; w < RED_THREADS / 32; ++w) s += sm[i][w];
-            tot[i] = s;
-        }
+        for (int i = 0; i < ND; ++i) tot[i] = total[i];
         *ticket = 0u;
     }
     return threadIdx.x == 0;
@@ -433,11 +434,11 @@ __global__ void __launch_bounds__(RED_THREADS) k_gcr_orth_update(size_t n, doubl
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         double we = w[e];
 #pragma unroll
-        for (int i = 0; i < J; ++i) we -= beta[i] * __ldg(Wb + (size_t)i * ld + e);
+        for (int i = 0; i < J; ++i) we = fma(-beta[i], __ldg(Wb + (size_t)i * ld + e), we);
         if (J > 0) w[e] = we;
-        const double re = r[e] - a * we;
+        const double re = fma(-a, we, r[e]);
         r[e] = re;
-        v[0] += re * re;
+        v[0] = fma(re, re, v[0]);
     }
     if (grid_reduce<1>(v, partials, ticket, t)) S->rr = t[0];
 }
@@ -567,8 +568,8 @@ __global__ void k_mx_grad_beta(MixedDev M, const double* __restrict__ lam_v, con
 // The units of work, 32 columns x kchunk levels, are dealt out over a grid that is resident at once,
 // and a warp keeps its sums over all its units: one reduction per warp (it runs on the FP64 pipe as
 // well) instead of one per 24 levels, and no last wave of blocks on a part of the chip.  At C192L70
-// 254 / 281 / 307 / 336 / 365 us for J = 0..4 (one unit per thread, blocks in waves: 280 / 314 / 343 / 381
-// / 417; the FP64 pipe's bound: 223 / 248 / 273 / 298 / 322); C48L30 20-33 us instead of 35-49.  Two, four
+// 252 / 276 / 305 / 330 / 356 us for J = 0..4 (one unit per thread, blocks in waves: 280 / 314 / 343 / 381
+// / 417; the FP64 pipe's bound: 223 / 248 / 273 / 298 / 322); C48L30 18-25 us instead of 35-49.  Two, four
 // and five blocks per SM: 256-369, 256-385, 258-391.
 constexpr int APPLY_BLOCKS = 3;   // resident blocks per SM
 
@@ -670,7 +671,7 @@ __global__ void __launch_bounds__(RED_THREADS, mixed_blocks(MODE)) k_mixed(
     for (unsigned q = blockIdx.x * (RED_THREADS / 32) + (threadIdx.x >> 5); q < G * nchunk; q += nwarp) {
         const unsigned ch = q / G, g = q - ch * G;
         const int k0 = ch * kchunk, k1 = min(M.nlev, k0 + kchunk);
-        if (g < gh) {   // horizontal faces
+        if (MODE != MX_RHS && g < gh) {   // horizontal faces
             const unsigned f = g * 32 + lane;
             if (f >= nfh) continue;
             const unsigned fl = __ldg(M.faceL + f), fr = __ldg(M.faceR + f);

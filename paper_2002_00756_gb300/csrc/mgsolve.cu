@@ -340,6 +340,14 @@ mg_status launch_apply(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, Y*
 //   up to 40 levels, 700k: C64L30 81/47 and 80/42 (C56L30, 564k: 71 and 78; C48L37 77/34 and 81/36).
 inline bool tma_level(int nlev, int ncol) { return (double)nlev * ncol >= (nlev > 40 ? 2.5e5 : 7e5); }
 
+// Grid of a vector pass with or without a reduction: two elements per thread until the GPU is full (C12L30's
+// <b, b>: 8.8 us; one per thread 10.6; C192L70's orthogonalisations 121 us on average, with 6, 16 or 32 blocks
+// per SM instead of 8: 131, 124, 129).
+inline int vec_grid(const mg_handle* h, size_t n) {
+    constexpr size_t per_block = 2 * mg::RED_THREADS;
+    return (int)std::max<size_t>(1, std::min<size_t>(h->red_grid, (n + per_block - 1) / per_block));
+}
+
 inline bool aligned(const void* p, size_t bytes) { return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) == 0; }
 
 inline int sweep_mode(const void* x, const void* xc) {
@@ -712,7 +720,7 @@ mg_status bicgstab(mg_handle* h, const double* b, double* x, double tol, int max
     if (!rh) return MG_ERR_UNSUPPORTED;
     const Lvl<double, double> L = View<double, double>::lvl(h, 0);
     const dim3 ag((L.ncol + 127) / 128, L.nlev);
-    const int G = h->red_grid, B = mg::RED_THREADS;
+    const int G = vec_grid(h, cells(h, 0)), B = mg::RED_THREADS;
     unsigned int* tk = h->tickets + TK_BICG;
     auto apply = [&](const double* in, double* out) -> mg_status {
         if (h->nine) return launch_apply9(h, 0, in, out, s);
@@ -813,7 +821,7 @@ template <int J>
 struct RunSums {
     static mg_status run(mg_handle* h, size_t n, const double* w, cudaStream_t s) {
         Prof pr(h, MG_K_GCR_DOTS, 0, 8.0 * n * (J + 2), s);   // w, r, w_i
-        mg::k_gcr_sums<J><<<h->red_grid, mg::RED_THREADS, 0, s>>>(n, w, h->W, h->glen, h->r, h->partials,
+        mg::k_gcr_sums<J><<<vec_grid(h, n), mg::RED_THREADS, 0, s>>>(n, w, h->W, h->glen, h->r, h->partials,
                                                                    h->tickets + TK_SUMS, h->gs);
         CK(cudaGetLastError());
         return MG_OK;
@@ -842,7 +850,7 @@ template <int J>
 struct RunOrth {
     static mg_status run(mg_handle* h, size_t n, cudaStream_t s) {
         Prof pr(h, MG_K_GCR_ORTH, 0, 8.0 * n * (J > 0 ? J + 4 : 3), s);
-        mg::k_gcr_orth_update<J><<<h->red_grid, mg::RED_THREADS, 0, s>>>(n, h->W, h->glen, h->r, h->partials,
+        mg::k_gcr_orth_update<J><<<vec_grid(h, n), mg::RED_THREADS, 0, s>>>(n, h->W, h->glen, h->r, h->partials,
                                                                          h->tickets + TK_ORTH, h->gs);
         CK(cudaGetLastError());
         return MG_OK;
@@ -853,7 +861,7 @@ template <int J>
 struct RunXupd {
     static mg_status run(mg_handle* h, size_t n, double* x, cudaStream_t s) {
         Prof pr(h, MG_K_GCR_UPDATE, 0, 8.0 * n * (J + 3), s);
-        mg::k_gcr_xupdate<J><<<h->red_grid, mg::RED_THREADS, 0, s>>>(n, x, h->Z, h->glen, h->gs);
+        mg::k_gcr_xupdate<J><<<vec_grid(h, n), mg::RED_THREADS, 0, s>>>(n, x, h->Z, h->glen, h->gs);
         CK(cudaGetLastError());
         return MG_OK;
     }
@@ -911,7 +919,7 @@ mg_status gcr_start(mg_handle* h, GcrRun& g, const double* b, cudaStream_t s) {
     CK(cudaMemsetAsync(g.x, 0, g.n * sizeof(double), s));
     {
         Prof pr(h, MG_K_DOT, 0, 8.0 * g.n, s);
-        mg::k_dot<<<h->red_grid, mg::RED_THREADS, 0, s>>>(g.n, b, b, h->partials, h->tickets + TK_DOT, &h->gs->bb);
+        mg::k_dot<<<vec_grid(h, g.n), mg::RED_THREADS, 0, s>>>(g.n, b, b, h->partials, h->tickets + TK_DOT, &h->gs->bb);
         CK(cudaGetLastError());
     }
     CK(cudaMemcpyAsync(h->host_sc, &h->gs->bb, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1651,7 +1659,7 @@ mg_status build_member(mg_ensemble* e, int i, mg_handle* h, const double* b, dou
     CK(cudaStreamBeginCaptureToGraph(e->cs, e->graph, root.data(), nullptr, root.size(), mode));
     CK(cudaMemcpyAsync(h->r, b, n * sizeof(double), cudaMemcpyDeviceToDevice, e->cs));
     CK(cudaMemsetAsync(x, 0, n * sizeof(double), e->cs));
-    mg::k_dot<<<h->red_grid, mg::RED_THREADS, 0, e->cs>>>(n, b, b, h->partials, h->tickets + TK_DOT, &h->gs->bb);
+    mg::k_dot<<<vec_grid(h, n), mg::RED_THREADS, 0, e->cs>>>(n, b, b, h->partials, h->tickets + TK_DOT, &h->gs->bb);
     mg::k_ens_init<<<1, 1, 0, e->cs>>>(h->gs, st, R, h->prm.max_iter, hs);
     CK(cudaGetLastError());
     TRY(end_segment(e, deps));
