@@ -355,12 +355,13 @@ inline int sweep_mode(const void* x, const void* xc) {
 }
 
 // levels per thread of the residual + restriction: long chunks (fewer prologues) where the level
-// fills the GPU several times over; the small levels need every thread (one level per thread at C48L30:
-// 6.5 us a launch against 13 with eight)
+// fills the GPU several times over (C192L70 60 us with 35, 62 with 8, events included; C96L70 21 with 2 or
+// 6, 22 with 12); the small levels need every thread (one level per thread at C48L30: 6.5 us a launch
+// against 13 with eight)
 inline int restrict_chunk(const mg_handle* h, int lev) {
     const DevLevel& d = h->lv[lev];
     if (d.restrict_kc > 0) return d.restrict_kc;
-    return d.ncol >= 100000 ? 24 : (double)h->nlev * d.ncol >= 2e6 ? 2 : 1;
+    return d.ncol >= 100000 ? 35 : (double)h->nlev * d.ncol >= 2e6 ? 2 : 1;
 }
 
 // One FP64 block-Jacobi sweep on level `lev`.  The iterate it starts from is x (NULL: zero) plus,

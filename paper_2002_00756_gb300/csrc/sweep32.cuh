@@ -336,7 +336,9 @@ __global__ void k_fill_rims(int n, int ncol, const int32_t* __restrict__ hd, T* 
 // Residual and restriction (Algorithm 1): bc[k][C] = sum_q w_q (b - H x)[k][child_q],
 // w = area_child / area_C.  One thread per coarse column (2 x 2 fine columns, whose rows are read 2
 // wide) and kchunk levels.  TREE: the children are summed in pairs (levels of n % 16 == 0), else
-// one after the other.
+// one after the other.  The loads in flight bound it: the loop stays rolled (two levels at a
+// time need more registers, fewer blocks fit: C192L70 72 us instead of 56, C96L70 21 instead of 17; three
+// couplings, x, b and the result at copy speed: 46 and 12).
 template <typename C, bool XZERO, bool TREE>
 __global__ void __launch_bounds__(128) k_restrict32(Lvl32<C, float> L, const float* __restrict__ x,
                                                     const float* __restrict__ b, const float* __restrict__ wq,
@@ -380,7 +382,7 @@ __global__ void __launch_bounds__(128) k_restrict32(Lvl32<C, float> L, const flo
             ld2(L.tv + (k0 * lx + cx[r]), tb[r]);
         }
     }
-#pragma unroll 2
+#pragma unroll 1
     for (int k = k0; k < k1; ++k) {
         const unsigned o = (unsigned)k * lx;
         float r_[2][2];
