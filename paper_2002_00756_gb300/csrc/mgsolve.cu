@@ -1380,13 +1380,8 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
                 if (l == 0 && prm->vcycle_precision == MG_FP32_P64)
                     for (double** p : {&d.ipd, &d.md, &d.ed}) TRY(dalloc(h, p, Np));
                 TRY(dalloc(h, &d.hd, 4 * (size_t)G.ncol));
-                k_rims<<<dim3((G.ncol + 127) / 128, 4), 128>>>(G.n, G.ncol, d.nbr, d.hd);
             }
-            if (l + 1 < L) {
-                TRY(dalloc(h, &d.par, 5 * (size_t)G.ncol));
-                k_parents<<<dim3((G.ncol + 127) / 128, 5), 128>>>(G.n, G.ncol, d.nbr, d.par);
-            }
-            TRY(pack_level(h, l, nullptr));
+            if (l + 1 < L) TRY(dalloc(h, &d.par, 5 * (size_t)G.ncol));
         }
         TRY(dalloc(h, &d.x64[0], Nl));
         TRY(dalloc(h, &d.x64[1], Nl));
@@ -1541,6 +1536,13 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
         TRY(dalloc(h, &h->schurB, N0));
         TRY(dalloc(h, &h->mb, (size_t)h->nu + N0));
         TRY(dalloc(h, &h->mx, (size_t)h->nu + N0));
+    }
+    // the levels' packed fields and factors: after the uploads, which would wait for them
+    for (int l = 0; l < L && gamma2 <= 0.0; ++l) {
+        DevLevel& d = h->lv[l];
+        if (d.hd) k_rims<<<dim3((d.ncol + 127) / 128, 4), 128>>>(d.n, d.ncol, d.nbr, d.hd);
+        if (d.par) k_parents<<<dim3((d.ncol + 127) / 128, 5), 128>>>(d.n, d.ncol, d.nbr, d.par);
+        TRY(pack_level(h, l, nullptr));
     }
     // GCR workspace; the slot stride is padded off a multiple of large powers of two so
     // the directions streamed side by side do not share their low address bits
