@@ -42,7 +42,7 @@ struct DevLevel {
     int32_t* par = nullptr;      // [5][ncol] coarse parents of the neighbours and of the column
     // FP64 level data (sweep64.cuh; also mg_smooth and mg_residual_restrict)
     double *te64 = nullptr, *tn64 = nullptr, *tbw64 = nullptr, *tbs64 = nullptr, *tv64 = nullptr;
-    double *e64 = nullptr, *ip64 = nullptr;
+    double *e64 = nullptr, *ip64 = nullptr, *pr64 = nullptr;
     double* wA64 = nullptr;      // area x scale
     // FP32 level data (sweep32.cuh): couplings in FP32 or BF16, reciprocal pivots, 1 / area; the
     // FP64 elimination of MG_FP32_P64's finest level; restriction weights onto the next level
@@ -86,6 +86,7 @@ struct mg_handle {
     std::vector<DevLevel> lv;
     double* rdz64 = nullptr;
     float* rdz32 = nullptr;
+    double om0 = 1.0;           // relaxation factor folded into the FP64 factors: prm.omega unless 0
     double scale = 1.0;         // power of two in the FP64 volume weights, 1 / (largest finest area x depth)
     double* a6 = nullptr;       // finest level: six premultiplied FP64 couplings and 1 + their sum, per cell
     bool nine = false;          // 9-cell stencil (mg_setup_9pt)
@@ -291,7 +292,8 @@ struct View<float, float> {
 
 Lvl64 lvl64(const mg_handle* h, int l) {
     const DevLevel& d = h->lv[l];
-    return {d.n, d.ncol, h->nlev, d.nbr, d.par, d.te64, d.tn64, d.tbw64, d.tbs64, d.tv64, d.e64, d.ip64, d.wA64, h->dz};
+    return {d.n, d.ncol, h->nlev, d.nbr, d.par, d.te64, d.tn64, d.tbw64, d.tbs64, d.tv64, d.e64, d.ip64, d.pr64,
+            d.wA64, h->dz, h->om0};
 }
 
 template <typename C, typename P>
@@ -387,9 +389,11 @@ mg_status launch_sweep64(mg_handle* h, int lev, const Lvl64& L, const double* x,
                                                          (xc ? 0.25 : 0.0) + (bcopy ? 1 : 0)), s, mode);
     auto shape = [&](auto r, auto c) -> cudaError_t {
         constexpr bool R = decltype(r)::value, B = decltype(c)::value;
-        if (L.nlev > 80) return sweep64_go<R, B, 16>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
-        if ((double)L.nlev * L.ncol < 2e6) return sweep64_go<R, B, 5>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
-        return sweep64_go<R, B, 10>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
+        switch (mg::sweep64_levels(L.nlev, L.ncol)) {
+            case 16: return sweep64_go<R, B, 16>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
+            case 5: return sweep64_go<R, B, 5>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
+            default: return sweep64_go<R, B, 10>(L, mode, x, xc, ncol_c, b, bcopy, xo, om, s);
+        }
     };
     if (raw && bcopy) CK(shape(std::true_type(), std::true_type()));
     else if (raw) CK(shape(std::true_type(), std::false_type()));
@@ -1152,7 +1156,8 @@ mg_status pack_level(mg_handle* h, int l, cudaStream_t s) {
     mg::k_pack64<<<grid, 128, 0, s>>>(d.n, d.ncol, h->nlev, d.fof, d.Th64, d.Tv64, d.wA64, h->dz, h->scale, d.te64, d.tn64,
                                       d.tbw64, d.tbs64, d.tv64);
     mg::k_factor64<<<(d.ncol + 63) / 64, 64, 0, s>>>(d.n, d.ncol, h->nlev, d.te64, d.tn64, d.tbw64, d.tbs64, d.tv64,
-                                                     d.wA64, h->dz, d.e64, d.ip64);
+                                                     d.wA64, h->dz, d.e64, d.ip64, d.pr64,
+                                                     mg::sweep64_chunks(h->nlev, d.ncol), h->om0);
     const dim3 halves((d.ncol + 63) / 64, 2);
     if (d.te32) {
         mg::k_pack32<float><<<grid, 128, 0, s>>>(d.n, d.ncol, h->nlev, d.fof, d.Th64, d.Tv64, d.te32, d.tn32, d.tv32);
@@ -1270,6 +1275,7 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
     h->n = n;
     h->nlev = nlev;
     h->prm = *prm;
+    if (prm->omega != 0.0) h->om0 = prm->omega;
     CK(cudaGetDevice(&h->device));
     CK(cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->device));
     h->red_grid = 8 * h->nsm;
@@ -1368,6 +1374,8 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
             for (double** p : {&d.te64, &d.tn64, &d.e64, &d.ip64}) TRY(dalloc(h, p, Nl));
             for (double** p : {&d.tbw64, &d.tbs64}) TRY(dalloc(h, p, (size_t)nlev * 6 * G.n));
             TRY(dalloc(h, &d.tv64, Nl + G.ncol));
+            if (mg::sweep64_levels(nlev, G.ncol) == 10)
+                TRY(dalloc(h, &d.pr64, (size_t)mg::sweep64_chunks(nlev, G.ncol) * G.ncol));
             if (prec == MG_FP32) {
                 for (float** p : {&d.te32, &d.tn32}) TRY(dalloc(h, p, Np));
                 TRY(dalloc(h, &d.tv32, Np + mg::padded(G.n)));
@@ -1385,13 +1393,15 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
         }
         TRY(dalloc(h, &d.x64[0], Nl));
         TRY(dalloc(h, &d.x64[1], Nl));
-        TRY(dalloc(h, &d.b64, Nl));
-        TRY(dalloc(h, &d.r64, Nl));
-        if (prec != MG_FP64) {
+        // right-hand sides and, below the finest level, the iterate that goes up
+        if (prec == MG_FP64) {
+            TRY(dalloc(h, &d.b64, Nl));
+            if (l > 0) TRY(dalloc(h, &d.r64, Nl));
+        } else {
             TRY(dalloc(h, &d.x32[0], Np));
             TRY(dalloc(h, &d.x32[1], Np));
             TRY(dalloc(h, &d.b32, Np));
-            TRY(dalloc(h, &d.r32, Np));
+            if (l > 0) TRY(dalloc(h, &d.r32, Np));
         }
         if (gamma2 > 0.0) {
             // 9-cell stencil: flux between cells k and k + 2 of every column,

@@ -27,10 +27,12 @@ struct Lvl64 {
     const double* tbw;    // [nlev][6 n] west face of each panel's first column, by (panel, j)
     const double* tbs;    // [nlev][6 n] south face of each panel's first row, by (panel, i)
     const double* tv;     // [nlev + 1][ncol] vertical faces, rows 0 and nlev zero
-    const double* e;      // [nlev][ncol] factors
+    const double* e;      // [nlev][ncol] factors; ip times om0
     const double* ip;
+    const double* pr;     // [chunks][ncol] product of e over each chunk of 10 levels, where sweeps use those
     const double* wA;     // [ncol] area x scale
     const double* dz;     // [nlev] layer depth
+    double om0;           // relaxation factor that ip holds
 };
 
 // v = *p where `on`, else v unchanged: a predicated load, not a branch.  A branch around the few
@@ -39,6 +41,14 @@ struct Lvl64 {
 // this form: 97 us instead of 122).
 __device__ __forceinline__ void ldp(double& v, const double* p, bool on) {
     asm("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.nc.f64 %0, [%1];\n}" : "+d"(v) : "l"(p), "r"((int)on));
+}
+
+// Levels per chunk: 10, where two blocks fit on an SM, 5 below 2M cells (twice the threads), 16 for
+// columns of more than 80 levels; and the chunks of a column, W.
+inline int sweep64_levels(int nlev, int ncol) { return nlev > 80 ? 16 : (double)nlev * ncol < 2e6 ? 5 : 10; }
+inline int sweep64_chunks(int nlev, int ncol) {
+    const int K = sweep64_levels(nlev, ncol);
+    return (nlev + K - 1) / K;
 }
 
 __host__ __device__ constexpr int sweep64_warps(int K) { return ((K < 16 ? 80 : 128) + K - 1) / K; }
@@ -51,9 +61,12 @@ __host__ __device__ constexpr int sweep64_warps(int K) { return ((K < 16 ? 80 : 
 //
 // W warps share 32 consecutive columns; warp w owns the levels [w nlev / W, (w + 1) nlev / W), at
 // most K, and holds them in registers.  The two recurrences run per chunk from a zero inflow, the
-// chunks' (outflow, product of e) pairs are exchanged through shared memory and folded in order by
-// every warp, and a second pass applies the true inflow.  (Chunks of 10, two columns per lane: 114 us
-// for the finest plain sweep at C96L70; this shape 125, but 5 and 7 levels per chunk 162.)
+// chunks' (outflow, product of e) pairs are folded in order by every warp, outflows exchanged through
+// shared memory, and a second pass applies the true inflow.  The FP64 pipe bounds it: chunks of 10 read
+// their products, and ip holds omega already (10.9 operations per cell of a plain sweep, 7.9 of a first one
+// instead of 12.9 and 9.9): plain 121 -> 104 us at C96L70, first 84 -> 74, with the prolongation 160 -> 156.
+// Chunks of 5 (small levels) multiply their products up: reading 16 of them costs more latency than the
+// operations saved (C12L30 solve 364 us against 347).
 //
 // BRAW: b is unweighted and weighted here (and, with BCOPY, stored for the later sweeps of the level).
 template <int MODE, bool BRAW, bool BCOPY, int K>
@@ -64,7 +77,8 @@ __global__ void __launch_bounds__(32 * sweep64_warps(K), K == 10 ? 2 : 1)
     constexpr bool RAW = (MODE == XM_PLAIN || MODE == XM_PROLONG);   // reads the fine iterate
     constexpr bool ZERO = MODE == XM_ZERO;
     constexpr int WMAX = sweep64_warps(K);
-    __shared__ double s_[3][WMAX][32];   // outflow upwards, product of e, outflow downwards
+    constexpr bool STORED = K == 10;   // the chunks' products of e are read, not multiplied up
+    __shared__ double s_[STORED ? 2 : 3][WMAX][32];   // outflow upwards, downwards, product of e
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
     const unsigned ncol = L.ncol, n = L.n;
     const unsigned c_raw = blockIdx.x * 32 + lane;
@@ -151,22 +165,27 @@ __global__ void __launch_bounds__(32 * sweep64_warps(K), K == 10 ? 2 : 1)
         }
     }
     // forwards: outflow e y of the chunk from zero inflow, fold, then y with the true inflow
-    double pr[WMAX];   // every chunk's product, read once for both directions
+    double pr[WMAX];   // every chunk's product of e, for both directions
     if (W > 1) {
+        if constexpr (STORED) {
+#pragma unroll
+            for (int u = 0; u < WMAX; ++u)
+                if (u < W) pr[u] = __ldg(L.pr + ((unsigned)u * ncol + c));
+        }
         double y = f[0], g = e[0];
 #pragma unroll
         for (int q = 1; q < K; ++q) {
             y = fma(e[q - 1], y, f[q]);
-            g *= e[q];
+            if (!STORED) g *= e[q];
         }
         s_[0][w][lane] = e[K - 1] * y;
-        s_[1][w][lane] = g;
+        if constexpr (!STORED) s_[2][w][lane] = g;
         __syncthreads();
         double in = 0.0;
 #pragma unroll
         for (int u = 0; u < WMAX; ++u)
             if (u < W) {
-                pr[u] = s_[1][u][lane];
+                if constexpr (!STORED) pr[u] = s_[2][u][lane];
                 if (u < w) in = fma(pr[u], in, s_[0][u][lane]);
             }
         f[0] += in;
@@ -175,24 +194,29 @@ __global__ void __launch_bounds__(32 * sweep64_warps(K), K == 10 ? 2 : 1)
     for (int q = 1; q < K; ++q) f[q] = fma(e[q - 1], f[q - 1], f[q]);
 #pragma unroll
     for (int q = 0; q < K; ++q) f[q] *= ip[q];
-    // backwards: the chunk's lowest value from zero inflow, fold, then d and the update
+    if (omega != L.om0) {   // (a pressure solver with a relaxation factor of its own)
+        const double scale = omega / L.om0;
+#pragma unroll
+        for (int q = 0; q < K; ++q) f[q] *= scale;
+    }
+    // backwards: the chunk's lowest value from zero inflow, fold, then d (times omega) and the update
     double d = 0.0;
     if (W > 1) {
         double g = f[K - 1];
 #pragma unroll
         for (int q = K - 2; q >= 0; --q) g = fma(e[q], g, f[q]);
-        s_[2][w][lane] = g;
+        s_[1][w][lane] = g;
         __syncthreads();
 #pragma unroll
         for (int u = WMAX - 1; u >= 0; --u)
-            if (u > w && u < W) d = fma(pr[u], d, s_[2][u][lane]);
+            if (u > w && u < W) d = fma(pr[u], d, s_[1][u][lane]);
     }
     const double om1 = 1.0 - omega;
 #pragma unroll
     for (int q = K - 1; q >= 0; --q) {
         d = fma(e[q], d, f[q]);
         if (active && k0 + q < k1)
-            xo[(unsigned)(k0 + q) * ncol + c] = ZERO ? omega * d : fma(om1, x0[q], omega * d);
+            xo[(unsigned)(k0 + q) * ncol + c] = ZERO ? d : fma(om1, x0[q], d);
     }
 }
 
@@ -355,7 +379,8 @@ __global__ void k_pack64(int n, int ncol, int nlev, const int32_t* __restrict__ 
 __global__ void k_factor64(int n, int ncol, int nlev, const double* __restrict__ te, const double* __restrict__ tn,
                            const double* __restrict__ tbw, const double* __restrict__ tbs,
                            const double* __restrict__ tv, const double* __restrict__ wA, const double* __restrict__ dz,
-                           double* __restrict__ e_, double* __restrict__ ip_) {
+                           double* __restrict__ e_, double* __restrict__ ip_, double* __restrict__ pr, int chunks,
+                           double om0) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncol) return;
     const int row = c / n, i = c - row * n, p = row / n, j = row - p * n;
@@ -363,7 +388,8 @@ __global__ void k_factor64(int n, int ncol, int nlev, const double* __restrict__
     const double* pts = j > 0 ? tn + c - n : tbs + p * n + i;
     const size_t sW = i > 0 ? ncol : 6 * n, sS = j > 0 ? ncol : 6 * n;
     const double a = wA[c];
-    double Q = 0.0, e = 0.0;
+    double Q = 0.0, e = 0.0, g = 1.0;
+    int w = 0;
 #pragma unroll 4
     for (int k = 0; k < nlev; ++k) {
         const size_t o = (size_t)k * ncol + c;
@@ -373,7 +399,12 @@ __global__ void k_factor64(int n, int ncol, int nlev, const double* __restrict__
         const double ip = recip64(Q + t);
         e = t * ip;
         e_[o] = e;
-        ip_[o] = ip;
+        ip_[o] = om0 * ip;
+        g *= e;
+        if (pr && k + 1 == (w + 1) * nlev / chunks) {
+            pr[(size_t)w++ * ncol + c] = g;
+            g = 1.0;
+        }
     }
 }
 
