@@ -169,14 +169,19 @@ __global__ void k_coef_grad(Lvl<double, double> L, const double* __restrict__ la
     grad[5 * N + e] = k > 0 ? -l * (x0 - x[e - ncol]) : 0.0;
 }
 
-// out = <a, b>
-__global__ void __launch_bounds__(RED_THREADS) k_dot(size_t n, const double* __restrict__ a,
-                                                     const double* __restrict__ b, double* partials,
-                                                     unsigned int* ticket, double* out) {
+// Start of a GCR solve: r = b, x = 0, <b, b>, in one pass over memory (a copy, a fill and a product before: C192L70
+// solve 10.50 -> 10.45 ms, together with the first iteration launched ahead).
+__global__ void __launch_bounds__(RED_THREADS) k_gcr_start(size_t n, const double* __restrict__ b, double* __restrict__ r,
+                                                           double* __restrict__ x, double* partials,
+                                                           unsigned int* ticket, double* bb) {
     double v[1] = {0.0}, t[1];
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        v[0] += a[i] * b[i];
-    if (grid_reduce<1>(v, partials, ticket, t)) *out = t[0];
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const double e = __ldg(b + i);
+        r[i] = e;
+        x[i] = 0.0;
+        v[0] = fma(e, e, v[0]);
+    }
+    if (grid_reduce<1>(v, partials, ticket, t)) *bb = t[0];
 }
 
 // ---- BiCGStab for the pressure system (van der Vorst 1992, right-preconditioned) ----

@@ -116,7 +116,7 @@ struct mg_handle {
     double* partials = nullptr;
     size_t npartials = 0;
     unsigned int* tickets = nullptr;
-    double* host_sc = nullptr;  // pinned
+    double* host_sc = nullptr;  // pinned: <r, r>, <b, b>
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     // one CUDA graph per GCR slot j and system (0 pressure, 1 mixed, 2 the mixed adjoint's
     // A-hat): the V-cycle, the
@@ -920,19 +920,18 @@ struct GcrRun {
 
 mg_status gcr_start(mg_handle* h, GcrRun& g, const double* b, cudaStream_t s) {
     CK(cudaEventRecord(h->ev0, s));
-    CK(cudaMemcpyAsync(h->r, b, g.n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemsetAsync(g.x, 0, g.n * sizeof(double), s));
     {
-        Prof pr(h, MG_K_DOT, 0, 8.0 * g.n, s);
-        mg::k_dot<<<vec_grid(h, g.n), mg::RED_THREADS, 0, s>>>(g.n, b, b, h->partials, h->tickets + TK_DOT, &h->gs->bb);
+        Prof pr(h, MG_K_DOT, 0, 24.0 * g.n, s);
+        mg::k_gcr_start<<<vec_grid(h, g.n), mg::RED_THREADS, 0, s>>>(g.n, b, h->r, g.x, h->partials, h->tickets + TK_DOT,
+                                                                    &h->gs->bb);
         CK(cudaGetLastError());
     }
-    CK(cudaMemcpyAsync(h->host_sc, &h->gs->bb, sizeof(double), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(h->host_sc + 1, &h->gs->bb, sizeof(double), cudaMemcpyDeviceToHost, s));
     return MG_OK;
 }
 
 void gcr_started(mg_handle* h, GcrRun& g) {
-    g.bb = h->host_sc[0];
+    g.bb = h->host_sc[1];
     g.it = 0;
     g.rel = 0.0;
     g.active = false;
@@ -1008,12 +1007,20 @@ mg_status gcr(mg_handle* h, int sys, size_t n, const double* b, double* x, doubl
     g.x = x;
     g.tol = tol;
     TRY(gcr_start(h, g, b, s));
+    // The first iteration follows without waiting for <b, b>, which only a zero, infinite or NaN right-hand
+    // side needs first: x stays 0 then and the iteration's outcome is dropped (one host round trip less per
+    // solve: C12L30 350 -> 337 us, C48L30 720 -> 704).  A pressure solver that synchronises could fail on such a right-hand side.
+    bool ahead = h->prm.max_iter > 0 && !(sys != 0 && ps_syncs(h));
+    if (ahead) TRY(gcr_launch(h, g, s, applyAS, applyP));
     CK(cudaStreamSynchronize(s));
     gcr_started(h, g);
     while (g.active) {
         NvtxRange it_("gcr iteration");
-        TRY(gcr_launch(h, g, s, applyAS, applyP));
-        CK(cudaStreamSynchronize(s));
+        if (!ahead) {
+            TRY(gcr_launch(h, g, s, applyAS, applyP));
+            CK(cudaStreamSynchronize(s));
+        }
+        ahead = false;
         TRY(gcr_landed(h, g, s));
     }
     CK(cudaEventRecord(h->ev1, s));
@@ -1670,9 +1677,8 @@ mg_status build_member(mg_ensemble* e, int i, mg_handle* h, const double* b, dou
     // start: r = b, x = 0, <b, b>, first decision
     std::vector<cudaGraphNode_t> deps;
     CK(cudaStreamBeginCaptureToGraph(e->cs, e->graph, root.data(), nullptr, root.size(), mode));
-    CK(cudaMemcpyAsync(h->r, b, n * sizeof(double), cudaMemcpyDeviceToDevice, e->cs));
-    CK(cudaMemsetAsync(x, 0, n * sizeof(double), e->cs));
-    mg::k_dot<<<vec_grid(h, n), mg::RED_THREADS, 0, e->cs>>>(n, b, b, h->partials, h->tickets + TK_DOT, &h->gs->bb);
+    mg::k_gcr_start<<<vec_grid(h, n), mg::RED_THREADS, 0, e->cs>>>(n, b, h->r, x, h->partials, h->tickets + TK_DOT,
+                                                                   &h->gs->bb);
     mg::k_ens_init<<<1, 1, 0, e->cs>>>(h->gs, st, R, h->prm.max_iter, hs);
     CK(cudaGetLastError());
     TRY(end_segment(e, deps));

@@ -103,6 +103,26 @@ def test_recurred_mixed_residual_is_the_true_one(mg, n, nlev, levels, rotation):
     h.destroy()
 
 
+def test_degenerate_right_hand_sides_leave_no_trace(mg):
+    """A solve launches its first iteration before it knows <b, b>: a zero right-hand side still converges
+    at once with x = 0, a NaN still breaks down, and the next solve gives the bits of the first."""
+    cfg = syn.small_config(10, 19, levels=2, seed=syn.BASE_SEED + 790)
+    inp = syn.make_inputs(cfg)
+    h = mg.mg_setup_config(cfg, inp)
+    b = torch.from_numpy(inp["rhs"]).cuda().ravel()
+    ref, x = torch.empty_like(b), torch.empty_like(b)
+    first = mg.pressure_solve(h, b, ref, 1e-9)
+    assert first.converged
+    for bad in (torch.zeros_like(b), torch.where(torch.arange(b.numel(), device="cuda") == 5, float("nan"), b)):
+        x.fill_(1.0)
+        info = mg.pressure_solve(h, bad, x, 1e-9)
+        assert info.converged == bool(torch.all(bad == 0)) and info.iters == 0 and float(x.abs().max()) == 0.0
+        info = mg.pressure_solve(h, b, x, 1e-9)
+        assert (info.status, info.iters, info.rel_res) == (first.status, first.iters, first.rel_res)
+        assert torch.equal(x, ref)
+    h.destroy()
+
+
 def test_smoothing_of_misaligned_vectors(mg):
     """Vectors that start on an odd double (8-byte alignment only) give what aligned ones give."""
     cfg = syn.small_config(20, 9, levels=3, seed=syn.BASE_SEED + 720)
