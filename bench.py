@@ -47,7 +47,9 @@ WORKLOAD = ("C192L70 pressure solve: GCR(5) FP64 outer + 4-level FP32 V-cycle, s
 SWEEP_VARIANTS = ("plain", "zero", "prolong", "prolong0")
 
 
-KERNEL_SOURCES = ("kernels.cuh", "krylov.cuh", "mgsolve.cu")   # device code and launch configurations
+# device code and launch configurations
+KERNEL_SOURCES = ("kernels.cuh", "krylov.cuh", "mgsolve.cu", "sweep32.cuh", "sweep64.cuh", "sweep_launch.cuh",
+                  "sweep_tma.cuh")
 
 
 def _source_digest() -> str:
