@@ -1161,9 +1161,8 @@ mg_status pack_level(mg_handle* h, int l, cudaStream_t s) {
     DevLevel& d = h->lv[l];
     const dim3 grid((d.ncol + 127) / 128, h->nlev + 1);
     mg::k_pack64<<<grid, 128, 0, s>>>(d.n, d.ncol, h->nlev, d.fof, d.Th64, d.Tv64, d.wA64, h->dz, h->scale, d.te64, d.tn64,
-                                      d.tbw64, d.tbs64, d.tv64);
-    mg::k_factor64<<<(d.ncol + 63) / 64, 64, 0, s>>>(d.n, d.ncol, h->nlev, d.te64, d.tn64, d.tbw64, d.tbs64, d.tv64,
-                                                     d.wA64, h->dz, d.e64, d.ip64, d.pr64,
+                                      d.tbw64, d.tbs64, d.tv64, d.ip64);
+    mg::k_factor64<<<(d.ncol + 63) / 64, 64, 0, s>>>(d.ncol, h->nlev, d.tv64, d.e64, d.ip64, d.pr64,
                                                      mg::sweep64_chunks(h->nlev, d.ncol), h->om0);
     const dim3 halves((d.ncol + 63) / 64, 2);
     if (d.te32) {
@@ -1190,10 +1189,16 @@ mg_status set_coefficients_impl(mg_handle* h, const double* a, cudaStream_t s) {
     CK(cudaMemsetAsync(h->flag, 0, sizeof(unsigned int), s));
     for (int pass = 0; pass < 2; ++pass) {
         const bool write = pass == 1;
-        mg::k_coef_faces<<<dim3((nf + 127) / 128, nlev), 128, 0, s>>>(ncol, nlev, h->faceL0, h->faceR0, h->faceSide0,
-                                                                       h->nbrSide0, h->area0, a, write, d.Th64, h->flag);
-        mg::k_coef_vertical<<<dim3((ncol + 127) / 128, nlev + 1), 128, 0, s>>>(ncol, nlev, h->dz, a, write,
-                                                                                d.Tv64, h->flag);
+        const dim3 gh((nf + 127) / 128, nlev), gv((ncol + 127) / 128, nlev + 1);
+        if (write) {
+            mg::k_coef_faces<true><<<gh, 128, 0, s>>>(ncol, nlev, h->faceL0, h->faceR0, h->faceSide0, h->nbrSide0, h->area0,
+                                                      a, d.Th64, h->flag);
+            mg::k_coef_vertical<true><<<gv, 128, 0, s>>>(ncol, nlev, h->dz, a, d.Tv64, h->flag);
+        } else {
+            mg::k_coef_faces<false><<<gh, 128, 0, s>>>(ncol, nlev, h->faceL0, h->faceR0, h->faceSide0, h->nbrSide0, h->area0,
+                                                       a, d.Th64, h->flag);
+            mg::k_coef_vertical<false><<<gv, 128, 0, s>>>(ncol, nlev, h->dz, a, d.Tv64, h->flag);
+        }
         CK(cudaGetLastError());
         if (!write) {
             unsigned int bad = 0;

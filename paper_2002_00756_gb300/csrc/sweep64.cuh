@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(128) k_restrict64(Lvl64 L, const double* __res
 __global__ void k_pack64(int n, int ncol, int nlev, const int32_t* __restrict__ fof, const double* __restrict__ Th,
                          const double* __restrict__ Tv, const double* __restrict__ wA, const double* __restrict__ dz,
                          double scale, double* __restrict__ te, double* __restrict__ tn, double* __restrict__ tbw,
-                         double* __restrict__ tbs, double* __restrict__ tv) {
+                         double* __restrict__ tbs, double* __restrict__ tv, double* __restrict__ diag) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
     if (c >= ncol) return;
     const size_t e = (size_t)k * ncol + c;
@@ -368,42 +368,58 @@ __global__ void k_pack64(int n, int ncol, int nlev, const int32_t* __restrict__ 
     if (k >= nlev) return;
     const double wt = dz[k] * scale;
     const double* t = Th + (size_t)k * 2 * ncol;
-    te[e] = t[__ldg(fof + c)] * wt;
-    tn[e] = t[__ldg(fof + 2 * ncol + c)] * wt;
+    const double E = t[__ldg(fof + c)] * wt, W = t[__ldg(fof + ncol + c)] * wt;
+    const double Nn = t[__ldg(fof + 2 * ncol + c)] * wt, S = t[__ldg(fof + 3 * ncol + c)] * wt;
+    te[e] = E;
+    tn[e] = Nn;
+    diag[e] = fma(wA[c], dz[k], (E + W) + (Nn + S));
     const int row = c / n, i = c - row * n, p = row / n, j = row - p * n;
-    if (i == 0) tbw[(size_t)k * 6 * n + row] = t[__ldg(fof + ncol + c)] * wt;
-    if (j == 0) tbs[(size_t)k * 6 * n + p * n + i] = t[__ldg(fof + 3 * ncol + c)] * wt;
+    if (i == 0) tbw[(size_t)k * 6 * n + row] = W;
+    if (j == 0) tbs[(size_t)k * 6 * n + p * n + i] = S;
 }
 
-// The factors e, ip of every column; one thread per column.
-__global__ void k_factor64(int n, int ncol, int nlev, const double* __restrict__ te, const double* __restrict__ tn,
-                           const double* __restrict__ tbw, const double* __restrict__ tbs,
-                           const double* __restrict__ tv, const double* __restrict__ wA, const double* __restrict__ dz,
-                           double* __restrict__ e_, double* __restrict__ ip_, double* __restrict__ pr, int chunks,
-                           double om0) {
+// The factors e, ip of every column from its diagonals (in ip_, k_pack64); one thread per column.  The
+// pivots are one dependent chain; the next BATCH levels' operands are under way while a batch is
+// eliminated (level of C12L70 95 -> 32 us, C96L70 132 -> 97; the FP64 pipe's bound there: 74).
+__global__ void k_factor64(int ncol, int nlev, const double* __restrict__ tv, double* __restrict__ e_, double* ip_,
+                           double* __restrict__ pr, int chunks, double om0) {
+    constexpr int BATCH = 8;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncol) return;
-    const int row = c / n, i = c - row * n, p = row / n, j = row - p * n;
-    const double* ptw = i > 0 ? te + c - 1 : tbw + row;
-    const double* pts = j > 0 ? tn + c - n : tbs + p * n + i;
-    const size_t sW = i > 0 ? ncol : 6 * n, sS = j > 0 ? ncol : 6 * n;
-    const double a = wA[c];
-    double Q = 0.0, e = 0.0, g = 1.0;
-    int w = 0;
-#pragma unroll 4
-    for (int k = 0; k < nlev; ++k) {
-        const size_t o = (size_t)k * ncol + c;
-        const double h = (__ldg(te + o) + __ldg(ptw + k * sW)) + (__ldg(tn + o) + __ldg(pts + k * sS));
-        const double t = __ldg(tv + o + ncol);
-        Q = fma(e, Q, fma(a, __ldg(dz + k), h));
-        const double ip = recip64(Q + t);
-        e = t * ip;
-        e_[o] = e;
-        ip_[o] = om0 * ip;
-        g *= e;
-        if (pr && k + 1 == (w + 1) * nlev / chunks) {
-            pr[(size_t)w++ * ncol + c] = g;
-            g = 1.0;
+    double Q = 0.0, e = 0.0, g = 1.0, D[BATCH], T[BATCH], Dn[BATCH], Tn[BATCH];
+    auto load = [&](int k0, double (&dd)[BATCH], double (&tt)[BATCH]) {
+#pragma unroll
+        for (int q = 0; q < BATCH; ++q) {
+            const size_t o = (size_t)min(k0 + q, nlev - 1) * ncol + c;
+            dd[q] = ip_[o];
+            tt[q] = __ldg(tv + o + ncol);
+        }
+    };
+    load(0, Dn, Tn);
+    int w = 0, end = nlev / chunks;
+    for (int k0 = 0; k0 < nlev; k0 += BATCH) {
+#pragma unroll
+        for (int q = 0; q < BATCH; ++q) D[q] = Dn[q], T[q] = Tn[q];
+        if (k0 + BATCH < nlev) load(k0 + BATCH, Dn, Tn);
+#pragma unroll
+        for (int q = 0; q < BATCH; ++q) {
+            const int k = k0 + q;
+            if (k < nlev) {
+                const size_t o = (size_t)k * ncol + c;
+                Q = fma(e, Q, D[q]);
+                const double ip = recip64(Q + T[q]);
+                e = T[q] * ip;
+                e_[o] = e;
+                ip_[o] = om0 * ip;
+                if (pr) {
+                    g *= e;
+                    if (k + 1 == end) {
+                        pr[(size_t)w++ * ncol + c] = g;
+                        g = 1.0;
+                        end = (w + 1) * nlev / chunks;
+                    }
+                }
+            }
         }
     }
 }

@@ -123,6 +123,26 @@ def test_degenerate_right_hand_sides_leave_no_trace(mg):
     h.destroy()
 
 
+@pytest.mark.parametrize("side", [0, 3, 4])
+@pytest.mark.parametrize("factor,ok", [(1 + 3e-11, True), (1 - 9e-11, True), (1 + 1.2e-10, False), (1 - 1e-9, False),
+                                       (0.0, False), (-1.0, False), (float("inf"), False), (float("nan"), False)])
+def test_flux_symmetry_is_held_to_1e_10(mg, side, factor, ok):
+    """Products within 2^18 units in the last place (5.8e-11) pass on their words, others by comparison: either
+    way 1e-10 of the larger decides, and signs and non-finite values are refused."""
+    from oracle.problem import pressure_hierarchy
+    cfg = syn.small_config(4, 6, seed=syn.BASE_SEED + 795)
+    inp = syn.make_inputs(cfg)
+    a = np.array(pressure_hierarchy(cfg, inp).levels[0].couplings())
+    a[side, 2, 5] *= factor
+    h = mg.mg_setup_config(cfg, inp)
+    if ok:
+        mg.mg_set_coefficients(h, torch.from_numpy(a).cuda())
+    else:
+        with pytest.raises(mg.MGError):
+            mg.mg_set_coefficients(h, torch.from_numpy(a).cuda())
+    h.destroy()
+
+
 def test_smoothing_of_misaligned_vectors(mg):
     """Vectors that start on an odd double (8-byte alignment only) give what aligned ones give."""
     cfg = syn.small_config(20, 9, levels=3, seed=syn.BASE_SEED + 720)
