@@ -209,6 +209,11 @@ const char* mg_last_cuda_error(void);
  * and ensembles (a leak check: it returns to its earlier value once they are destroyed). */
 int64_t mg_inject_alloc_failure(int64_t nth);
 int64_t mg_live_allocations(void);
+/* mg_inject_wait_limit: polls after which a sweep's wait for its tensor copies gives up, for this
+ * handle's later calls (not for an ensemble recorded before); 0: every such wait runs out at once,
+ * negative: the default.  A sweep whose wait runs out gives NaN and waits for its copies before it
+ * ends.  Synchronous. */
+mg_status mg_inject_wait_limit(mg_handle* h, int32_t polls);
 
 /* Sizes of the handle's problem: ncol and N of the finest level, velocity unknowns
  * (0 without mixed data).  Any pointer may be NULL. */

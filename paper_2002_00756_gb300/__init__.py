@@ -87,6 +87,7 @@ _SIGS = {
     "mg_ensemble_create": [_VP, _I32, _VP, _VP, _D, ctypes.POINTER(ctypes.c_void_p)],
     "mg_ensemble_solve": [_VP, ctypes.POINTER(_Info), ctypes.POINTER(ctypes.c_int32), _VP],
     "mg_ensemble_destroy": [_VP],
+    "mg_inject_wait_limit": [_VP, _I32],
     "mg_destroy": [_VP],
     "mg_sizes": [_VP, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)],
     "helmholtz_apply": [_VP, _DP, _DP, _VP],

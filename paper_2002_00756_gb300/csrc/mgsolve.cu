@@ -100,6 +100,7 @@ struct mg_handle {
     int32_t* nbrSide0 = nullptr;
     unsigned int* flag = nullptr;
     unsigned int* timeout = nullptr;   // device: a bounded wait of a sweep ran into its limit
+    int polls = mg::WAIT_POLLS;        // that limit (mg_inject_wait_limit)
     // pressure solver K_H(A_H, P_H, eps_H) of the Schur-complement step (Sec. 4.1, Table 1)
     mg_pressure_solver ps{MG_PS_MG, 1e-2, 0.8, 10, 200};
     double* bv[8] = {};             // BiCGStab vectors r^, r, p, v, s, t, p^, s^ (allocated on demand)
@@ -434,7 +435,7 @@ mg_status launch_sweep32(mg_handle* h, int lev, const float* x, const float* xc,
     const mg::SweepMaps* maps = nullptr;
     const bool tiles = d.sweep_bd > 0 ? d.sweep_bd == 128 : tma_level(L.nlev, L.ncol);
     if (tiles && d.maps.size() == 2 && mode != mg::XM_PROLONG0) maps = &d.maps[x == d.x32[1]];
-    const mg::SweepCall32<C, P> q{L, mode, x, xc, b, raw, bcopy, xo, out64, om, maps, h->nsm, h->timeout};
+    const mg::SweepCall32<C, P> q{L, mode, x, xc, b, raw, bcopy, xo, out64, om, maps, h->nsm, h->polls, h->timeout};
     CK((mg::sweep32_run<C, P>(q, s)));
     if (L.n == 1 && !out64) {   // (a C1 column has several edges on one axis)
         mg::k_fill_rims<float><<<dim3(1, L.nlev), 32, 0, s>>>(L.n, L.ncol, L.hd, static_cast<float*>(xo));
@@ -900,6 +901,16 @@ void capture_graph(mg_handle* h, Body& body, cudaGraphExec_t* out) {
         h->graphs_off = true;
         cudaGetLastError();
     }
+}
+
+// Drop the cached graphs of the systems from `first` on; the next solve captures them again.
+void drop_graphs(mg_handle* h, int first) {
+    for (int sys = first; sys < 3; ++sys)
+        for (cudaGraphExec_t& g : h->gexec[sys])
+            if (g) {
+                cudaGraphExecDestroy(g);
+                g = nullptr;
+            }
 }
 
 // One GCR solve as resumable steps, so that several solves (an ensemble of handles) can
@@ -1764,6 +1775,15 @@ int64_t mg_inject_alloc_failure(int64_t nth) {
 
 int64_t mg_live_allocations(void) { return g_live.load(); }
 
+mg_status mg_inject_wait_limit(mg_handle* h, int32_t polls) {
+    if (!h) return MG_ERR_ARG;
+    DeviceGuard dg(h->device);
+    CK(cudaDeviceSynchronize());
+    h->polls = polls < 0 ? mg::WAIT_POLLS : polls;
+    drop_graphs(h, 0);
+    return MG_OK;
+}
+
 const char* mg_status_string(mg_status s) {
     switch (s) {
         case MG_OK: return "ok";
@@ -1878,13 +1898,7 @@ mg_status mg_set_pressure_solver(mg_handle* h, const mg_pressure_solver* ps) {
     }
     CK(cudaDeviceSynchronize());
     h->ps = *ps;
-    // the cached mixed-solve graphs hold the previous pressure solver
-    for (int sys = 1; sys < 3; ++sys)
-        for (cudaGraphExec_t& g : h->gexec[sys])
-            if (g) {
-                cudaGraphExecDestroy(g);
-                g = nullptr;
-            }
+    drop_graphs(h, 1);   // (those of the mixed solves hold the previous pressure solver)
     return MG_OK;
 }
 
@@ -2319,13 +2333,7 @@ mg_status mg_autotune(mg_handle* h, int32_t* choices, void* stream) {
             if (restr_ms[l] < best_t[l]) best_t[l] = restr_ms[l], best_kc[l] = kc, best_as[l] = 0;
     }
     for (int l = 0; l < L; ++l) h->lv[l].restrict_kc = best_kc[l];
-    // the cached GCR graphs hold the old launch shapes
-    for (auto& row : h->gexec)
-        for (cudaGraphExec_t& g : row)
-            if (g) {
-                cudaGraphExecDestroy(g);
-                g = nullptr;
-            }
+    drop_graphs(h, 0);   // (they hold the old launch shapes)
     if (choices)
         for (int l = 0; l < L; ++l) {
             choices[3 * l] = best_bd[l];

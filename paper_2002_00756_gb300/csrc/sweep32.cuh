@@ -535,6 +535,7 @@ struct SweepCall32 {
     double omega;
     const SweepMaps* maps;   // tensor maps of x, xc, b and the level's data (sweep_tma.cuh), or NULL
     int nsm;
+    int polls;               // limit of a TMA wait
     unsigned int* timeout;   // set by a TMA wait that runs into its limit
 };
 

@@ -42,7 +42,7 @@ cudaError_t go_tma(const SweepCall32<C, P>& q, cudaStream_t s) {
     const int per_sm = std::max(1, std::min({227 * 1024 / (Y.total + 1024), tma_blocks(MODE, BRAW, sizeof(P)) * tma_threads(K) / threads, 8}));
     const int grid = std::min(6 * q.L.n * tr, per_sm * q.nsm);
     kern<<<grid, threads, Y.total, s>>>(*q.maps, q.L, static_cast<const double*>(BRAW ? q.b : nullptr), q.bcopy,
-                                        static_cast<O*>(q.xo), (float)q.omega, tr, tw, q.timeout);
+                                        static_cast<O*>(q.xo), (float)q.omega, tr, tw, q.polls, q.timeout);
     return cudaGetLastError();
 }
 

@@ -56,9 +56,10 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// waits for the phase of the given parity; false after the iteration limit
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    for (int i = 0; i < (1 << 20); ++i) {
+constexpr int WAIT_POLLS = 1 << 20;   // default limit of a wait, and that of a late copy's second wait
+// waits for the phase of the given parity; false after `polls` polls
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int polls) {
+    for (int i = 0; i < polls; ++i) {
         uint32_t ok;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
@@ -80,6 +81,13 @@ __device__ __forceinline__ void tma_load(void* dst, const CUtensorMap* m, int x,
 // The lower half of the levels is walked upwards, the upper half downwards, each by a group of G
 // warps with a chunk of up to K steps per warp.  Each group has its own boxes, its own mbarrier and
 // issues its own copies, so its buffers are refilled as soon as its own warps have read them.
+//
+// A copy that does not arrive within the limit: the group's threads agree on it where they meet anyway
+// (a reduction over the barrier: 0.2-0.5 % of a solve; a mark in shared memory costs more), and from then
+// on issue no copy and touch the mbarrier no more, whose
+// phase is still open.  They go through their remaining tiles all the same, because the other group's
+// interface waits for them, and give NaN, which the interface hands to the other half of the column.
+// Before they leave they wait once more, with the default limit, for the copies in flight, and report.
 __host__ __device__ constexpr int tma_max_levels(int K) { return K == 7 ? 70 : 80; }
 __host__ __device__ constexpr int tma_chunks(int nlev, int K) { return ((nlev + 1) / 2 + K - 1) / K; }
 __host__ __device__ constexpr int tma_threads(int K) { return 64 * tma_chunks(tma_max_levels(K), K); }
@@ -135,7 +143,7 @@ template <typename C, typename P, int MODE, typename O, bool BRAW, int K, bool F
 __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(P)))
     k_sweep_tma(const __grid_constant__ SweepMaps M, Lvl32<C, P> L, const double* __restrict__ braw,
                 float* __restrict__ bcopy, O* __restrict__ xo, float omega, int tiles_row, int tile_w,
-                unsigned int* __restrict__ timeout) {
+                int polls, unsigned int* __restrict__ timeout) {
     static_assert(MODE != XM_PROLONG0, "iterate source");
     constexpr bool PRO = MODE == XM_PROLONG, ZERO = MODE == XM_ZERO, PADO = sizeof(O) == 4, D64 = sizeof(P) == 8;
     constexpr int TW = 16 / (int)sizeof(C), TP = 32 + TW;   // te: columns to the west, row pitch
@@ -156,9 +164,20 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
     P* const sy = reinterpret_cast<P*>(sm_all + Y.sy) + w * 32 + lane;
     float* const so = reinterpret_cast<float*>(sm_all + Y.so) + w * 32 + lane;
     P* const si = reinterpret_cast<P*>(sm_all + Y.si) + lane;   // [2 tiles][2 halves][3][32]
-    auto group_sync = [&]() {
-        if (up) asm volatile("bar.sync 2, %0;" ::"r"(gthreads) : "memory");
-        else asm volatile("bar.sync 1, %0;" ::"r"(gthreads) : "memory");
+    // the group meets; whether any of its threads says v
+    auto group_any = [&](bool v) {
+        uint32_t any;
+        if (up)
+            asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 2, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+                         : "=r"(any)
+                         : "r"((uint32_t)v), "r"(gthreads)
+                         : "memory");
+        else
+            asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+                         : "=r"(any)
+                         : "r"((uint32_t)v), "r"(gthreads)
+                         : "memory");
+        return any != 0;
     };
     const int pair = 3 + (up ? G - 1 : 0);   // barriers pair .. pair + G - 2 between the group's chunks
     // padded column of a tile's first parent, and of the row of parents its N (odd rows) or S (even
@@ -206,8 +225,8 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
         for (int i = 0; i < (BRAW ? K : 0); ++i) bn[i] = __ldg(braw + (level(i) * L.ncol + c));
     };
     if (BRAW && (int)blockIdx.x < ntiles) fetch_b(blockIdx.x);
-    uint32_t phase = 0;
-    bool late = false;
+    uint32_t phase = 0, open = 0;   // open: parity of the phase that a late copy has left open
+    bool late = false;              // the same for all of the group's threads
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, phase ^= 1) {
         const int row = t / tiles_row, i0 = (t - row * tiles_row) * tile_w;
         const int p = row / n, j = row - p * n, cols = min(tile_w, n - i0);
@@ -234,7 +253,7 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
                 q.e[i] = __ldg(L.e + o);
             }
         }
-        late |= !mbar_wait(bar, phase);
+        const bool miss = !late && !mbar_wait(bar, phase, polls);
         P an = P(0);   // a_next of the chunk's last step
         // reads the chunk, walking the rows of the boxes in direction D
         auto read = [&](auto dir) {
@@ -299,9 +318,12 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
         if (up) read(std::integral_constant<int, -1>());
         else read(std::integral_constant<int, 1>());
         // the group's values are in registers: the next tile's copies may overwrite its boxes
-        group_sync();
+        if (group_any(miss)) {
+            late = true;
+            open = phase;
+        }
         if (t + (int)gridDim.x < ntiles) {
-            if (gtid == 0) issue(t + gridDim.x);
+            if (gtid == 0 && !late) issue(t + gridDim.x);
             if (BRAW) fetch_b(t + gridDim.x);
         }
         if (BRAW && lane < cols) {
@@ -336,6 +358,7 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
                 ql = FULL || i < len ? q.ip[i] : ql;
                 xl = FULL || i < len ? q.x[i] : xl;
             }
+            if (late) y = P(__int_as_float(0x7fc00000));
             P* const mine = si + (2 * phase + up) * 96;
             const P* const other = si + (2 * phase + !up) * 96;
             mine[0] = ql;
@@ -371,9 +394,9 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
             }
         }
     }
-    if (late) {   // a copy did not arrive within the limit: reported (the tile's result is NaN)
+    if (late) {
         atomicExch(timeout, 1u);
-        mbar_wait(bar, phase ^ 1);
+        mbar_wait(bar, open, WAIT_POLLS);
     }
 }
 
