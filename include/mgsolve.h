@@ -62,7 +62,8 @@ typedef enum {
     MG_ERR_NOMEM = -3,          /* device or host allocation failed in mg_setup */
     MG_ERR_NOT_CONVERGED = -4,  /* max_iter reached; info and the best iterate are filled */
     MG_ERR_BREAKDOWN = -5,      /* Krylov breakdown: <w, w> = 0 or a non-finite scalar */
-    MG_ERR_TIMEOUT = -6,        /* a bounded device-side wait of a solve ran into its limit */
+    MG_ERR_TIMEOUT = -6,        /* a bounded device-side wait of a solve ran into its limit (the calls that
+                                   do not synchronise cannot say so: their result is NaN then) */
     MG_ERR_UNSUPPORTED = -7     /* request outside what the handle was set up for */
 } mg_status;
 

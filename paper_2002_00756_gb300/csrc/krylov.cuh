@@ -179,12 +179,13 @@ __global__ void k_coef_grad(Lvl<double, double> L, const double* __restrict__ la
     grad[5 * N + e] = k > 0 ? -l * (x0 - x[e - ncol]) : 0.0;
 }
 
-// Start of a GCR solve: r = b, x = 0, <b, b>, in one pass over memory (a copy, a fill and a product before: C192L70
+// Start of a GCR solve: r = b, x = 0, <b, b> and no wait run out yet, in one pass over memory (a copy, a fill and a product before: C192L70
 // solve 10.50 -> 10.45 ms, together with the first iteration launched ahead).
 __global__ void __launch_bounds__(RED_THREADS) k_gcr_start(size_t n, const double* __restrict__ b, double* __restrict__ r,
                                                            double* __restrict__ x, double* partials,
-                                                           unsigned int* ticket, double* bb) {
+                                                           unsigned int* ticket, double* bb, unsigned int* timeout) {
     double v[1] = {0.0}, t[1];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *timeout = 0u;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const double e = __ldg(b + i);
         r[i] = e;
@@ -226,8 +227,9 @@ __global__ void k_apply_a6(Lvl<double, double> L, const double* __restrict__ a6,
 // r = r^ = b, x = 0; rho = <b, b>
 __global__ void __launch_bounds__(RED_THREADS) k_bicg_start(size_t n, const double* __restrict__ b, double* r,
                                                             double* rh, double* x, double tol, double* partials,
-                                                            unsigned int* ticket, BicgScal* S) {
+                                                            unsigned int* ticket, BicgScal* S, unsigned int* timeout) {
     double v[1] = {0.0}, t[1];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *timeout = 0u;
     MG_GRID_STRIDE(i, n) {
         const double bi = b[i];
         r[i] = bi;
@@ -331,7 +333,7 @@ struct EnsState {
     double bb;     // <b, b>
     double rel;    // ||r|| / ||b|| after the last iteration
     int it;        // iterations done
-    int status;    // MG_OK, MG_ERR_NOT_CONVERGED or MG_ERR_BREAKDOWN
+    int status;    // MG_OK, MG_ERR_NOT_CONVERGED, MG_ERR_BREAKDOWN or MG_ERR_TIMEOUT
 };
 
 struct EnsHandles {
@@ -368,12 +370,13 @@ __global__ void k_ens_init(const GcrScal* S, EnsState* st, int R, int max_iter, 
 }
 
 // after the iteration of slot j: the convergence test and the solution update of a single solve
-__global__ void k_ens_decide(const GcrScal* S, EnsState* st, int j, int R, int max_iter, double tol, EnsHandles hs) {
+__global__ void k_ens_decide(const GcrScal* S, EnsState* st, int j, int R, int max_iter, double tol, EnsHandles hs,
+                             const unsigned int* timeout) {
     const int it = st->it + 1;
     st->it = it;
     const double rr = S->rr;
     if (!isfinite(rr)) {   // breakdown: stop without the update (x keeps the last cycle's value)
-        st->status = MG_ERR_BREAKDOWN;
+        st->status = *timeout ? MG_ERR_TIMEOUT : MG_ERR_BREAKDOWN;
         ens_set_slots(hs, R, 0, false);
         cudaGraphSetConditional(hs.w, 0u);
         return;

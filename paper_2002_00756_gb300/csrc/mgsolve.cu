@@ -714,6 +714,15 @@ mg_status run_jacobi(mg_handle* h, double omega, int sweeps, const double* b, do
     return run_cycle(h, Cycle{1, omega, 0, 0, sweeps}, b, x, s);
 }
 
+// The status of a solve whose residual is no longer finite: a sweep's copy that did not arrive leaves NaN
+// and a flag, which every solve clears at its start.
+mg_status broken(mg_handle* h, cudaStream_t s) {
+    unsigned int late = 0;
+    CK(cudaMemcpyAsync(&late, h->timeout, sizeof late, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    return late ? MG_ERR_TIMEOUT : MG_ERR_BREAKDOWN;
+}
+
 // BiCGStab(H, P, tol) on the finest level (Sec. 4.1 solver list; Table 1 "Krylov" rows) from
 // x = 0: the vector updates and inner products run in the kernels above with device scalars;
 // the host reads them once per iteration to test convergence.  *iters counts a half step as 0.5.
@@ -736,7 +745,7 @@ mg_status bicgstab(mg_handle* h, const double* b, double* x, double tol, int max
         return MG_OK;
     };
     *iters = 0.0;
-    mg::k_bicg_start<<<G, B, 0, s>>>(n, b, r, rh, x, tol, h->partials, tk, h->bs);
+    mg::k_bicg_start<<<G, B, 0, s>>>(n, b, r, rh, x, tol, h->partials, tk, h->bs, h->timeout);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(h->host_bs, h->bs, sizeof(mg::BicgScal), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -758,12 +767,12 @@ mg_status bicgstab(mg_handle* h, const double* b, double* x, double tol, int max
         CK(cudaMemcpyAsync(h->host_bs, h->bs, sizeof(mg::BicgScal), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         const mg::BicgScal& S = *h->host_bs;
-        if (!std::isfinite(S.alpha) || !std::isfinite(S.ss)) return MG_ERR_BREAKDOWN;
+        if (!std::isfinite(S.alpha) || !std::isfinite(S.ss)) return broken(h, s);
         if (S.half) {
             *iters = i + 0.5;
             return MG_OK;
         }
-        if (!std::isfinite(S.omega) || !std::isfinite(S.rr) || !std::isfinite(S.rho)) return MG_ERR_BREAKDOWN;
+        if (!std::isfinite(S.omega) || !std::isfinite(S.rr) || !std::isfinite(S.rho)) return broken(h, s);
         *iters = i + 1.0;
         if (S.rr <= S.tol2bb) return MG_OK;
         if (S.omega == 0.0 || S.rho == 0.0) return MG_ERR_BREAKDOWN;
@@ -934,7 +943,7 @@ mg_status gcr_start(mg_handle* h, GcrRun& g, const double* b, cudaStream_t s) {
     {
         Prof pr(h, MG_K_DOT, 0, 24.0 * g.n, s);
         mg::k_gcr_start<<<vec_grid(h, g.n), mg::RED_THREADS, 0, s>>>(g.n, b, h->r, g.x, h->partials, h->tickets + TK_DOT,
-                                                                    &h->gs->bb);
+                                                                    &h->gs->bb, h->timeout);
         CK(cudaGetLastError());
     }
     CK(cudaMemcpyAsync(h->host_sc + 1, &h->gs->bb, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -984,10 +993,7 @@ mg_status gcr_landed(mg_handle* h, GcrRun& g, cudaStream_t s) {
     ++g.it;
     const double rr = h->host_sc[0];
     if (!std::isfinite(rr)) {
-        unsigned int late = 0;   // a sweep's copy that did not arrive leaves NaN and this flag
-        CK(cudaMemcpyAsync(&late, h->timeout, sizeof late, cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        g.st = late ? MG_ERR_TIMEOUT : MG_ERR_BREAKDOWN;
+        g.st = broken(h, s);
         g.active = false;
         return MG_OK;
     }
@@ -1694,7 +1700,7 @@ mg_status build_member(mg_ensemble* e, int i, mg_handle* h, const double* b, dou
     std::vector<cudaGraphNode_t> deps;
     CK(cudaStreamBeginCaptureToGraph(e->cs, e->graph, root.data(), nullptr, root.size(), mode));
     mg::k_gcr_start<<<vec_grid(h, n), mg::RED_THREADS, 0, e->cs>>>(n, b, h->r, x, h->partials, h->tickets + TK_DOT,
-                                                                   &h->gs->bb);
+                                                                   &h->gs->bb, h->timeout);
     mg::k_ens_init<<<1, 1, 0, e->cs>>>(h->gs, st, R, h->prm.max_iter, hs);
     CK(cudaGetLastError());
     TRY(end_segment(e, deps));
@@ -1712,7 +1718,7 @@ mg_status build_member(mg_ensemble* e, int i, mg_handle* h, const double* b, dou
         TRY(run_vcycle(h, h->r, z, e->cs));
         TRY(apply_gcr(h, z, w, j, e->cs));
         TRY(dispatch_j<RunOrth>(j, h, n, e->cs));
-        mg::k_ens_decide<<<1, 1, 0, e->cs>>>(h->gs, st, j, R, h->prm.max_iter, tol, hs);
+        mg::k_ens_decide<<<1, 1, 0, e->cs>>>(h->gs, st, j, R, h->prm.max_iter, tol, hs, h->timeout);
         CK(cudaGetLastError());
         TRY(end_segment(e, deps));
         TRY(add_conditional(wbody, {inode}, hs.x[j], cudaGraphCondTypeIf, &xnode, &xbody));

@@ -84,10 +84,10 @@ __device__ __forceinline__ void tma_load(void* dst, const CUtensorMap* m, int x,
 //
 // A copy that does not arrive within the limit: the group's threads agree on it where they meet anyway
 // (a reduction over the barrier: 0.2-0.5 % of a solve; a mark in shared memory costs more), and from then
-// on issue no copy and touch the mbarrier no more, whose
-// phase is still open.  They go through their remaining tiles all the same, because the other group's
-// interface waits for them, and give NaN, which the interface hands to the other half of the column.
-// Before they leave they wait once more, with the default limit, for the copies in flight, and report.
+// on issue no copy and touch the mbarrier no more, whose phase is still open.  They go through their
+// remaining tiles all the same, because the other group's interface waits for them, and give NaN, which
+// the interface hands to the other half of the column.  Before they leave they wait once more, with the
+// default limit, for the copies in flight, and report.
 __host__ __device__ constexpr int tma_max_levels(int K) { return K == 7 ? 70 : 80; }
 __host__ __device__ constexpr int tma_chunks(int nlev, int K) { return ((nlev + 1) / 2 + K - 1) / K; }
 __host__ __device__ constexpr int tma_threads(int K) { return 64 * tma_chunks(tma_max_levels(K), K); }
