@@ -29,17 +29,21 @@ cudaError_t shape(const SweepCall32<C, P>& q, cudaStream_t s) {
     return go<C, P, MODE, B, O, BRAW, BIG_K>(q, s);
 }
 
+constexpr int TMA_SMEM = 227 * 1024;   // shared memory of an SM, and the most a block can have
+
 template <typename C, typename P, int MODE, typename O, bool BRAW, int K, bool FULL>
 cudaError_t go_tma(const SweepCall32<C, P>& q, cudaStream_t s) {
     const TmaLayout<C, P, MODE, BRAW, K> Y(q.L.nlev);
     auto kern = k_sweep_tma<C, P, MODE, O, BRAW, K, FULL>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Y.total);
+    // (the limit is the function's, for every thread and handle: the device's maximum, whatever this launch
+    // takes.  Two threads with handles of different heights could lower one of Y.total under each other.)
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TMA_SMEM);
     if (e != cudaSuccess) return e;
     const int threads = 64 * tma_chunks(q.L.nlev, K);
     // tiles: up to 32 columns of a row, a multiple of 16 bytes of the couplings wide (tensor coordinates)
     constexpr int Q = 16 / (int)sizeof(C);
     const int tr = (q.L.n + TMA_COLS - 1) / TMA_COLS, tw = ((q.L.n + tr - 1) / tr + Q - 1) / Q * Q;
-    const int per_sm = std::max(1, std::min({227 * 1024 / (Y.total + 1024), tma_blocks(MODE, BRAW, sizeof(P)) * tma_threads(K) / threads, 8}));
+    const int per_sm = std::max(1, std::min({TMA_SMEM / (Y.total + 1024), tma_blocks(MODE, BRAW, sizeof(P)) * tma_threads(K) / threads, 8}));
     const int grid = std::min(6 * q.L.n * tr, per_sm * q.nsm);
     kern<<<grid, threads, Y.total, s>>>(*q.maps, q.L, static_cast<const double*>(BRAW ? q.b : nullptr), q.bcopy,
                                         static_cast<O*>(q.xo), (float)q.omega, tr, tw, q.polls, q.timeout);
