@@ -379,7 +379,7 @@ mg_status mixed_coefficient_gradient(mg_handle* h, const double* lam_u, const do
 
 /* Autotuner of the column tiles: for every multigrid level, times the candidate forms of the
  * block-Jacobi sweep (FP32 V-cycles: register chunks, or tensor-copy tiles for 8 to 80 levels) and
- * of the residual + restriction (4, 8, 16, 24, 35 or 70 levels per thread) with CUDA events around
+ * of the residual + restriction (the built-in levels per thread, and 4, 8, 16, 24, 35 or 70) with CUDA events around
  * every launch of full V-cycles on the handle's own buffers, and keeps the fastest per
  * level for every later call.  Every form gives the same result bit for bit (each output
  * element is computed from the same inputs in the same order), so tuning
@@ -387,7 +387,8 @@ mg_status mixed_coefficient_gradient(mg_handle* h, const double* lam_u, const do
  * graphs (they are captured again by the next solve).  MG_ERR_UNSUPPORTED while per-launch
  * profiling (mg_profile_start) is on.
  * choices: NULL or 3 * levels int32 written per level: sweep form (64: register chunks, 128: tiles),
- * restriction levels per thread, 0 (0 and -1 on the coarsest level, which has no restriction). */
+ * fastest of the listed restriction levels per thread, 1 where the built-in number is faster than it and
+ * stays, 0 where it is taken (0 and -1 on the coarsest level, which has no restriction). */
 mg_status mg_autotune(mg_handle* h, int32_t* choices, void* stream);
 
 /* [u; p] = P_mixed [ru; rp], the Schur-complement preconditioner with one V-cycle. */

@@ -476,7 +476,8 @@ def mixed_coefficient_gradient(h: Handle, lam_u, u, p, grad_g, grad_beta_up, gra
 
 def mg_autotune(h: Handle, stream=None) -> list[tuple[int, int, int]]:
     """Pick the fastest sweep form and restriction launch shape per level (see mg_autotune in
-    mgsolve.h); returns (sweep form, restriction levels per thread, 0 or -1) per level."""
+    mgsolve.h); returns (sweep form, fastest listed restriction levels per thread, whether the
+    built-in number stays instead) per level."""
     ch = (ctypes.c_int32 * (3 * h.levels))()
     _check(load().mg_autotune(h.ptr, ch, _stream(stream)), "mg_autotune")
     return [(ch[3 * l], ch[3 * l + 1], ch[3 * l + 2]) for l in range(h.levels)]

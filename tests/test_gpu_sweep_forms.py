@@ -1,0 +1,50 @@
+"""The launch forms of the column kernels: what the autotuner keeps, and that every form agrees."""
+import numpy as np
+import pytest
+
+import synthetic as syn
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def mg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2002_00756_gb300.build import build
+    build()
+    import paper_2002_00756_gb300 as m
+    m.load()
+    return m
+
+
+def setup(mg, n, nlev, levels, precision, **kw):
+    cfg = syn.small_config(n, nlev, levels=levels, seed=syn.BASE_SEED + 850 + n, **kw)
+    inp = syn.make_inputs(cfg)
+    return cfg, inp, mg.mg_setup_config(cfg, inp, precision=precision), torch.from_numpy(inp["rhs"]).cuda().ravel()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_tuning_does_not_slow_the_restriction_down(mg, precision):
+    """C48L30, whose built-in restriction takes one level per thread (half the time of eight): the tuner
+    keeps it, unless one of its own numbers measures faster.  Times within 25 % (events around launches
+    of some 10 us)."""
+    _, _, h, b = setup(mg, 48, 30, 3, precision)
+    x = torch.empty_like(b)
+
+    def restrictions():
+        out = []
+        for level in (0, 1):
+            mg.mg_profile_start(h, 256, "restrict", level)
+            for _ in range(60):
+                mg.vcycle(h, b, x)
+            out.append(float(np.median([r["ms"] for r in mg.mg_profile_stop(h)])))
+        return out
+
+    restrictions()
+    before = restrictions()
+    mg.mg_autotune(h)
+    after = restrictions()
+    assert all(t <= 1.25 * s for s, t in zip(before, after)), (before, after)
+    h.destroy()
