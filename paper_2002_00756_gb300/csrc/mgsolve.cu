@@ -86,7 +86,7 @@ struct mg_handle {
     std::vector<DevLevel> lv;
     double* rdz64 = nullptr;
     float* rdz32 = nullptr;
-    double om0 = 1.0;           // relaxation factor folded into the FP64 factors: prm.omega unless 0
+    double om0 = 1.0;           // relaxation factor folded into the FP64 factors (prm.omega)
     double scale = 1.0;         // power of two in the FP64 volume weights, 1 / (largest finest area x depth)
     double* a6 = nullptr;       // finest level: six premultiplied FP64 couplings and 1 + their sum, per cell
     bool nine = false;          // 9-cell stencil (mg_setup_9pt)
@@ -1304,7 +1304,8 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
     h->n = n;
     h->nlev = nlev;
     h->prm = *prm;
-    if (prm->omega != 0.0) h->om0 = prm->omega;
+    // (a factor near the ends of FP64's range stays outside: a pressure solver with another omega divides it out)
+    if (std::fabs(prm->omega) >= 0x1p-100 && std::fabs(prm->omega) <= 0x1p100) h->om0 = prm->omega;
     CK(cudaGetDevice(&h->device));
     CK(cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->device));
     h->red_grid = 8 * h->nsm;

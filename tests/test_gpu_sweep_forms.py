@@ -48,3 +48,21 @@ def test_tuning_does_not_slow_the_restriction_down(mg, precision):
     after = restrictions()
     assert all(t <= 1.25 * s for s, t in zip(before, after)), (before, after)
     h.destroy()
+
+
+@pytest.mark.parametrize("omega", [0.0, 1e-310, 1e-200, 1e300])
+def test_line_relaxation_has_its_own_omega(mg, omega):
+    """The FP64 factors hold the V-cycle's relaxation factor; a pressure solver with another one gives what a
+    handle set up with that one gives, also where the quotient of the two is out of range.  Three roundings
+    per level of 9: 1e-13 of the largest element."""
+    cfg = syn.small_config(10, 9, levels=2, seed=syn.BASE_SEED + 860)
+    inp = syn.make_inputs(cfg)
+    x = []
+    for om in (0.8, omega):
+        h = mg.mg_setup(cfg.n, cfg.nlev, inp["z_if"], inp["g"], levels=2, omega=om)
+        mg.mg_set_pressure_solver(h, "jacobi", omega=0.8, sweeps=3)
+        b = torch.from_numpy(inp["rhs"]).cuda().ravel()
+        x.append(torch.empty_like(b))
+        mg.helmholtz_solve(h, b, x[-1])
+        h.destroy()
+    assert float((x[0] - x[1]).abs().max()) <= 1e-13 * float(x[0].abs().max())
