@@ -517,9 +517,7 @@ struct MixedDev {
     // coefficient gradient: d(kappa_f / d_f) / d g_i = c_s dt / (2 d_f) for both cells of f
     const double* cdh;              // [nfh]      c_s dt / (2 centre distance)
     const double* cdv;              // [nlev+1]   c_s dt / (2 dzc), 0 on surface and lid
-    // 1 / W_f of interior faces as factors at hand: kd_h divv rel and kd_v / (c_s dt area)
-    const double* rel;              // [nfh]      1 / ((c_s dt)^2 edge length)
-    const double* rcA;              // [ncol]     1 / (c_s dt area)
+    const double* rW;               // 1 / Wf, of the same rounded weights (their own errors cancel in W^-1 M^T W)
     double eps;                     // strength of B_w
 };
 
@@ -532,12 +530,12 @@ __global__ void k_mx_adj_scale(MixedDev M, size_t nu, const double* __restrict__
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nu + np; i += (size_t)gridDim.x * blockDim.x) {
         if (i < nu) {
             const double w = __ldg(M.Wf + i);
-            out_u[i] = MULT ? in_u[i] * w : in_u[i] * recip64(w);
+            out_u[i] = MULT ? in_u[i] * w : in_u[i] / w;
         } else {
             const size_t e = i - nu;
             const int k = (int)(e / M.ncol), c = (int)(e - (size_t)k * M.ncol);
             const double v = __ldg(area + c) * __ldg(dz + k);
-            out_p[e] = MULT ? -(in_p[e] * v) : -(in_p[e] * recip64(v));
+            out_p[e] = MULT ? -(in_p[e] * v) : -(in_p[e] / v);
         }
     }
 }
@@ -656,10 +654,12 @@ enum { MX_A = 0, MX_HAT = 1, MX_RHS = 2, MX_UPDATE = 3, MX_UPDATE_W = 4 };
 // that is resident at once (as k_apply_gcr's).  Face numbers, couplings and weights of the columns are
 // read once per unit, not once per level; with J >= 0 the GCR sums of the new direction J are taken in
 // the same pass, while its rows are in registers (a pass over J + 2 vectors and three launches less).
-// The FP64 pipe bounds MX_A and MX_HAT: 29 and 34 operations per cell (18 / 22 of them on its two
+// The FP64 pipe bounds MX_A and MX_HAT: 29 and 32 operations per cell (18 / 20 of them on its two
 // horizontal faces) and 4 (J + 2) of the sums.  A-hat's weights therefore come from Step 3, which
-// stores W u' beside u' (one product per face instead of six), and its quotient by W from factors
-// that are loaded anyway.
+// stores W u' beside u' (one product per face instead of six), and its quotient by W is a product with
+// the stored reciprocal.  (1 / W put together from kd and the geometry would save the load, but its error is
+// not the one of W u': RMS error of A^T v against long double 7.9e-17 at C24L30, 7.2e-17 with the stored
+// reciprocal, 6.7e-17 with the quotient.)
 // C48L30, sums of 0..4 directions included, on average: MX_A 38 us (four launches of a thread per row and
 // level: 56), MX_HAT 54 us (91); the FP64 pipe's bound with J = 2: 32 and 36.  Steps 1 and 3 have few
 // registers and run on five blocks per SM.
@@ -680,6 +680,8 @@ __global__ void __launch_bounds__(RED_THREADS, mixed_blocks(MODE)) k_mixed(
     const unsigned G = MODE == MX_RHS ? gc : UPD ? gh + gc : gh + 2 * gc;
     const size_t nh = (size_t)M.nlev * nfh, nu = nh + (size_t)(M.nlev + 1) * ncol;
     const double *uv = u + nh, *wv = MODE == MX_HAT ? wu + nh : uv;
+    // m / W_e: the plain quotient in mixed_apply_transpose, the reciprocal in a solve's operator
+    auto over_w = [&](double m, size_t e) { return J < 0 ? m / __ldg(M.Wf + e) : m * __ldg(M.rW + e); };
     // row e of [u; p] comes out as y
     auto put = [&](double* to, size_t e, double y) {
         *to = y;
@@ -703,7 +705,7 @@ __global__ void __launch_bounds__(RED_THREADS, mixed_blocks(MODE)) k_mixed(
                     wt[i] = __ldg((MODE == MX_HAT ? M.wfT : M.wf) + (size_t)i * nfh + f);
                 }
             }
-            const double rm = UPD ? __ldg(M.rmlump_h + f) : 0.0, rel = MODE == MX_HAT ? __ldg(M.rel + f) : 0.0;
+            const double rm = UPD ? __ldg(M.rmlump_h + f) : 0.0;
 #pragma unroll 2
             for (int k = k0; k < k1; ++k) {
                 const double *ul = (MODE == MX_HAT ? wu : u) + (size_t)k * nfh, *pl = p + (size_t)k * ncol;
@@ -720,8 +722,9 @@ __global__ void __launch_bounds__(RED_THREADS, mixed_blocks(MODE)) k_mixed(
 #pragma unroll
                         for (int i = 0; i < 6; ++i) m = fma(wt[i], __ldg(ul + cf[i]), m);
                         if (MODE == MX_A) y = m;
+                        if (MODE == MX_HAT) y = fma(M.ms, uf, over_w(m, o));
                     }
-                    y = fma(kd, MODE == MX_HAT ? fma(rel * __ldg(M.divv + k), m, dp) : dp, y);
+                    y = fma(kd, dp, y);
                 }
                 put(yu + o, o, y);
             }
@@ -729,7 +732,6 @@ __global__ void __launch_bounds__(RED_THREADS, mixed_blocks(MODE)) k_mixed(
             const unsigned c = (g - gh) * 32 + lane;
             if (c >= ncol) continue;
             const int k2 = k1 == M.nlev ? k1 + 1 : k1;
-            const double rcA = MODE == MX_HAT ? __ldg(M.rcA + c) : 0.0;
             double ub = k0 > 0 ? __ldg(uv + (size_t)(k0 - 1) * ncol + c) : 0.0, u0 = __ldg(uv + (size_t)k0 * ncol + c);
             double pb = k0 > 0 ? __ldg(p + (size_t)(k0 - 1) * ncol + c) : 0.0;
 #pragma unroll 2
@@ -746,7 +748,7 @@ __global__ void __launch_bounds__(RED_THREADS, mixed_blocks(MODE)) k_mixed(
                         if (MODE == MX_HAT) {   // the couplings of the faces above and below to this one
                             const double m = fma(__ldg(M.w_up + o - ncol), __ldg(wv + o - ncol),
                                                  __ldg(M.w_dn + o + ncol) * __ldg(wv + o + ncol));
-                            y = fma(kd, fma(rcA, m, dp), M.mv * u0);
+                            y = fma(kd, dp, fma(M.mv, u0, over_w(m, nh + o)));
                         }
                         if (UPD) y = fma(-kd, dp, u0) * __ldg(M.rmlump + o);
                     }

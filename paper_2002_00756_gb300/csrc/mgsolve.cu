@@ -1121,6 +1121,11 @@ __global__ void k_rims(int n, int ncol, const int32_t* __restrict__ nbr, int32_t
     hd[(size_t)s * ncol + c] = d;
 }
 
+__global__ void k_reciprocal(size_t n, const double* __restrict__ a, double* __restrict__ r) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        r[i] = 1.0 / a[i];
+}
+
 __global__ void k_parents(int n, int ncol, const int32_t* __restrict__ nbr, int32_t* __restrict__ par) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
     if (c < ncol) par[(size_t)s * ncol + c] = mg::parent_col(s < 4 ? nbr[(size_t)s * ncol + c] : c, n);
@@ -1542,14 +1547,12 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
                 if (found < 0) return MG_ERR_ARG;   // the coupling pattern is symmetric by construction
                 wfT[(size_t)t * nfh + f] = hm.wf[(size_t)found * nfh + gf];
             }
-        std::vector<double> cdh(nfh), cdv(nlev + 1, 0.0), rel(nfh), rcA(ncol0);
+        std::vector<double> cdh(nfh), cdv(nlev + 1, 0.0);
         for (int f = 0; f < nfh; ++f) cdh[f] = c / (2.0 * G.cdist[G.faceSide[f] * ncol0 + G.faceL[f]]);
         for (int kf = 1; kf < nlev; ++kf) cdv[kf] = c / (2.0 * vg.dzc[kf]);
-        for (int f = 0; f < nfh; ++f) rel[f] = 1.0 / (c * c * G.edge_len[G.faceSide[f] * ncol0 + G.faceL[f]]);
-        for (int col = 0; col < ncol0; ++col) rcA[col] = 1.0 / (c * G.area[col]);
         int32_t *fL, *fR, *dcf = nullptr;
         double *dkd_h, *dkd_v, *dsdiv, *dwu, *dwd, *dml, *ddivv, *dwf = nullptr, *dmlh, *dwfT = nullptr, *dWf, *dcdh,
-            *dcdv, *drel, *drcA;
+            *dcdv, *drW;
         TRY(upload(h, &fL, G.faceL));
         TRY(upload(h, &fR, G.faceR));
         TRY(upload(h, &dkd_h, kd_h));
@@ -1568,10 +1571,11 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
         TRY(upload(h, &dWf, Wf));
         TRY(upload(h, &dcdh, cdh));
         TRY(upload(h, &dcdv, cdv));
-        TRY(upload(h, &drel, rel));
-        TRY(upload(h, &drcA, rcA));
+        TRY(dalloc(h, &drW, Wf.size()));
+        k_reciprocal<<<4 * h->nsm, 256>>>(Wf.size(), dWf, drW);
+        CK(cudaGetLastError());
         h->md = mg::MixedDev{ncol0, nlev, nfh, fL, fR, h->lv[0].fof, dsdiv, dkd_h, dkd_v, dwu, dwd, dml, ddivv,
-                             hm.ncf, dcf, dwf, hm.ms, mv, dmlh, dwfT, dWf, dcdh, dcdv, drel, drcA, mixed->eps};
+                             hm.ncf, dcf, dwf, hm.ms, mv, dmlh, dwfT, dWf, dcdh, dcdv, drW, mixed->eps};
         h->nu = (int64_t)nlev * nfh + (int64_t)NV0;
         TRY(dalloc(h, &h->schurB, N0));
         TRY(dalloc(h, &h->mb, (size_t)h->nu + N0));
