@@ -336,7 +336,7 @@ mg_status mg_ensemble_solve(mg_ensemble* e, mg_solve_info* infos, int32_t* statu
 
 void mg_ensemble_destroy(mg_ensemble* e);
 
-/* [yu; yp] = A [u; p], the mixed operator (needs mixed data). */
+/* [yu; yp] = A [u; p], the mixed operator (needs mixed data).  yp may be p; yu must not overlap u or p. */
 mg_status mixed_apply(mg_handle* h, const double* u, const double* p, double* yu, double* yp,
                       void* stream);
 

@@ -2269,8 +2269,15 @@ mg_status mixed_apply(mg_handle* h, const double* u, const double* p, double* yu
     if (!h || !u || !p || !yu || !yp) return MG_ERR_ARG;
     if (!h->mixed) return MG_ERR_UNSUPPORTED;
     DeviceGuard dg(h->device);
-    Prof pr(h, MG_K_MIXED, 0, 8.0 * (2.0 * h->nu + 3.0 * cells(h, 0)), S(stream));
-    return launch_mixed<mg::MX_A, -1>(h, u, p, yu, yp, nullptr, S(stream));
+    cudaStream_t s = S(stream);
+    const bool in_place = yp == p;   // (velocity rows read p of both cells: the pressure rows wait in mx then)
+    double* const to = in_place ? h->mx + h->nu : yp;
+    {
+        Prof pr(h, MG_K_MIXED, 0, 8.0 * (2.0 * h->nu + 3.0 * cells(h, 0)), s);
+        TRY((launch_mixed<mg::MX_A, -1>(h, u, p, yu, to, nullptr, s)));
+    }
+    if (in_place) CK(cudaMemcpyAsync(yp, to, cells(h, 0) * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    return MG_OK;
 }
 
 mg_status schur_precond(mg_handle* h, const double* ru, const double* rp, double* u, double* p, void* stream) {

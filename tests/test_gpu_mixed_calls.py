@@ -60,3 +60,22 @@ def test_the_transposed_mass_costs_three_roundings(mg):
     got = np.abs(yu.cpu().numpy()[one])
     assert np.max(np.abs(got - 1 / 6)) <= 3 * (1 + 2.0 ** -50) * 2.0 ** -53 / 6
     h.destroy()
+
+
+@pytest.mark.parametrize("n,nlev,consistent", [(10, 19, False), (48, 30, True)])
+def test_pressure_rows_in_place(mg, n, nlev, consistent):
+    """mixed_apply with yp = p, and the Schur-complement step in place of its right-hand side, give the bits
+    of separate arrays."""
+    cfg = syn.small_config(n, nlev, levels=1, seed=syn.BASE_SEED + 880, mixed=True, consistent_mass=consistent)
+    inp = syn.make_inputs(cfg)
+    h = mg.mg_setup_config(cfg, inp)
+    u, p = (torch.from_numpy(inp[k]).cuda().ravel() for k in ("rhs_u", "rhs_p"))
+    yu, yp, zu, zp = torch.empty_like(u), torch.empty_like(p), torch.empty_like(u), p.clone()
+    mg.mixed_apply(h, u, p, yu, yp)
+    mg.mixed_apply(h, u, zp, zu, zp)
+    assert torch.equal(yu, zu) and torch.equal(yp, zp)
+    mg.schur_precond(h, u, p, yu, yp)
+    zu, zp = u.clone(), p.clone()
+    mg.schur_precond(h, zu, zp, zu, zp)
+    assert torch.equal(yu, zu) and torch.equal(yp, zp)
+    h.destroy()
