@@ -179,11 +179,15 @@ __global__ void k_coef_grad(Lvl<double, double> L, const double* __restrict__ la
     grad[5 * N + e] = k > 0 ? -l * (x0 - x[e - ncol]) : 0.0;
 }
 
-// Start of a GCR solve: r = b, x = 0, <b, b> and no wait run out yet, in one pass over memory (a copy, a fill and a product before: C192L70
-// solve 10.50 -> 10.45 ms, together with the first iteration launched ahead).
+// Start of a GCR solve: r = b, x = 0, <b, b> and no wait run out yet, in one pass over memory (a copy, a fill and
+// a product before).  <b, b> goes straight to the host, which waits for it before the first iteration: a zero
+// right-hand side costs no more than this (C192L70 98 us).  Launching the first iteration ahead of <b, b>
+// instead: a zero right-hand side 985 us, other solves 342 -> 343 us (C12L30), 711 -> 718 (C48L30), 9.33 -> 9.27 ms
+// (C192L70).
 __global__ void __launch_bounds__(RED_THREADS) k_gcr_start(size_t n, const double* __restrict__ b, double* __restrict__ r,
                                                            double* __restrict__ x, double* partials,
-                                                           unsigned int* ticket, double* bb, unsigned int* timeout) {
+                                                           unsigned int* ticket, double* bb, double* host_bb,
+                                                           unsigned int* timeout) {
     double v[1] = {0.0}, t[1];
     if (blockIdx.x == 0 && threadIdx.x == 0) *timeout = 0u;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -192,7 +196,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_gcr_start(size_t n, const doubl
         x[i] = 0.0;
         v[0] = fma(e, e, v[0]);
     }
-    if (grid_reduce<1>(v, partials, ticket, t)) *bb = t[0];
+    if (grid_reduce<1>(v, partials, ticket, t)) {
+        *bb = t[0];
+        if (host_bb) *host_bb = t[0];   // (pinned; a copy of its own would be one more step before the host knows)
+    }
 }
 
 // ---- BiCGStab for the pressure system (van der Vorst 1992, right-preconditioned) ----

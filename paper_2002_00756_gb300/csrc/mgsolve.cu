@@ -943,10 +943,9 @@ mg_status gcr_start(mg_handle* h, GcrRun& g, const double* b, cudaStream_t s) {
     {
         Prof pr(h, MG_K_DOT, 0, 24.0 * g.n, s);
         mg::k_gcr_start<<<vec_grid(h, g.n), mg::RED_THREADS, 0, s>>>(g.n, b, h->r, g.x, h->partials, h->tickets + TK_DOT,
-                                                                    &h->gs->bb, h->timeout);
+                                                                    &h->gs->bb, h->host_sc + 1, h->timeout);
         CK(cudaGetLastError());
     }
-    CK(cudaMemcpyAsync(h->host_sc + 1, &h->gs->bb, sizeof(double), cudaMemcpyDeviceToHost, s));
     return MG_OK;
 }
 
@@ -1024,20 +1023,12 @@ mg_status gcr(mg_handle* h, int sys, size_t n, const double* b, double* x, doubl
     g.x = x;
     g.tol = tol;
     TRY(gcr_start(h, g, b, s));
-    // The first iteration follows without waiting for <b, b>, which only a zero, infinite or NaN right-hand
-    // side needs first: x stays 0 then and the iteration's outcome is dropped (one host round trip less per
-    // solve: C12L30 350 -> 337 us, C48L30 720 -> 704).  A pressure solver that synchronises could fail on such a right-hand side.
-    bool ahead = h->prm.max_iter > 0 && !(sys != 0 && ps_syncs(h));
-    if (ahead) TRY(gcr_launch(h, g, s, applyAS, applyP));
     CK(cudaStreamSynchronize(s));
     gcr_started(h, g);
     while (g.active) {
         NvtxRange it_("gcr iteration");
-        if (!ahead) {
-            TRY(gcr_launch(h, g, s, applyAS, applyP));
-            CK(cudaStreamSynchronize(s));
-        }
-        ahead = false;
+        TRY(gcr_launch(h, g, s, applyAS, applyP));
+        CK(cudaStreamSynchronize(s));
         TRY(gcr_landed(h, g, s));
     }
     CK(cudaEventRecord(h->ev1, s));
@@ -1705,7 +1696,7 @@ mg_status build_member(mg_ensemble* e, int i, mg_handle* h, const double* b, dou
     std::vector<cudaGraphNode_t> deps;
     CK(cudaStreamBeginCaptureToGraph(e->cs, e->graph, root.data(), nullptr, root.size(), mode));
     mg::k_gcr_start<<<vec_grid(h, n), mg::RED_THREADS, 0, e->cs>>>(n, b, h->r, x, h->partials, h->tickets + TK_DOT,
-                                                                   &h->gs->bb, h->timeout);
+                                                                   &h->gs->bb, nullptr, h->timeout);
     mg::k_ens_init<<<1, 1, 0, e->cs>>>(h->gs, st, R, h->prm.max_iter, hs);
     CK(cudaGetLastError());
     TRY(end_segment(e, deps));
