@@ -33,11 +33,12 @@
 
 namespace mg {
 
-// Columns of a padded row before its first cell, and its length: rows start on 128-byte lines where
-// that costs little memory, on 32-byte sectors on small meshes.
+// Columns before a field's first cell, and the length of a padded row: rows start on 128-byte lines, on
+// 32-byte sectors on small meshes.  A row's east rim and the next row's west rim share the gap between
+// them; tensor boxes reach beyond a row's end into the next row, for lanes that store nothing.
 __host__ __device__ inline int pad_off(int n) { return n >= 48 ? 32 : 8; }
-__host__ __device__ inline int pad_row(int n) { return n >= 48 ? (n + 32 + 4 + 31) / 32 * 32 : (n + 16 + 7) / 8 * 8; }
-__host__ __device__ inline int padded(int n) { return 6 * (n + 2) * pad_row(n); }
+__host__ __device__ inline int pad_row(int n) { return n >= 48 ? (n + 2 + 31) / 32 * 32 : (n + 2 + 7) / 8 * 8; }
+__host__ __device__ inline int padded(int n) { return 6 * (n + 2) * pad_row(n) + pad_off(n); }
 
 // a column's position: panel, row and column in it, and its padded column
 struct Pos {
