@@ -44,6 +44,7 @@ struct DevLevel {
     double *te64 = nullptr, *tn64 = nullptr, *tbw64 = nullptr, *tbs64 = nullptr, *tv64 = nullptr;
     double *e64 = nullptr, *ip64 = nullptr, *pr64 = nullptr;
     double* wA64 = nullptr;      // area x scale
+    bool wants64 = false, packed64 = false;   // somebody uses them; they are those of the face form (ready64)
     // FP32 level data (sweep32.cuh): couplings in FP32 or BF16, reciprocal pivots, 1 / area; the
     // FP64 elimination of MG_FP32_P64's finest level; restriction weights onto the next level
     // [4][ncol_next] (the 9-cell stencil's as well); tensor maps, iterate in x32[0] / x32[1]
@@ -171,6 +172,12 @@ thread_local cudaError_t g_last_cuda = cudaSuccess;
         }                              \
     } while (0)
 
+#define TRY(call)                         \
+    do {                                  \
+        mg_status s_ = (call);            \
+        if (s_ != MG_OK) return s_;       \
+    } while (0)
+
 // Every device and pinned-host allocation of the library goes through mem_alloc / mem_free.
 // They count the live allocations (mg_live_allocations) and carry the failure injection of
 // mg_inject_alloc_failure: with g_fail_at = n > 0, the n-th allocation attempted after the call
@@ -212,6 +219,28 @@ mg_status dalloc(mg_handle* h, P** p, size_t count) {
     return MG_OK;
 }
 
+// Several arrays in one allocation, each from a 256-byte boundary on.
+struct Pieces {
+    struct Piece {
+        void** to;
+        size_t at;
+    };
+    std::vector<Piece> pieces;
+    size_t bytes = 0;
+    template <typename P>
+    void add(P** to, size_t count) {
+        *to = nullptr;
+        pieces.push_back({reinterpret_cast<void**>(to), bytes});
+        bytes += (count * sizeof(P) + 255) / 256 * 256;
+    }
+    mg_status alloc(mg_handle* h) {
+        char* base = nullptr;
+        TRY(dalloc(h, &base, bytes));
+        for (const Piece& p : pieces) *p.to = base + p.at;
+        return MG_OK;
+    }
+};
+
 template <typename P, typename S>
 mg_status upload(mg_handle* h, P** p, const std::vector<S>& src) {
     mg_status st = dalloc(h, p, src.size());
@@ -229,12 +258,6 @@ struct NvtxRange {
     explicit NvtxRange(const char* name) { nvtxRangePushA(name); }
     ~NvtxRange() { nvtxRangePop(); }
 };
-
-#define TRY(call)                         \
-    do {                                  \
-        mg_status s_ = (call);            \
-        if (s_ != MG_OK) return s_;       \
-    } while (0)
 
 inline cudaStream_t S(void* s) { return static_cast<cudaStream_t>(s); }
 
@@ -1168,15 +1191,59 @@ mg_status build_maps(mg_handle* h, int l) {
     return ok ? MG_OK : MG_ERR_CUDA;
 }
 
-// The level data of the sweeps and restrictions from level l's FP64 face form, in every precision the
-// handle holds.
-mg_status pack_level(mg_handle* h, int l, cudaStream_t s) {
+// Memory of level l's FP64 level data, in one piece: a failed call leaves nothing behind.
+mg_status alloc64(mg_handle* h, int l) {
+    DevLevel& d = h->lv[l];
+    const size_t N = cells(h, l), rim = (size_t)h->nlev * 6 * d.n;
+    Pieces p;
+    for (double** q : {&d.te64, &d.tn64, &d.e64, &d.ip64}) p.add(q, N);
+    for (double** q : {&d.tbw64, &d.tbs64}) p.add(q, rim);
+    if (mg::sweep64_levels(h->nlev, d.ncol) == 10) p.add(&d.pr64, (size_t)mg::sweep64_chunks(h->nlev, d.ncol) * d.ncol);
+    p.add(&d.tv64, N + d.ncol);
+    return p.alloc(h);
+}
+
+mg_status pack64(mg_handle* h, int l, cudaStream_t s) {
     DevLevel& d = h->lv[l];
     const dim3 grid((d.ncol + 127) / 128, h->nlev + 1);
     mg::k_pack64<<<grid, 128, 0, s>>>(d.n, d.ncol, h->nlev, d.fof, d.Th64, d.Tv64, d.wA64, h->dz, h->scale, d.te64, d.tn64,
                                       d.tbw64, d.tbs64, d.tv64, d.ip64);
     mg::k_factor64<<<(d.ncol + 63) / 64, 64, 0, s>>>(d.ncol, h->nlev, d.tv64, d.e64, d.ip64, d.pr64,
                                                      mg::sweep64_chunks(h->nlev, d.ncol), h->om0);
+    CK(cudaGetLastError());
+    return MG_OK;
+}
+
+// A handle whose V-cycle is not in FP64 has FP64 level data for mg_smooth, mg_smooth_noalloc and
+// mg_residual_restrict alone (40 of about 300 bytes per cell, C96L70: 0.12 ms for the finest level).  They are
+// packed when one of these first asks, on its stream, and from then on by mg_set_coefficients; levels that
+// mg_smooth_noalloc takes have their memory from set-up, others from that first call.  A call under stream
+// capture records the packing, which has then not run yet.
+mg_status ready64(mg_handle* h, int l, cudaStream_t s) {
+    DevLevel& d = h->lv[l];
+    if (d.packed64) return MG_OK;
+    cudaStreamCaptureStatus cst;
+    CK(cudaStreamIsCapturing(s, &cst));
+    if (!d.tv64) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // (allocation is no work on the stream)
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        const mg_status st = alloc64(h, l);
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        TRY(st);
+    }
+    TRY(pack64(h, l, s));
+    d.wants64 = true;
+    d.packed64 = cst == cudaStreamCaptureStatusNone;
+    return MG_OK;
+}
+
+// The level data of the sweeps and restrictions from level l's FP64 face form, in every precision that
+// is in use.
+mg_status pack_level(mg_handle* h, int l, cudaStream_t s) {
+    DevLevel& d = h->lv[l];
+    d.packed64 = d.wants64;
+    if (d.wants64) TRY(pack64(h, l, s));
+    const dim3 grid((d.ncol + 127) / 128, h->nlev + 1);
     const dim3 halves((d.ncol + 63) / 64, 2);
     if (d.te32) {
         mg::k_pack32<float><<<grid, 128, 0, s>>>(d.n, d.ncol, h->nlev, d.fof, d.Th64, d.Tv64, d.te32, d.tn32, d.tv32);
@@ -1397,11 +1464,8 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
             std::vector<double> wA(G.ncol);
             for (int c = 0; c < G.ncol; ++c) wA[c] = G.area[c] * h->scale;
             TRY(upload(h, &d.wA64, wA));
-            for (double** p : {&d.te64, &d.tn64, &d.e64, &d.ip64}) TRY(dalloc(h, p, Nl));
-            for (double** p : {&d.tbw64, &d.tbs64}) TRY(dalloc(h, p, (size_t)nlev * 6 * G.n));
-            TRY(dalloc(h, &d.tv64, Nl + G.ncol));
-            if (mg::sweep64_levels(nlev, G.ncol) == 10)
-                TRY(dalloc(h, &d.pr64, (size_t)mg::sweep64_chunks(nlev, G.ncol) * G.ncol));
+            d.wants64 = prec == MG_FP64;
+            if (d.wants64 || Nl <= (size_t)MG_NOALLOC_MAX_CELLS) TRY(alloc64(h, l));
             if (prec == MG_FP32) {
                 for (float** p : {&d.te32, &d.tn32}) TRY(dalloc(h, p, Np));
                 TRY(dalloc(h, &d.tv32, Np + mg::padded(G.n)));
@@ -1415,7 +1479,7 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
                     for (double** p : {&d.ipd, &d.md, &d.ed}) TRY(dalloc(h, p, Np));
                 TRY(dalloc(h, &d.hd, 4 * (size_t)G.ncol));
             }
-            if (l + 1 < L) TRY(dalloc(h, &d.par, 5 * (size_t)G.ncol));
+            if (l + 1 < L && prec == MG_FP64) TRY(dalloc(h, &d.par, 5 * (size_t)G.ncol));
         }
         TRY(dalloc(h, &d.x64[0], Nl));
         TRY(dalloc(h, &d.x64[1], Nl));
@@ -2224,6 +2288,7 @@ mg_status mg_smooth(mg_handle* h, int32_t level, const double* b, const double* 
     DeviceGuard dg(h->device);
     cudaStream_t s = S(stream);
     DevLevel& d = h->lv[level];
+    if (!h->nine && sweeps > 0) TRY(ready64(h, level, s));
     const Lvl64 L = lvl64(h, level);
     const size_t n = cells(h, level);
     const double* cur = x_in;
@@ -2244,6 +2309,7 @@ mg_status mg_residual_restrict(mg_handle* h, int32_t level, const double* b, con
     if (level + 1 >= h->L || !b || !x || !bc) return MG_ERR_ARG;
     DeviceGuard dg(h->device);
     if (h->nine) return restrict9<double, double, double>(h, level, x, b, bc, S(stream));
+    TRY(ready64(h, level, S(stream)));
     return launch_restrict64<true>(h, level, x, b, bc, S(stream));
 }
 
@@ -2440,6 +2506,7 @@ extern "C" mg_status mg_smooth_noalloc(mg_handle* h, int32_t level, const double
     double* scratch = nullptr;
     TRY(scratch_address(h->device, &scratch));
     cudaStream_t s = S(stream);
+    if (sweeps > 0) TRY(ready64(h, level, s));
     const Lvl64 L = lvl64(h, level);
     if (sweeps == 0) {
         if (!x_in) CK(cudaMemsetAsync(x_out, 0, n * sizeof(double), s));

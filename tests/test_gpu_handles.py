@@ -37,3 +37,60 @@ def test_padding_of_the_fp32_fields(mg):
     panel: 52 times 1.547.  248 in all, and 20 allocations of which a 2 MB page may be partly used."""
     used, cells = device_bytes(mg, 64, 80, "fp32_p64")
     assert used <= (24 + 16 + 56 + 32 + 40 + 52 * 1.547) * cells + 20 * 2 ** 21, used / cells
+
+
+def test_large_fp32_levels_hold_fp64_data_on_demand(mg):
+    """C128L30, 2.9M cells, restart 1: 24 + 16 + 56 + 32 bytes per cell and seven FP32 fields padded by 1.27,
+    without the 40 of the FP64 level data; 20 allocations as above."""
+    used, cells = device_bytes(mg, 128, 30, "fp32")
+    assert used <= (24 + 16 + 56 + 32 + 28 * 1.27) * cells + 20 * 2 ** 21, used / cells
+
+
+@pytest.mark.parametrize("n,nlev", [(24, 30), (128, 30)])
+def test_fp64_calls_of_an_fp32_handle(mg, n, nlev):
+    """mg_smooth and mg_residual_restrict of an FP32 handle give the bits of an FP64 handle's: at their first call,
+    first captured into a graph and called eagerly before and after it is replayed, and after other
+    couplings have been set, by the graph as well."""
+    cfg = syn.small_config(n, nlev, levels=2, seed=syn.BASE_SEED + 910)
+    inp = syn.make_inputs(cfg)
+    h = [mg.mg_setup_config(cfg, inp, precision=p) for p in ("fp64", "fp32", "fp32")]
+    b, x0 = torch.from_numpy(inp["rhs"]).cuda().ravel(), torch.from_numpy(syn.normal(9, 0, cfg.ncell)).cuda()
+
+    def calls(hd):
+        x, bc = torch.empty_like(b), torch.empty(hd.level_cells(1), dtype=torch.float64, device="cuda")
+        mg.mg_smooth(hd, 0, b, x0, x, 2)
+        mg.mg_residual_restrict(hd, 0, b, x, bc)
+        return x, bc
+
+    def same(u, v):
+        return all(torch.equal(s, t) for s, t in zip(u, v))
+
+    ref = calls(h[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = calls(h[1])
+    assert same(calls(h[1]), ref)          # (nothing of the graph has run)
+    graph.replay()
+    assert same(out, ref) and same(calls(h[1]), ref) and same(calls(h[2]), ref)
+    # couplings of another operator: unit ones weighted by the cells' own volumes
+    z = np.asarray(inp["z_if"])
+    dz = torch.from_numpy(np.diff(z)).cuda()
+    area = torch.from_numpy(areas(mg, cfg)).cuda()
+    a = torch.zeros((6, cfg.nlev, cfg.ncol), dtype=torch.float64, device="cuda")
+    a[:4] = 1e10 / area
+    a[4, :-1] = 300.0 / dz[:-1, None]
+    a[5, 1:] = 300.0 / dz[1:, None]
+    for hd in h:
+        mg.mg_set_coefficients(hd, a.ravel())
+    other = calls(h[0])
+    assert not same(other, ref)
+    graph.replay()
+    assert same(out, other) and same(calls(h[1]), other) and same(calls(h[2]), other)
+    for hd in h:
+        hd.destroy()
+
+
+def areas(mg, cfg):
+    from oracle.geometry import Mesh
+    return np.asarray(Mesh(cfg.n, syn.make_inputs(cfg)["z_if"], cfg.radius).area).ravel()
