@@ -1445,15 +1445,22 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
         const mg::HGeom& G = hg[l];
         d.n = G.n;
         d.ncol = G.ncol;
-        std::vector<double> rA(G.ncol);
-        for (int c = 0; c < G.ncol; ++c) rA[c] = 1.0 / G.area[c];
-        TRY(upload(h, &d.nbr, G.nbr));
-        TRY(upload(h, &d.fof, G.face_of));
-        TRY(upload(h, &d.rA64, rA));
+        std::vector<double> rA(G.ncol), columns(2 * (size_t)G.ncol);   // 1 / area; that and area x scale
+        for (int c = 0; c < G.ncol; ++c) {
+            columns[c] = rA[c] = 1.0 / G.area[c];
+            columns[G.ncol + c] = G.area[c] * h->scale;
+        }
+        std::vector<int32_t> sides(G.nbr);   // neighbours, then faces
+        sides.insert(sides.end(), G.face_of.begin(), G.face_of.end());
+        TRY(upload(h, &d.nbr, sides));
+        d.fof = d.nbr + G.nbr.size();
+        TRY(upload(h, &d.rA64, columns));
+        d.wA64 = d.rA64 + G.ncol;
         TRY(upload(h, &d.Th64, co[l].Th));
         TRY(upload(h, &d.Tv64, co[l].Tv));
         const size_t Nl = (size_t)nlev * G.ncol;
         const size_t Np = gamma2 > 0.0 ? Nl : (size_t)nlev * mg::padded(G.n);   // an FP32 field
+        Pieces own;   // (arrays that set-up does not upload: small handles' set-up is mostly allocations)
         if (prec != MG_FP64) TRY(upload(h, &d.rA32, rA));
         if (gamma2 > 0.0) {
             if (prec != MG_FP64) {
@@ -1461,37 +1468,32 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
                 TRY(upload(h, &d.Tv32, co[l].Tv));
             }
         } else {
-            std::vector<double> wA(G.ncol);
-            for (int c = 0; c < G.ncol; ++c) wA[c] = G.area[c] * h->scale;
-            TRY(upload(h, &d.wA64, wA));
             d.wants64 = prec == MG_FP64;
             if (d.wants64 || Nl <= (size_t)MG_NOALLOC_MAX_CELLS) TRY(alloc64(h, l));
             if (prec == MG_FP32) {
-                for (float** p : {&d.te32, &d.tn32}) TRY(dalloc(h, p, Np));
-                TRY(dalloc(h, &d.tv32, Np + mg::padded(G.n)));
+                for (float** p : {&d.te32, &d.tn32}) own.add(p, Np);
+                own.add(&d.tv32, Np + mg::padded(G.n));
             } else if (prec == MG_FP32_BF16COEF) {
-                for (bf16** p : {&d.te16, &d.tn16}) TRY(dalloc(h, p, Np));
-                TRY(dalloc(h, &d.tv16, Np + mg::padded(G.n)));
+                for (bf16** p : {&d.te16, &d.tn16}) own.add(p, Np);
+                own.add(&d.tv16, Np + mg::padded(G.n));
             }
             if (prec != MG_FP64) {
-                TRY(dalloc(h, &d.ip32, Np));
+                own.add(&d.ip32, Np);
                 if (l == 0 && prm->vcycle_precision == MG_FP32_P64)
-                    for (double** p : {&d.ipd, &d.md, &d.ed}) TRY(dalloc(h, p, Np));
-                TRY(dalloc(h, &d.hd, 4 * (size_t)G.ncol));
+                    for (double** p : {&d.ipd, &d.md, &d.ed}) own.add(p, Np);
+                own.add(&d.hd, 4 * (size_t)G.ncol);
             }
-            if (l + 1 < L && prec == MG_FP64) TRY(dalloc(h, &d.par, 5 * (size_t)G.ncol));
+            if (l + 1 < L && prec == MG_FP64) own.add(&d.par, 5 * (size_t)G.ncol);
         }
-        TRY(dalloc(h, &d.x64[0], Nl));
-        TRY(dalloc(h, &d.x64[1], Nl));
+        for (double*& p : d.x64) own.add(&p, Nl);
         // right-hand sides and, below the finest level, the iterate that goes up
         if (prec == MG_FP64) {
-            TRY(dalloc(h, &d.b64, Nl));
-            if (l > 0) TRY(dalloc(h, &d.r64, Nl));
+            own.add(&d.b64, Nl);
+            if (l > 0) own.add(&d.r64, Nl);
         } else {
-            TRY(dalloc(h, &d.x32[0], Np));
-            TRY(dalloc(h, &d.x32[1], Np));
-            TRY(dalloc(h, &d.b32, Np));
-            if (l > 0) TRY(dalloc(h, &d.r32, Np));
+            for (float*& p : d.x32) own.add(&p, Np);
+            own.add(&d.b32, Np);
+            if (l > 0) own.add(&d.r32, Np);
         }
         if (gamma2 > 0.0) {
             // 9-cell stencil: flux between cells k and k + 2 of every column,
@@ -1508,12 +1510,13 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
                         dzc2;
             }
             TRY(upload(h, &d.T2_64, t2));
-            for (double*& p : d.s64) TRY(dalloc(h, &p, Nl));
+            for (double*& p : d.s64) own.add(&p, Nl);
             if (prec == MG_FP32) {
                 TRY(upload(h, &d.T2_32, t2));
-                for (float*& p : d.s32) TRY(dalloc(h, &p, Nl));
+                for (float*& p : d.s32) own.add(&p, Nl);
             }
         }
+        TRY(own.alloc(h));
         if (l + 1 < L) {
             const mg::HGeom& Gc = hg[l + 1];
             std::vector<double> w(4 * (size_t)Gc.ncol);

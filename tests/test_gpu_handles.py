@@ -94,3 +94,18 @@ def test_fp64_calls_of_an_fp32_handle(mg, n, nlev):
 def areas(mg, cfg):
     from oracle.geometry import Mesh
     return np.asarray(Mesh(cfg.n, syn.make_inputs(cfg)["z_if"], cfg.radius).area).ravel()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32_bf16"])
+def test_a_level_takes_few_allocations(mg, precision):
+    """Set-up of a small handle is mostly allocations and uploads.  A level's: connectivity, column factors,
+    two face forms, FP32 column factors and restriction weights, FP64 level data, and one for all else."""
+    lib, count = mg.load(), []
+    for levels in (2, 3):
+        cfg = syn.small_config(12, 10, levels=levels, seed=syn.BASE_SEED + 920)
+        inp = syn.make_inputs(cfg)
+        lib.mg_inject_alloc_failure(0)
+        h = mg.mg_setup_config(cfg, inp, precision=precision)
+        count.append(lib.mg_inject_alloc_failure(0))
+        h.destroy()
+    assert count[1] - count[0] <= 8, count
