@@ -114,29 +114,27 @@ __device__ __forceinline__ bool coef_agree(double u, double v) {
     return u >= 0.0 && v >= 0.0 && isfinite(u) && isfinite(v) && fabs(u - v) <= 1e-10 * fmax(fabs(u), fabs(v));
 }
 
+// horizontal face f of level k
 template <bool WRITE>
-__global__ void k_coef_faces(int ncol, int nlev, const int32_t* __restrict__ faceL, const int32_t* __restrict__ faceR,
-                             const int32_t* __restrict__ faceSide, const int32_t* __restrict__ nbrSide,
-                             const double* __restrict__ area, const double* __restrict__ a, double* __restrict__ Th,
-                             unsigned int* bad) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y, nf = 2 * ncol;
-    if (f >= nf || k >= nlev) return;
+__device__ __forceinline__ void coef_face(int f, int k, int ncol, int nlev, const int32_t* __restrict__ faceL,
+                                          const int32_t* __restrict__ faceR, const int32_t* __restrict__ faceSide,
+                                          const int32_t* __restrict__ nbrSide, const double* __restrict__ area,
+                                          const double* __restrict__ a, double* __restrict__ Th, unsigned int* bad) {
     const size_t N = (size_t)nlev * ncol, o = (size_t)k * ncol;
     const int L = faceL[f], s = faceSide[f];
     const double tl = a[s * N + o + L] * area[L];
     if (WRITE) {
-        Th[(size_t)k * nf + f] = tl;
+        Th[(size_t)k * 2 * ncol + f] = tl;
     } else {
         const int R = faceR[f], sr = nbrSide[s * ncol + L];
         if (!coef_agree(tl, a[sr * N + o + R] * area[R])) atomicOr(bad, 1u);
     }
 }
 
+// vertical face kf of column c
 template <bool WRITE>
-__global__ void k_coef_vertical(int ncol, int nlev, const double* __restrict__ dz, const double* __restrict__ a,
-                                double* __restrict__ Tv, unsigned int* bad) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x, kf = blockIdx.y;
-    if (c >= ncol || kf > nlev) return;
+__device__ __forceinline__ void coef_vertical(int c, int kf, int ncol, int nlev, const double* __restrict__ dz,
+                                              const double* __restrict__ a, double* __restrict__ Tv, unsigned int* bad) {
     const size_t N = (size_t)nlev * ncol;
     if (WRITE) {
         Tv[(size_t)kf * ncol + c] = kf == 0 || kf == nlev ? 0.0 : a[4 * N + (size_t)(kf - 1) * ncol + c] * dz[kf - 1];
@@ -152,16 +150,32 @@ __global__ void k_coef_vertical(int ncol, int nlev, const double* __restrict__ d
 }
 
 // a6[s][e] = a[s][e] (s < 6) and a6[6][e] = 1 + their sum: the FP64 operator of the GCR apply
-__global__ void k_coef_cells(size_t N, const double* __restrict__ a, double* __restrict__ a6) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < N; e += (size_t)gridDim.x * blockDim.x) {
-        double d = 1.0;
+__device__ __forceinline__ void coef_cell(size_t e, size_t N, const double* __restrict__ a, double* __restrict__ a6) {
+    double d = 1.0;
 #pragma unroll
-        for (int s = 0; s < 6; ++s) {
-            const double v = a[s * N + e];
-            a6[s * N + e] = v;
-            d += v;
-        }
-        a6[6 * N + e] = d;
+    for (int s = 0; s < 6; ++s) {
+        const double v = a[s * N + e];
+        a6[s * N + e] = v;
+        d += v;
+    }
+    a6[6 * N + e] = d;
+}
+
+// One launch for the checks and one for the stores: rows of the grid are the horizontal faces' levels,
+// then the vertical faces', then (WRITE) the cells'.  Small handles' calls are mostly launches and two host
+// round trips: C12L30 FP64 60 us, with a launch per
+// kind, a cleared flag and pageable read-back 78; C30L1 47 and 64.
+template <bool WRITE>
+__global__ void __launch_bounds__(128) k_coef(int ncol, int nlev, const int32_t* __restrict__ faceL, const int32_t* __restrict__ faceR,
+                       const int32_t* __restrict__ faceSide, const int32_t* __restrict__ nbrSide,
+                       const double* __restrict__ area, const double* __restrict__ dz, const double* __restrict__ a,
+                       double* __restrict__ Th, double* __restrict__ Tv, double* __restrict__ a6, unsigned int* bad) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    if (k < nlev) {
+        if (i < 2 * ncol) coef_face<WRITE>(i, k, ncol, nlev, faceL, faceR, faceSide, nbrSide, area, a, Th, bad);
+    } else if (i < ncol) {
+        if (k <= 2 * nlev) coef_vertical<WRITE>(i, k - nlev, ncol, nlev, dz, a, Tv, bad);
+        else if (WRITE) coef_cell((size_t)(k - 2 * nlev - 1) * ncol + i, (size_t)nlev * ncol, a, a6);
     }
 }
 

@@ -1264,30 +1264,21 @@ mg_status pack_level(mg_handle* h, int l, cudaStream_t s) {
 // form in its precision.  A first pass only checks them (flux symmetry, sign, no flux through
 // surface and lid); the operator is changed only if every check passes.
 mg_status set_coefficients_impl(mg_handle* h, const double* a, cudaStream_t s) {
-    const int ncol = h->lv[0].ncol, nlev = h->nlev, nf = 2 * ncol;
+    const int ncol = h->lv[0].ncol, nlev = h->nlev, blocks = (2 * ncol + 127) / 128;
     const DevLevel& d = h->lv[0];
-    CK(cudaMemsetAsync(h->flag, 0, sizeof(unsigned int), s));
-    for (int pass = 0; pass < 2; ++pass) {
-        const bool write = pass == 1;
-        const dim3 gh((nf + 127) / 128, nlev), gv((ncol + 127) / 128, nlev + 1);
-        if (write) {
-            mg::k_coef_faces<true><<<gh, 128, 0, s>>>(ncol, nlev, h->faceL0, h->faceR0, h->faceSide0, h->nbrSide0, h->area0,
-                                                      a, d.Th64, h->flag);
-            mg::k_coef_vertical<true><<<gv, 128, 0, s>>>(ncol, nlev, h->dz, a, d.Tv64, h->flag);
-        } else {
-            mg::k_coef_faces<false><<<gh, 128, 0, s>>>(ncol, nlev, h->faceL0, h->faceR0, h->faceSide0, h->nbrSide0, h->area0,
-                                                       a, d.Th64, h->flag);
-            mg::k_coef_vertical<false><<<gv, 128, 0, s>>>(ncol, nlev, h->dz, a, d.Tv64, h->flag);
-        }
-        CK(cudaGetLastError());
-        if (!write) {
-            unsigned int bad = 0;
-            CK(cudaMemcpyAsync(&bad, h->flag, sizeof bad, cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            if (bad) return MG_ERR_ARG;
-        }
+    mg::k_coef<false><<<dim3(blocks, 2 * nlev + 1), 128, 0, s>>>(ncol, nlev, h->faceL0, h->faceR0, h->faceSide0, h->nbrSide0,
+                                                                 h->area0, h->dz, a, d.Th64, d.Tv64, h->a6, h->flag);
+    CK(cudaGetLastError());
+    unsigned int* const bad = reinterpret_cast<unsigned int*>(h->host_sc + 2);
+    CK(cudaMemcpyAsync(bad, h->flag, sizeof *bad, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    if (*bad) {
+        CK(cudaMemsetAsync(h->flag, 0, sizeof *h->flag, s));   // (clear at the start of every call)
+        CK(cudaStreamSynchronize(s));
+        return MG_ERR_ARG;
     }
-    mg::k_coef_cells<<<4 * h->nsm, 256, 0, s>>>(cells(h, 0), a, h->a6);
+    mg::k_coef<true><<<dim3(blocks, 3 * nlev + 1), 128, 0, s>>>(ncol, nlev, h->faceL0, h->faceR0, h->faceSide0, h->nbrSide0,
+                                                                h->area0, h->dz, a, d.Th64, d.Tv64, h->a6, h->flag);
     CK(cudaGetLastError());
     TRY(pack_level(h, 0, s));
     CK(cudaStreamSynchronize(s));
@@ -1436,6 +1427,7 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
     TRY(upload(h, &h->nbrSide0, hg[0].nbr_side));
     TRY(dalloc(h, &h->flag, 1));
     TRY(dalloc(h, &h->timeout, 1));
+    CK(cudaMemset(h->flag, 0, sizeof(unsigned int)));
     CK(cudaMemset(h->timeout, 0, sizeof(unsigned int)));
     // MG_FP32_P64 stores and computes as MG_FP32; only the finest level's elimination differs
     const int prec = prm->vcycle_precision == MG_FP32_P64 ? MG_FP32 : prm->vcycle_precision;

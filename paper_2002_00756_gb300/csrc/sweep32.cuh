@@ -466,32 +466,52 @@ __global__ void k_pack32(int n, int ncol, int nlev, const int32_t* __restrict__ 
 }
 
 // The pivots of both halves of every column: ip (1 / p; q at a half's last step) and, for an FP64
-// elimination, the multipliers m and e.  One thread per column and half (blockIdx.y).
+// elimination, the multipliers m and e.  One thread per column and half (blockIdx.y); the next BATCH
+// steps' operands are under way while a batch is eliminated (as in k_factor64; with k_pack32 at C24L128 46 -> 25 us).
 template <typename C, typename P>
 __global__ void k_factor32(Lvl32<C, P> L, P* __restrict__ ip_, P* __restrict__ m_, P* __restrict__ e_) {
+    constexpr int BATCH = 8;
     const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= (unsigned)L.ncol) return;
     const bool up = blockIdx.y;
     const int nlev = L.nlev, hs = (nlev + 1) >> 1, ns = up ? nlev - hs : hs;
+    if (c >= (unsigned)L.ncol || ns == 0) return;
     const unsigned np = L.np, ncolp = L.ncolp;
     const Pos at(c, L.n, np);
     const float rA = __ldg(L.rA + c);
+    auto level = [&](int s) { return (unsigned)(up ? nlev - 1 - s : s); };
+    float H[BATCH], T[BATCH], Z[BATCH], Hn[BATCH], Tn[BATCH], Zn[BATCH];   // horizontal sum, face ahead, 1 / dz
+    auto load = [&](int s0) {
+#pragma unroll
+        for (int q = 0; q < BATCH; ++q) {
+            const unsigned k = level(min(s0 + q, ns - 1)), o = k * ncolp + at.cp;
+            Hn[q] = addr(addr(ldf(L.te + o), ldf(L.te + (o - 1))), addr(ldf(L.tn + o), ldf(L.tn + (o - np))));
+            Tn[q] = ldf(L.tv + ((up ? k : k + 1) * ncolp + at.cp));
+            Zn[q] = __ldg(L.rdz + k);
+        }
+    };
+    load(0);
     P q = P(0), ip = P(0);
     float tb = 0.f;
-#pragma unroll 4
-    for (int s = 0; s < ns; ++s) {
-        const unsigned k = up ? nlev - 1 - s : s, o = k * ncolp + at.cp;
-        const float te = ldf(L.te + o), tw = ldf(L.te + (o - 1)), tn = ldf(L.tn + o), ts = ldf(L.tn + (o - np));
-        const float ta = ldf(L.tv + ((up ? k : k + 1) * ncolp + at.cp)), rdz = __ldg(L.rdz + k);
-        const P an = mulr(P(rdz), P(ta)), m = mulr(mulr(P(rdz), P(tb)), ip);
-        q = fmad(m, q, fmad(P(rA), P(addr(addr(te, tw), addr(tn, ts))), P(1)));
-        ip = P(1) / (q + an);
-        ip_[o] = s == ns - 1 ? q : ip;
-        if (sizeof(P) == 8) {
-            m_[o] = m;
-            e_[o] = mulr(an, ip);
+    for (int s0 = 0; s0 < ns; s0 += BATCH) {
+#pragma unroll
+        for (int i = 0; i < BATCH; ++i) H[i] = Hn[i], T[i] = Tn[i], Z[i] = Zn[i];
+        if (s0 + BATCH < ns) load(s0 + BATCH);
+#pragma unroll
+        for (int i = 0; i < BATCH; ++i) {
+            const int s = s0 + i;
+            if (s < ns) {
+                const unsigned o = level(s) * ncolp + at.cp;
+                const P an = mulr(P(Z[i]), P(T[i])), m = mulr(mulr(P(Z[i]), P(tb)), ip);
+                q = fmad(m, q, fmad(P(rA), P(H[i]), P(1)));
+                ip = P(1) / (q + an);
+                ip_[o] = s == ns - 1 ? q : ip;
+                if (sizeof(P) == 8) {
+                    m_[o] = m;
+                    e_[o] = mulr(an, ip);
+                }
+                tb = T[i];
+            }
         }
-        tb = ta;
     }
 }
 

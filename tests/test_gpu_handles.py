@@ -109,3 +109,27 @@ def test_a_level_takes_few_allocations(mg, precision):
         count.append(lib.mg_inject_alloc_failure(0))
         h.destroy()
     assert count[1] - count[0] <= 8, count
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_a_refused_set_of_couplings_leaves_no_trace(mg, precision):
+    """The check's flag is cleared by the call that found it set, not at the start of every call."""
+    cfg = syn.small_config(6, 5, levels=2, seed=syn.BASE_SEED + 930)
+    inp = syn.make_inputs(cfg)
+    h = mg.mg_setup_config(cfg, inp, precision=precision)
+    good = torch.zeros((6, cfg.nlev, cfg.ncol), dtype=torch.float64, device="cuda")
+    b = torch.from_numpy(inp["rhs"]).cuda().ravel()
+    ref, x = torch.empty_like(b), torch.empty_like(b)
+    mg.vcycle(h, b, ref)
+    for s, k, c in ((0, 2, 5), (4, 4, 3), (5, 0, 7)):
+        bad = good.clone()
+        bad[s, k, c] = 1.0      # a flux from one side only, through the lid, through the surface
+        with pytest.raises(mg.MGError) as e:
+            mg.mg_set_coefficients(h, bad.ravel())
+        assert e.value.status == mg.MG_ERR_ARG
+        mg.vcycle(h, b, x)
+        assert torch.equal(x, ref)
+    mg.mg_set_coefficients(h, good.ravel())
+    mg.helmholtz_apply(h, b, x)
+    assert torch.equal(x, b)
+    h.destroy()
