@@ -152,28 +152,35 @@ struct Chunk {
 //   xo: padded FP32 iterate, or the caller's FP64 array.
 // (chunks of 8 for columns of more than 80 levels: at most 8 chunks a half, whose barriers are the
 // block's 16)
-__host__ __device__ constexpr int sweep32_warps(int K) { return K == 8 ? 16 : 2 * ((40 + K - 1) / K); }
+__host__ __device__ constexpr int sweep32_warps(int K) { return K < 5 ? 2 : K == 8 ? 16 : 2 * ((40 + K - 1) / K); }
+
+// Groups of 32 columns per block: short columns, whose halves are a warp each, take four (blocks of two warps
+// start too slowly: FP32 V-cycle of C256L6 on three levels 250 -> 153 us, of C192L4 140 -> 112).
+__host__ __device__ constexpr int sweep32_groups(int K) { return K < 5 ? 4 : 1; }
 
 // Two warps meet: both wait, so that the two uses of a barrier (forwards, backwards) cannot mix; the
 // receiving warp is there first as a rule.
 __device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 
 template <typename C, typename P, int MODE, typename B, typename O, bool BRAW, int K>
-__global__ void __launch_bounds__(32 * sweep32_warps(K), sizeof(P) == 8 || K != 10 ? 1 : 3)
+__global__ void __launch_bounds__(32 * sweep32_warps(K) * sweep32_groups(K), sizeof(P) == 8 || K != 10 ? 1 : 3)
     k_sweep32(Lvl32<C, P> L, const float* __restrict__ x, const float* __restrict__ xc, const B* __restrict__ b,
               float* __restrict__ bcopy, O* __restrict__ xo, float omega) {
     constexpr bool PRO = (MODE == XM_PROLONG || MODE == XM_PROLONG0);
     constexpr bool RAW = (MODE == XM_PLAIN || MODE == XM_PROLONG);   // reads the fine iterate
     constexpr bool ZERO = MODE == XM_ZERO, PADO = sizeof(O) == 4;
     __shared__ P sy[sweep32_warps(K)][32];   // handed-on y, then (halves' ends) the interface's values
-    __shared__ P si[2][3][32];
+    constexpr int M = sweep32_groups(K);
+    __shared__ P si_[M][2][3][32];
     __shared__ float so[sweep32_warps(K)][32];   // handed-back out
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, G = blockDim.x >> 6;
+    const int lane = threadIdx.x & 31, group = M > 1 ? threadIdx.x >> 6 : 0;
+    const int w = (threadIdx.x >> 5) - 2 * group, G = M > 1 ? 1 : blockDim.x >> 6;
+    P(&si)[2][3][32] = si_[group];
     const bool up = w >= G;   // the upper half, walked downwards
     const int u = up ? w - G : w;
     const int nlev = L.nlev, hs = (nlev + 1) >> 1, ns = up ? nlev - hs : hs;
     const unsigned ncol = L.ncol, n = L.n, np = L.np, ncolp = L.ncolp;
-    const unsigned c_raw = blockIdx.x * 32 + lane;
+    const unsigned c_raw = (blockIdx.x * M + group) * 32 + lane;
     const bool active = c_raw < ncol;
     const unsigned c = active ? c_raw : ncol - 1;
     const int s0 = u * ns / G, len = (u + 1) * ns / G - s0;
@@ -228,7 +235,9 @@ __global__ void __launch_bounds__(32 * sweep32_warps(K), sizeof(P) == 8 || K != 
             if (BRAW && active && j < len) bcopy[o] = bk;
             const float ta = ldf(L.tv + ((up ? k : k + 1) * ncolp + at.cp)), rdz = __ldg(L.rdz + k);
             q.ip[j] = __ldg(L.ip + o);
-            if constexpr (sizeof(P) == 8) {
+            if constexpr (K == 1) {   // (a half's only step: nothing behind it, and out does not need e)
+                q.m[j] = q.e[j] = P(0);
+            } else if constexpr (sizeof(P) == 8) {
                 q.m[j] = __ldg(L.m + o);
                 q.e[j] = __ldg(L.e + o);
             } else {
@@ -294,7 +303,7 @@ __global__ void __launch_bounds__(32 * sweep32_warps(K), sizeof(P) == 8 || K != 
         si[up][0][lane] = ql;
         si[up][1][lane] = y;
         si[up][2][lane] = an;
-        pair_sync(2 * G - 1);
+        pair_sync(2 * G - 1 + group);
         // (a single level: nothing above, and p = q + a_next)
         const P dlt = nlev == 1 ? mulr(y, P(1) / (ql + an))
                                 : interface32(ql, y, an, si[!up][0][lane], si[!up][1][lane], si[!up][2][lane]);

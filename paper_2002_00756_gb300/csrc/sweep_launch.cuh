@@ -16,14 +16,25 @@ constexpr double SMALL_CELLS = 2e6;
 
 template <typename C, typename P, int MODE, typename B, typename O, bool BRAW, int K>
 cudaError_t go(const SweepCall32<C, P>& q, cudaStream_t s) {
+    constexpr int M = sweep32_groups(K);   // (G is 1 where M is not)
     const int G = ((q.L.nlev + 1) / 2 + K - 1) / K;
-    k_sweep32<C, P, MODE, B, O, BRAW, K><<<(q.L.ncol + 31) / 32, 64 * G, 0, s>>>(
+    k_sweep32<C, P, MODE, B, O, BRAW, K><<<(q.L.ncol + 32 * M - 1) / (32 * M), 64 * G * M, 0, s>>>(
         q.L, q.x, q.xc, static_cast<const B*>(q.b), q.bcopy, static_cast<O*>(q.xo), (float)q.omega);
     return cudaGetLastError();
 }
 
+// The short columns' chunk is a whole half: with 5 or 10 steps for one or three, the steps past its end cost
+// more than the chunk (V-cycle, FP32 / FP64 elimination, 64 threads a block: C192L1 160 / 310 us with 5, 127 / 179
+// with 1; C192L4 165 / 340 and 142 / 245 with 2; C256L6 463 / 899 with 10, 299 / 606 with 5, 268 / 484 with 3).
 template <typename C, typename P, int MODE, typename B, typename O, bool BRAW>
 cudaError_t shape(const SweepCall32<C, P>& q, cudaStream_t s) {
+    switch ((q.L.nlev + 1) / 2) {
+        case 1: return go<C, P, MODE, B, O, BRAW, 1>(q, s);
+        case 2: return go<C, P, MODE, B, O, BRAW, 2>(q, s);
+        case 3: return go<C, P, MODE, B, O, BRAW, 3>(q, s);
+        case 4: return go<C, P, MODE, B, O, BRAW, 4>(q, s);
+        default: break;
+    }
     if (q.L.nlev > 80) return go<C, P, MODE, B, O, BRAW, TALL_K>(q, s);
     if ((double)q.L.nlev * q.L.ncol < SMALL_CELLS) return go<C, P, MODE, B, O, BRAW, SMALL_K>(q, s);
     return go<C, P, MODE, B, O, BRAW, BIG_K>(q, s);
