@@ -381,7 +381,7 @@ mg_status mixed_coefficient_gradient(mg_handle* h, const double* lam_u, const do
                                      double* grad_g, double* grad_beta_up, double* grad_beta_dn, void* stream);
 
 /* Autotuner of the column tiles: for every multigrid level, times the candidate forms of the
- * block-Jacobi sweep (FP32 V-cycles: register chunks, or tensor-copy tiles for 8 to 80 levels) and
+ * block-Jacobi sweep (FP32 V-cycles: register chunks, or tensor-copy tiles for 8 levels or more) and
  * of the residual + restriction (the built-in levels per thread, and 4, 8, 16, 24, 35 or 70) with CUDA events around
  * every launch of full V-cycles on the handle's own buffers, and keeps the fastest per
  * level for every later call.  Every form gives the same result bit for bit (each output

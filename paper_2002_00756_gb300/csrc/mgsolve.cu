@@ -364,7 +364,13 @@ mg_status launch_apply(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, Y*
 //   columns of more than 40 levels, whose chunks fill an SM with one block, 250k: C32L50 74.0/28.2 and 72.7/25.5,
 //   C32L70 94/35 and 88/32, C48L41 89/52 and 86/41 (C48L50 92.9/55 and 94.9/50; C24L70, 242k: 92.9 and 93.7);
 //   up to 40 levels, 700k: C64L30 81/47 and 80/42 (C56L30, 564k: 71 and 78; C48L37 77/34 and 81/36).
-inline bool tma_level(int nlev, int ncol) { return (double)nlev * ncol >= (nlev > 40 ? 2.5e5 : 7e5); }
+// C48L50 alone is 2 us slower for it; what decides there is the throughput beside other solves.
+//   more than 80 levels, one block of tiles per SM, 2M: C128L100 778 and 537 (alone; before the chunks 725),
+//   C192L100 1467 and 1050 (1333), C64L128 324 and 274, C80L100 365 and 335; C48L100, 1.4M: 190 and 195,
+//   C48L81 166 and 178.
+inline bool tma_level(int nlev, int ncol) {
+    return (double)nlev * ncol >= (nlev > 80 ? 2e6 : nlev > 40 ? 2.5e5 : 7e5);
+}
 
 // Grid of a vector pass with or without a reduction: two elements per thread until the GPU is full (C12L30's
 // <b, b>: 8.8 us; one per thread 10.6; C192L70's orthogonalisations 121 us on average, with 6, 16 or 32 blocks
@@ -457,7 +463,9 @@ mg_status launch_sweep32(mg_handle* h, int lev, const float* x, const float* xc,
     Prof pr(h, MG_K_SWEEP, lev, (double)L.nlev * L.ncol * per, s, mode);
     const mg::SweepMaps* maps = nullptr;
     const bool tiles = d.sweep_bd > 0 ? d.sweep_bd == 128 : tma_level(L.nlev, L.ncol);
-    if (tiles && d.maps.size() == 2 && mode != mg::XM_PROLONG0) maps = &d.maps[x == d.x32[1]];
+    // (an FP64 elimination's chunks of taller columns have no room beside the boxes)
+    const bool has = mode != mg::XM_PROLONG0 && (sizeof(P) == 4 || L.nlev <= mg::tma_max_levels(8));
+    if (tiles && has && d.maps.size() == 2) maps = &d.maps[x == d.x32[1]];
     const mg::SweepCall32<C, P> q{L, mode, x, xc, b, raw, bcopy, xo, out64, om, maps, h->nsm, h->polls, h->timeout};
     CK((mg::sweep32_run<C, P>(q, s)));
     if (L.n == 1 && !out64) {   // (a C1 column has several edges on one axis)
@@ -1145,12 +1153,11 @@ __global__ void k_parents(int n, int ncol, const int32_t* __restrict__ nbr, int3
     if (c < ncol) par[(size_t)s * ncol + c] = mg::parent_col(s < 4 ? nbr[(size_t)s * ncol + c] : c, n);
 }
 
-// Tensor maps of the TMA sweep (sweep_tma.cuh) for an FP32 level of 8 to 80 levels (two blocks'
-// boxes per SM).
+// Tensor maps of the TMA sweep (sweep_tma.cuh) for an FP32 level of 8 levels or more.
 mg_status build_maps(mg_handle* h, int l) {
     DevLevel& d = h->lv[l];
     d.maps.clear();
-    if (h->nine || !d.ip32 || h->nlev < 8 || h->nlev > 80) return MG_OK;
+    if (h->nine || !d.ip32 || h->nlev < 8) return MG_OK;
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult found;
     CK(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found));

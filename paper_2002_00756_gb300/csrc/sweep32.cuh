@@ -163,7 +163,7 @@ __host__ __device__ constexpr int sweep32_groups(int K) { return K < 5 ? 4 : 1; 
 __device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 
 template <typename C, typename P, int MODE, typename B, typename O, bool BRAW, int K>
-__global__ void __launch_bounds__(32 * sweep32_warps(K) * sweep32_groups(K), sizeof(P) == 8 || K != 10 ? 1 : 3)
+__global__ void __launch_bounds__(32 * sweep32_warps(K) * sweep32_groups(K), sizeof(P) == 8 ? 1 : K == 10 ? 3 : K == 8 && MODE == XM_ZERO ? 2 : 1)
     k_sweep32(Lvl32<C, P> L, const float* __restrict__ x, const float* __restrict__ xc, const B* __restrict__ b,
               float* __restrict__ bcopy, O* __restrict__ xo, float omega) {
     constexpr bool PRO = (MODE == XM_PROLONG || MODE == XM_PROLONG0);

@@ -38,8 +38,9 @@ constexpr int TMA_COLS = 32;
 // Resident blocks per SM that the registers are capped for: two where shared memory allows no more, and
 // for a caller's right-hand side read ahead in registers (three: 91 us instead of 72 at C192L70, spills);
 // three for the other sweeps from zero (17 us instead of 19 on C96L70).
-__host__ __device__ constexpr int tma_blocks(int mode, bool braw, int psize) {
-    return mode == XM_ZERO && !braw && psize == 4 ? 3 : 2;
+// One for columns of more than 80 levels (chunks of 10), whose boxes take up to 190 KB.
+__host__ __device__ constexpr int tma_blocks(int mode, bool braw, int psize, int K) {
+    return K == 10 ? 1 : mode == XM_ZERO && !braw && psize == 4 ? 3 : 2;
 }
 
 template <typename C>
@@ -88,7 +89,7 @@ __device__ __forceinline__ void tma_load(void* dst, const CUtensorMap* m, int x,
 // remaining tiles all the same, because the other group's interface waits for them, and give NaN, which
 // the interface hands to the other half of the column.  Before they leave they wait once more, with the
 // default limit, for the copies in flight, and report.
-__host__ __device__ constexpr int tma_max_levels(int K) { return K == 7 ? 70 : 80; }
+__host__ __device__ constexpr int tma_max_levels(int K) { return K == 7 ? 70 : K == 8 ? 80 : 128; }
 __host__ __device__ constexpr int tma_chunks(int nlev, int K) { return ((nlev + 1) / 2 + K - 1) / K; }
 __host__ __device__ constexpr int tma_threads(int K) { return 64 * tma_chunks(tma_max_levels(K), K); }
 
@@ -140,7 +141,7 @@ struct TmaLayout {
 // ahead; its FP32 copy is stored in bcopy.  P = double: the FP64 pivots and multipliers are read
 // directly as well (their boxes would leave room for one block per SM only).
 template <typename C, typename P, int MODE, typename O, bool BRAW, int K, bool FULL>
-__global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(P)))
+__global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(P), K))
     k_sweep_tma(const __grid_constant__ SweepMaps M, Lvl32<C, P> L, const double* __restrict__ braw,
                 float* __restrict__ bcopy, O* __restrict__ xo, float omega, int tiles_row, int tile_w,
                 int polls, unsigned int* __restrict__ timeout) {

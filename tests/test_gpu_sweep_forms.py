@@ -86,3 +86,9 @@ def test_short_columns_cost_no_more_than_longer_ones(mg):
     """C256L6 in chunks cut to its columns against twice the levels (0.8 of
     its time; 1.37 with chunks of 10)."""
     assert vcycle_time(mg, 256, 6) <= 1.0 * vcycle_time(mg, 256, 12)
+
+
+def test_tall_columns_run_on_tiles(mg):
+    """C128L100 against C128L80, 1.25 times the cells: no change to a form of half the rate (1.4
+    times the time; 2.0 on register chunks)."""
+    assert vcycle_time(mg, 128, 100) <= 1.7 * vcycle_time(mg, 128, 80)
