@@ -449,14 +449,14 @@ mg_status launch_restrict64(mg_handle* h, int lev, const double* x, const double
 }
 
 // The same of the FP32 V-cycle (fields padded).  raw: b is the caller's FP64 array, its FP32 copy goes
-// to bcopy.  xo: padded FP32, or FP64 with out64.
+// to bcopy unless that is NULL.  xo: padded FP32, or FP64 with out64.
 template <typename C, typename P>
 mg_status launch_sweep32(mg_handle* h, int lev, const float* x, const float* xc, const void* b, bool raw, float* bcopy,
                          void* xo, bool out64, double om, cudaStream_t s) {
     const Lvl32<C, P> L = lvl32<C, P>(h, lev);
     const DevLevel& d = h->lv[lev];
     const int mode = sweep_mode(x, xc);
-    double per = (raw ? 12.0 : 4.0) + sizeof(C) + (sizeof(P) == 8 ? 24.0 : 4.0) + (out64 ? 8.0 : 4.0);
+    double per = (raw ? (bcopy ? 12.0 : 8.0) : 4.0) + sizeof(C) + (sizeof(P) == 8 ? 24.0 : 4.0) + (out64 ? 8.0 : 4.0);
     if (mode != mg::XM_ZERO) per += 2.0 * sizeof(C);
     if (x) per += 4.0;
     if (xc) per += 1.0;
@@ -602,11 +602,10 @@ mg_status mgv(mg_handle* h, const Cycle& cy, int l, const void* b, void* out, cu
         const bool final = coarsest && i == npre - 1;
         T* dst = (cur == ws[0]) ? ws[1] : ws[0];
         const bool raw = finest && i == 0;
-        // (a raw sweep writes T: a single-sweep FP32 cycle converts its result)
-        const bool direct = final && !(raw && wide);
-        TRY(Cyc::sweep(h, l, cur, nullptr, raw ? b : bT, raw, raw ? Cyc::b(d) : nullptr, direct ? out : dst,
-                       direct && wide, om, s));
-        if (final) return direct ? MG_OK : launch_emit<T, double>(h, l, dst, nullptr, static_cast<double*>(out), s);
+        // (a cycle of one sweep has no use for b in the cycle's form)
+        TRY(Cyc::sweep(h, l, cur, nullptr, raw ? b : bT, raw, raw && !final ? Cyc::b(d) : nullptr, final ? out : dst,
+                       final && wide, om, s));
+        if (final) return MG_OK;
         cur = dst;
     }
     // residual and restriction onto level l+1

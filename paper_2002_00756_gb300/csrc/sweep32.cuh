@@ -148,7 +148,7 @@ struct Chunk {
 // Register sweep: small levels, tall columns, and sweeps that start from the prolongation alone.  A block has 32 columns; its 2 G warps take the chunks of the two halves' walks, up to
 // K steps each, and load them independently; the recurrence is then handed from warp to warp
 // through shared memory and named barriers (one per pair of neighbouring chunks and half).
-//   BRAW: b is the caller's FP64 array, its FP32 copy is stored in bcopy.
+//   BRAW: b is the caller's FP64 array, its FP32 copy is stored in bcopy unless that is NULL.
 //   xo: padded FP32 iterate, or the caller's FP64 array.
 // (chunks of 8 for columns of more than 80 levels: at most 8 chunks a half, whose barriers are the
 // block's 16)
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(32 * sweep32_warps(K) * sweep32_groups(K), siz
             const int s = min(s0 + j, last);   // (steps past the chunk's end repeat the walk's last one, unused)
             const unsigned k = level(s), o = k * ncolp + at.cp;
             const float bk = BRAW ? (float)__ldg(b + (k * ncol + c)) : (float)__ldg(b + o);
-            if (BRAW && active && j < len) bcopy[o] = bk;
+            if (BRAW && bcopy && active && j < len) bcopy[o] = bk;
             const float ta = ldf(L.tv + ((up ? k : k + 1) * ncolp + at.cp)), rdz = __ldg(L.rdz + k);
             q.ip[j] = __ldg(L.ip + o);
             if constexpr (K == 1) {   // (a half's only step: nothing behind it, and out does not need e)
@@ -559,7 +559,7 @@ struct SweepCall32 {
     const float* xc;
     const void* b;       // FP64 when raw, padded FP32 otherwise
     bool raw;
-    float* bcopy;        // raw: where to store the FP32 copy
+    float* bcopy;        // raw: where to store the FP32 copy, or NULL
     void* xo;            // plain FP64 with out64, padded FP32 otherwise
     bool out64;
     double omega;

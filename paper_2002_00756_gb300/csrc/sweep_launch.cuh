@@ -89,7 +89,8 @@ cudaError_t outs(const SweepCall32<C, P>& q, cudaStream_t s) {
 template <typename C, typename P>
 cudaError_t sweep32_run(const SweepCall32<C, P>& q, cudaStream_t s) {
     if (q.raw) {
-        if (q.mode != XM_ZERO || !q.bcopy || q.out64) return cudaErrorInvalidValue;
+        if (q.mode != XM_ZERO) return cudaErrorInvalidValue;
+        if (q.out64) return form<C, P, XM_ZERO, double, true>(q, s);
         return form<C, P, XM_ZERO, float, true>(q, s);
     }
     switch (q.mode) {

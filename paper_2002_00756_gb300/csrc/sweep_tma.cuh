@@ -138,7 +138,7 @@ struct TmaLayout {
 };
 
 // FULL: every chunk has K steps.  BRAW: b is the caller's plain FP64 array, read directly one tile
-// ahead; its FP32 copy is stored in bcopy.  P = double: the FP64 pivots and multipliers are read
+// ahead; its FP32 copy is stored in bcopy unless that is NULL.  P = double: the FP64 pivots and multipliers are read
 // directly as well (their boxes would leave room for one block per SM only).
 template <typename C, typename P, int MODE, typename O, bool BRAW, int K, bool FULL>
 __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(P), K))
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
             if (gtid == 0 && !late) issue(t + gridDim.x);
             if (BRAW) fetch_b(t + gridDim.x);
         }
-        if (BRAW && lane < cols) {
+        if (BRAW && bcopy && lane < cols) {
 #pragma unroll
             for (int i = 0; i < K; ++i)
                 if (FULL || i < len) bcopy[level(i) * L.ncolp + cp] = q.r[i];

@@ -92,3 +92,19 @@ def test_tall_columns_run_on_tiles(mg):
     """C128L100 against C128L80, 1.25 times the cells: no change to a form of half the rate (1.4
     times the time; 2.0 on register chunks)."""
     assert vcycle_time(mg, 128, 100) <= 1.7 * vcycle_time(mg, 128, 80)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32_p64"])
+@pytest.mark.parametrize("n,nlev", [(10, 20), (12, 3), (96, 41), (24, 90)])
+def test_a_cycle_of_one_sweep_is_one_launch(mg, n, nlev, precision):
+    """One level, one sweep from zero: FP64 in, FP64 out, no copy of b and no conversion."""
+    from oracle.problem import pressure_hierarchy
+    cfg, inp, h, b = setup(mg, n, nlev, 1, precision, n_coarse=1)
+    x = torch.full_like(b, float("nan"))
+    mg.mg_profile_start(h, 16)
+    mg.vcycle(h, b, x)
+    assert [r["kind"] for r in mg.mg_profile_stop(h)] == ["sweep"]
+    ref = pressure_hierarchy(cfg, inp).vcycle(inp["rhs"], cfg.omega, cfg.n_pre, cfg.n_post, 1).ravel()
+    err = float(np.max(np.abs(x.cpu().numpy() - ref)) / np.max(np.abs(ref)))
+    assert err <= (1e-11 if precision == "fp64" else 1e-6), err
+    h.destroy()
