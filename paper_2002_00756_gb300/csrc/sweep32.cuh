@@ -525,25 +525,34 @@ __global__ void k_factor32(Lvl32<C, P> L, P* __restrict__ ip_, P* __restrict__ m
 }
 
 // x_out = (x or 0) + xc[parent] (Eq. prolongation, natural injection) or, without xc, the
-// conversion of x; T or O FP32: padded, FP64: plain; one thread per column and level.
+// conversion of x; T or O FP32: padded, FP64: plain; one thread per column and kchunk levels, which share the
+// column's position and edges.
 template <typename T, typename O>
-__global__ void k_emit(int n, int ncol, const int32_t* __restrict__ hd, const T* __restrict__ x,
+__global__ void k_emit(int n, int ncol, int nlev, int kchunk, const int32_t* __restrict__ hd, const T* __restrict__ x,
                        const T* __restrict__ xc, O* __restrict__ xo) {
     constexpr bool PAD = sizeof(T) == 4, PADO = sizeof(O) == 4;
-    const unsigned c = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= (unsigned)ncol) return;
     const unsigned np = pad_row(n), ncolp = padded(n);
     const Pos at(c, n, np);
-    T v = T(0);
-    if (x) v = x[PAD ? k * ncolp + at.cp : k * ncol + c];
-    if (xc)
-        v += __ldg(xc + (PAD ? k * padded(n >> 1) + at.parent(0, 0, n, pad_row(n >> 1))
-                             : k * (ncol >> 2) + parent_col(c, n)));
-    xo[PADO ? k * ncolp + at.cp : k * ncol + c] = (O)v;
-    if constexpr (PADO) {
-        for (int s = 0; s < 4; ++s) {
-            const int d = hd[(unsigned)s * ncol + c];
-            if (d >= 0) xo[k * ncolp + d] = (O)v;
+    const unsigned from = PAD ? at.cp : c, to = PADO ? at.cp : c, parent = !xc ? 0 : PAD ? at.parent(0, 0, n, pad_row(n >> 1)) : parent_col(c, n);
+    const unsigned lf = PAD ? ncolp : ncol, lt = PADO ? ncolp : ncol, lc = PAD ? padded(n >> 1) : ncol >> 2;
+    int rim[4] = {-1, -1, -1, -1};
+    if (PADO && (at.i == 0 || at.j == 0 || at.i + 1 == (unsigned)n || at.j + 1 == (unsigned)n)) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s) rim[s] = __ldg(hd + (unsigned)s * ncol + c);
+    }
+    const unsigned k0 = blockIdx.y * kchunk, k1 = min(nlev, (int)k0 + kchunk);
+#pragma unroll 4
+    for (unsigned k = k0; k < k1; ++k) {
+        T v = T(0);
+        if (x) v = __ldg(x + (k * lf + from));
+        if (xc) v += __ldg(xc + (k * lc + parent));
+        xo[k * lt + to] = (O)v;
+        if constexpr (PADO) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (rim[s] >= 0) xo[k * lt + rim[s]] = (O)v;
         }
     }
 }

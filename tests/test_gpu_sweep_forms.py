@@ -108,3 +108,37 @@ def test_a_cycle_of_one_sweep_is_one_launch(mg, n, nlev, precision):
     err = float(np.max(np.abs(x.cpu().numpy() - ref)) / np.max(np.abs(ref)))
     assert err <= (1e-11 if precision == "fp64" else 1e-6), err
     h.destroy()
+
+
+def launch_times(mg, n, nlev, kind, variant=0, **kw):
+    _, _, h, b = setup(mg, n, nlev, 2, "fp32", **kw)
+    x, t = torch.empty_like(b), []
+    mg.vcycle(h, b, x)
+    mg.mg_profile_start(h, 4096, kind, 0)
+    for _ in range(15):
+        mg.vcycle(h, b, x)
+    t = [r["ms"] for r in mg.mg_profile_stop(h) if r["variant"] == variant]
+    h.destroy()
+    return float(np.median(t))
+
+
+def test_prolongation_onto_a_level_without_sweeps(mg):
+    """C192L60 without any sweeps on the finest level: the prolongation writes 9 bytes per cell, the restriction of
+    b reads 5; 1.3 times its time (2.7 with a thread per cell, each with the divisions that find its parent)."""
+    kw = dict(n_pre=0, n_post=0)
+    assert launch_times(mg, 192, 60, "prolong", **kw) <= 1.9 * launch_times(mg, 192, 60, "restrict", **kw)
+
+
+@pytest.mark.parametrize("n,nlev", [(10, 9), (96, 20)])
+@pytest.mark.parametrize("n_pre,n_post", [(0, 0), (2, 0), (0, 2)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_cycles_without_sweeps_on_one_side(mg, n, nlev, n_pre, n_post, precision):
+    """The levels' plain copies and prolongations, one level per thread and eight, against the oracle."""
+    from oracle.problem import pressure_hierarchy
+    cfg, inp, h, b = setup(mg, n, nlev, 2, precision, n_pre=n_pre, n_post=n_post)
+    ref = pressure_hierarchy(cfg, inp).vcycle(inp["rhs"], cfg.omega, n_pre, n_post, cfg.n_coarse).ravel()
+    x = torch.full_like(b, float("nan"))
+    mg.vcycle(h, b, x)
+    err = float(np.max(np.abs(x.cpu().numpy() - ref)) / np.max(np.abs(ref)))
+    assert err <= (1e-11 if precision == "fp64" else 1e-6), err
+    h.destroy()
