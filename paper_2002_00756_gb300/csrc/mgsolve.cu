@@ -464,7 +464,7 @@ mg_status launch_sweep32(mg_handle* h, int lev, const float* x, const float* xc,
     const mg::SweepMaps* maps = nullptr;
     const bool tiles = d.sweep_bd > 0 ? d.sweep_bd == 128 : tma_level(L.nlev, L.ncol);
     // (an FP64 elimination's chunks of taller columns have no room beside the boxes)
-    const bool has = mode != mg::XM_PROLONG0 && (sizeof(P) == 4 || L.nlev <= mg::tma_max_levels(8));
+    const bool has = sizeof(P) == 4 || L.nlev <= mg::tma_max_levels(8);
     if (tiles && has && d.maps.size() == 2) maps = &d.maps[x == d.x32[1]];
     const mg::SweepCall32<C, P> q{L, mode, x, xc, b, raw, bcopy, xo, out64, om, maps, h->nsm, h->polls, h->timeout};
     CK((mg::sweep32_run<C, P>(q, s)));

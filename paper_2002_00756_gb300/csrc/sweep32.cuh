@@ -145,9 +145,9 @@ struct Chunk {
 };
 
 // ---------------------------------------------------------------------------------------
-// Register sweep: small levels, tall columns, and sweeps that start from the prolongation alone.  A block has 32 columns; its 2 G warps take the chunks of the two halves' walks, up to
-// K steps each, and load them independently; the recurrence is then handed from warp to warp
-// through shared memory and named barriers (one per pair of neighbouring chunks and half).
+// Register sweep: small levels and short columns.  A block has 32 columns; its 2 G warps take the chunks of
+// the two halves' walks, up to K steps each, and load them independently; the recurrence is then handed
+// from warp to warp through shared memory and named barriers (one per pair of neighbouring chunks and half).
 //   BRAW: b is the caller's FP64 array, its FP32 copy is stored in bcopy unless that is NULL.
 //   xo: padded FP32 iterate, or the caller's FP64 array.
 // (chunks of 8 for columns of more than 80 levels: at most 8 chunks a half, whose barriers are the
@@ -163,7 +163,7 @@ __host__ __device__ constexpr int sweep32_groups(int K) { return K < 5 ? 4 : 1; 
 __device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 
 template <typename C, typename P, int MODE, typename B, typename O, bool BRAW, int K>
-__global__ void __launch_bounds__(32 * sweep32_warps(K) * sweep32_groups(K), sizeof(P) == 8 ? 1 : K == 10 ? 3 : K == 8 && MODE == XM_ZERO ? 2 : 1)
+__global__ void __launch_bounds__(32 * sweep32_warps(K) * sweep32_groups(K), sizeof(P) == 4 && K == 8 && MODE == XM_ZERO ? 2 : 1)
     k_sweep32(Lvl32<C, P> L, const float* __restrict__ x, const float* __restrict__ xc, const B* __restrict__ b,
               float* __restrict__ bcopy, O* __restrict__ xo, float omega) {
     constexpr bool PRO = (MODE == XM_PROLONG || MODE == XM_PROLONG0);

@@ -9,11 +9,9 @@
 namespace mg {
 namespace {
 
-// Levels per chunk of the register sweep: 10 where the level fills the GPU, 5 below 2M cells (twice
-// the threads); columns of more than 80 levels take 8, so that a block has at most 16 warps (a
-// sweep from zero on the registers of two blocks per SM: C50L110 21 -> 17 us, C40L128 16 -> 13).
-constexpr int BIG_K = 10, SMALL_K = 5, TALL_K = 8;
-constexpr double SMALL_CELLS = 2e6;
+// Levels per chunk of the register sweep: 5; columns of more than 80 levels take 8, so that a block has at
+// most 16 warps (a sweep from zero on the registers of two blocks per SM: C50L110 21 -> 17 us, C40L128 16 -> 13).
+constexpr int CHUNK_K = 5, TALL_K = 8;
 
 template <typename C, typename P, int MODE, typename B, typename O, bool BRAW, int K>
 cudaError_t go(const SweepCall32<C, P>& q, cudaStream_t s) {
@@ -37,8 +35,7 @@ cudaError_t shape(const SweepCall32<C, P>& q, cudaStream_t s) {
         default: break;
     }
     if (q.L.nlev > 80) return go<C, P, MODE, B, O, BRAW, TALL_K>(q, s);
-    if ((double)q.L.nlev * q.L.ncol < SMALL_CELLS) return go<C, P, MODE, B, O, BRAW, SMALL_K>(q, s);
-    return go<C, P, MODE, B, O, BRAW, BIG_K>(q, s);
+    return go<C, P, MODE, B, O, BRAW, CHUNK_K>(q, s);
 }
 
 constexpr int TMA_SMEM = 227 * 1024;   // shared memory of an SM, and the most a block can have
@@ -65,15 +62,13 @@ cudaError_t go_tma(const SweepCall32<C, P>& q, cudaStream_t s) {
 // tiles where the level has them, else register chunks
 template <typename C, typename P, int MODE, typename O, bool BRAW>
 cudaError_t form(const SweepCall32<C, P>& q, cudaStream_t s) {
-    if constexpr (MODE != XM_PROLONG0) {
-        if (q.maps) {
-            if constexpr (sizeof(P) == 4) {
-                if (q.L.nlev > tma_max_levels(8)) return go_tma<C, P, MODE, O, BRAW, 10, false>(q, s);
-            }
-            if (q.L.nlev > tma_max_levels(7)) return go_tma<C, P, MODE, O, BRAW, 8, false>(q, s);
-            if (q.L.nlev == tma_chunks(q.L.nlev, 7) * 14) return go_tma<C, P, MODE, O, BRAW, 7, true>(q, s);
-            return go_tma<C, P, MODE, O, BRAW, 7, false>(q, s);
+    if (q.maps) {
+        if constexpr (sizeof(P) == 4) {
+            if (q.L.nlev > tma_max_levels(8)) return go_tma<C, P, MODE, O, BRAW, 10, false>(q, s);
         }
+        if (q.L.nlev > tma_max_levels(7)) return go_tma<C, P, MODE, O, BRAW, 8, false>(q, s);
+        if (q.L.nlev == tma_chunks(q.L.nlev, 7) * 14) return go_tma<C, P, MODE, O, BRAW, 7, true>(q, s);
+        return go_tma<C, P, MODE, O, BRAW, 7, false>(q, s);
     }
     return shape<C, P, MODE, typename std::conditional<BRAW, double, float>::type, O, BRAW>(q, s);
 }

@@ -1,5 +1,5 @@
 // The column sweep of large FP32 levels with every operand brought by TMA (the same arithmetic as
-// k_sweep32 in sweep32.cuh; not for XM_PROLONG0).
+// k_sweep32 in sweep32.cuh).
 //
 // A tile is up to 32 consecutive columns of one row of a panel, all levels.  One thread issues one
 // tensor copy per stream and half tile (box: columns x nlev / 2 of the level-major array), so no
@@ -121,11 +121,11 @@ struct TmaLayout {
         te = add(it, H, 32 * CS + 16);
         tn = add(it, H, 32 * CS);
         ts = add(it, H, 32 * CS);
-        x = add(it, H + 1, 160);
-        xn = add(it, H, 128);
-        xs = add(it, H, 128);
-        c0 = add(MODE == XM_PROLONG, H + 1, 96);
-        c1 = add(MODE == XM_PROLONG, H, 96);
+        x = add(it && MODE != XM_PROLONG0, H + 1, 160);
+        xn = add(it && MODE != XM_PROLONG0, H, 128);
+        xs = add(it && MODE != XM_PROLONG0, H, 128);
+        c0 = add(MODE == XM_PROLONG || MODE == XM_PROLONG0, H + 1, 96);
+        c1 = add(MODE == XM_PROLONG || MODE == XM_PROLONG0, H, 96);
         tx = bytes;
         group = o;
         rdz = 2 * o + K * 160;
@@ -145,8 +145,9 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
     k_sweep_tma(const __grid_constant__ SweepMaps M, Lvl32<C, P> L, const double* __restrict__ braw,
                 float* __restrict__ bcopy, O* __restrict__ xo, float omega, int tiles_row, int tile_w,
                 int polls, unsigned int* __restrict__ timeout) {
-    static_assert(MODE != XM_PROLONG0, "iterate source");
-    constexpr bool PRO = MODE == XM_PROLONG, ZERO = MODE == XM_ZERO, PADO = sizeof(O) == 4, D64 = sizeof(P) == 8;
+    constexpr bool PRO = MODE == XM_PROLONG || MODE == XM_PROLONG0;
+    constexpr bool RAW = MODE == XM_PLAIN || MODE == XM_PROLONG;   // reads the fine iterate
+    constexpr bool ZERO = MODE == XM_ZERO, PADO = sizeof(O) == 4, D64 = sizeof(P) == 8;
     constexpr int TW = 16 / (int)sizeof(C), TP = 32 + TW;   // te: columns to the west, row pitch
     extern __shared__ __align__(128) unsigned char sm_all[];
     const TmaLayout<C, P, MODE, BRAW, K> Y(L.nlev);
@@ -195,9 +196,11 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
         if (!D64) tma_load(sm + Y.ip, &M.ip, c, kb, bar);
         if (!D64 || !ZERO) tma_load(sm + Y.tv, &M.tv, c, kb, bar);
         if (!ZERO) {
-            tma_load(sm + Y.x, &M.x, c - 4, kx, bar);
-            tma_load(sm + Y.xn, &M.xr, c + np, kb, bar);
-            tma_load(sm + Y.xs, &M.xr, c - np, kb, bar);
+            if (RAW) {
+                tma_load(sm + Y.x, &M.x, c - 4, kx, bar);
+                tma_load(sm + Y.xn, &M.xr, c + np, kb, bar);
+                tma_load(sm + Y.xs, &M.xr, c - np, kb, bar);
+            }
             tma_load(sm + Y.te, &M.te, c - TW, kb, bar);
             tma_load(sm + Y.tn, &M.tn, c, kb, bar);
             tma_load(sm + Y.ts, &M.tn, c - np, kb, bar);
@@ -273,10 +276,10 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
             // (before the walk's first step the face behind and its m are zero)
             float xb = 0.f, x0 = 0.f, tb = 0.f, ipb = 0.f;
             if (!D64 || !ZERO) tb = lds<C>(qtv - D * 32);
-            if (!ZERO) x0 = qx[0];
+            if (RAW) x0 = qx[0];
             if (PRO) x0 += qc[0];
             if (s0 > 0) {
-                if (!ZERO) xb = qx[-D * 40];
+                if (RAW) xb = qx[-D * 40];
                 if (PRO) xb += qc[-D * 24];
                 if (!D64) ipb = qi[-D * 32];
             }
@@ -297,8 +300,14 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
                 q.x[i] = x0;
                 q.r[i] = bk;
                 if constexpr (!ZERO) {
-                    float xa = qx[D * (i + 1) * 40];
-                    float xE = qx[D * i * 40 + 1], xW = qx[D * i * 40 - 1], xN = qn[D * i * 32], xS = qs[D * i * 32];
+                    float xa = 0.f, xE = 0.f, xW = 0.f, xN = 0.f, xS = 0.f;
+                    if (RAW) {
+                        xa = qx[D * (i + 1) * 40];
+                        xE = qx[D * i * 40 + 1];
+                        xW = qx[D * i * 40 - 1];
+                        xN = qn[D * i * 32];
+                        xS = qs[D * i * 32];
+                    }
                     if (PRO) {
                         const float cm = qc[D * i * 24], co = qo[D * i * 24], ca = qa[D * i * 24];
                         xa += qc[D * (i + 1) * 24];

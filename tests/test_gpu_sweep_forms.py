@@ -142,3 +142,10 @@ def test_cycles_without_sweeps_on_one_side(mg, n, nlev, n_pre, n_post, precision
     err = float(np.max(np.abs(x.cpu().numpy() - ref)) / np.max(np.abs(ref)))
     assert err <= (1e-11 if precision == "fp64" else 1e-6), err
     h.destroy()
+
+
+def test_a_sweep_from_the_prolongation_alone_runs_on_tiles(mg):
+    """C128L70 without sweeps before the coarse correction: the first sweep after it reads less than a plain one
+    and takes about its time (twice that on register chunks)."""
+    first, plain = (launch_times(mg, 128, 70, "sweep", v, n_pre=0) for v in (3, 0))
+    assert first <= 1.3 * plain, (first, plain)
