@@ -368,7 +368,12 @@ mg_status launch_apply(mg_handle* h, int lev, const Lvl<T, C>& L, const X* x, Y*
 //   more than 80 levels, one block of tiles per SM, 2M: C128L100 778 and 537 (alone; before the chunks 725),
 //   C192L100 1467 and 1050 (1333), C64L128 324 and 274, C80L100 365 and 335; C48L100, 1.4M: 190 and 195,
 //   C48L81 166 and 178.
+// Short columns stay on chunks where these hold a half without waste and the tiles' chunks of 7 would be about
+// half empty: 8 levels (a chunk of 4) and 15 to 20 (two of 4 or 5).  Finest sweep from zero / plain / with
+// prolongation, tiles and chunks: C256L8 49/47/54 and 19/33/37, C224L16 59/61/68 and 41/52/57, C192L20 45/49/51 and
+// 35/43/47; C256L9 49/47/55 and 45/55/59, C224L14 33/39/42 and 39/51/55, C192L24 45/51/53 and 37/76/82.
 inline bool tma_level(int nlev, int ncol) {
+    if (nlev <= 8 || (nlev >= 15 && nlev <= 20)) return false;
     return (double)nlev * ncol >= (nlev > 80 ? 2e6 : nlev > 40 ? 2.5e5 : 7e5);
 }
 

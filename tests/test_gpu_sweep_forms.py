@@ -149,3 +149,9 @@ def test_a_sweep_from_the_prolongation_alone_runs_on_tiles(mg):
     and takes about its time (twice that on register chunks)."""
     first, plain = (launch_times(mg, 128, 70, "sweep", v, n_pre=0) for v in (3, 0))
     assert first <= 1.3 * plain, (first, plain)
+
+
+def test_short_columns_that_chunks_hold_without_waste(mg):
+    """C256L8 in registers (a chunk of 4 per half) against C256L10 on tiles: 0.7 of its time (as much of it on tiles,
+    whose chunks of 7 would be half empty)."""
+    assert launch_times(mg, 256, 8, "sweep") <= 0.85 * launch_times(mg, 256, 10, "sweep")
