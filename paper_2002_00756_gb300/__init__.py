@@ -108,6 +108,7 @@ _SIGS = {
     "mixed_solve_adjoint": [_VP, _DP, _DP, _DP, _DP, _D, ctypes.POINTER(_Info), _VP],
     "mixed_coefficient_gradient": [_VP, _DP, _DP, _DP, _DP, _DP, _DP, _VP],
     "mg_autotune": [_VP, ctypes.POINTER(ctypes.c_int32), _VP],
+    "mg_apply_choices": [_VP, ctypes.POINTER(ctypes.c_int32)],
     "schur_precond": [_VP, _DP, _DP, _DP, _DP, _VP],
     "mg_profile_start": [_VP, _I32, _I32, _I32],
     "mg_profile_stop": [_VP, ctypes.POINTER(_KRec), _I32, ctypes.POINTER(ctypes.c_int32)],
@@ -481,6 +482,14 @@ def mg_autotune(h: Handle, stream=None) -> list[tuple[int, int, int]]:
     ch = (ctypes.c_int32 * (3 * h.levels))()
     _check(load().mg_autotune(h.ptr, ch, _stream(stream)), "mg_autotune")
     return [(ch[3 * l], ch[3 * l + 1], ch[3 * l + 2]) for l in range(h.levels)]
+
+
+def mg_apply_choices(h: Handle, choices):
+    """Take the launch forms of an earlier mg_autotune (its list, one triple per level)"""
+    if len(choices) != h.levels:
+        raise ValueError("one triple per level")
+    flat = [int(v) for c in choices for v in c]
+    _check(load().mg_apply_choices(h.ptr, (ctypes.c_int32 * len(flat))(*flat)), "mg_apply_choices")
 
 
 def mixed_apply_transpose(h: Handle, u, p, yu, yp, stream=None):

@@ -2433,6 +2433,22 @@ mg_status mg_autotune(mg_handle* h, int32_t* choices, void* stream) {
     return MG_OK;
 }
 
+mg_status mg_apply_choices(mg_handle* h, const int32_t* choices) {
+    if (!h || !choices) return MG_ERR_ARG;
+    for (int l = 0; l < h->L; ++l) {
+        const int form = choices[3 * l], kc = choices[3 * l + 1];
+        if ((form != 0 && form != 64 && form != 128) || kc < 0) return MG_ERR_ARG;
+    }
+    DeviceGuard dg(h->device);
+    CK(cudaDeviceSynchronize());
+    for (int l = 0; l < h->L; ++l) {
+        h->lv[l].sweep_bd = choices[3 * l];
+        h->lv[l].restrict_kc = choices[3 * l + 2] == 1 ? 0 : choices[3 * l + 1];
+    }
+    drop_graphs(h, 0);
+    return MG_OK;
+}
+
 mg_status mg_profile_start(mg_handle* h, int32_t capacity, int32_t kind, int32_t level) {
     if (!h || capacity < 1 || capacity > (1 << 20)) return MG_ERR_ARG;
     h->prof_kind = kind < 0 ? -1 : kind;

@@ -155,3 +155,89 @@ def test_short_columns_that_chunks_hold_without_waste(mg):
     """C256L8 in registers (a chunk of 4 per half) against C256L10 on tiles: 0.7 of its time (as much of it on tiles,
     whose chunks of 7 would be half empty)."""
     assert launch_times(mg, 256, 8, "sweep") <= 0.85 * launch_times(mg, 256, 10, "sweep")
+
+
+def forced(mg, h, form, kc=0):
+    mg.mg_apply_choices(h, [(form, kc, 0)] * h.levels)
+
+
+# n not a multiple of 4 or 8, single tiles and several; 8 levels, both ends of the chunks of 7, 8 and 10,
+# short columns (chunks of 1 to 4, four groups a block), levels above and below 2M cells
+FORMS = [(2, 8, 1), (6, 8, 2), (10, 9, 2), (20, 30, 2), (24, 70, 3), (50, 71, 2), (33, 80, 1), (26, 81, 2), (34, 128, 2), (92, 41, 2),
+         (66, 80, 2), (64, 128, 2)]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp32_p64", "fp32_bf16"])
+@pytest.mark.parametrize("n,nlev,levels", FORMS)
+def test_tiles_and_register_chunks_agree_bit_for_bit(mg, n, nlev, levels, precision):
+    """Each form forced on every level: the same rounding, so the same V-cycle (sweeps from zero, plain,
+    with prolongation across panel edges); and any number of levels per thread of the restriction."""
+    _, _, h, b = setup(mg, n, nlev, levels, precision)
+    x, y = torch.full_like(b, float("nan")), torch.full_like(b, float("nan"))
+    forced(mg, h, 64)
+    mg.vcycle(h, b, x)
+    forced(mg, h, 128, 3)
+    mg.vcycle(h, b, y)
+    assert torch.equal(x, y)
+    forced(mg, h, 0)
+    mg.vcycle(h, b, y)
+    assert torch.equal(x, y)
+    h.destroy()
+    _, _, h, b = setup(mg, n, nlev, levels, precision, n_pre=0)   # (a sweep from the prolongation alone)
+    forced(mg, h, 64)
+    mg.vcycle(h, b, x)
+    forced(mg, h, 128)
+    mg.vcycle(h, b, y)
+    assert torch.equal(x, y)
+    h.destroy()
+
+
+@pytest.mark.parametrize("n,nlev,levels,precision,kw", [
+    (92, 41, 2, "fp64", {}),                   # FP64 chunks of 10, uneven: products of 8 and 9 levels
+    (96, 43, 2, "fp64", {}),
+    (96, 41, 2, "fp32", dict(n_pre=0)),        # chunks in registers, from a prolongation alone
+    (80, 81, 2, "fp32", {}),                   # tall tiles
+    (52, 128, 2, "fp32", {}),
+    (8, 1, 2, "fp32", {}), (6, 2, 1, "fp32_p64", {}), (10, 3, 2, "fp32", {}), (12, 4, 2, "fp32_p64", {}),
+    (10, 5, 2, "fp32_p64", {}), (6, 6, 1, "fp32", {}), (14, 7, 2, "fp32", {}), (10, 8, 2, "fp32_p64", {}),
+])
+def test_vcycle_against_the_oracle(mg, n, nlev, levels, precision, kw):
+    """1e-6 of the largest element in FP32, 1e-11 in FP64, as for the other shapes."""
+    from oracle.problem import pressure_hierarchy
+    cfg, inp, h, b = setup(mg, n, nlev, levels, precision, **kw)
+    ref = pressure_hierarchy(cfg, inp).vcycle(inp["rhs"], cfg.omega, cfg.n_pre, cfg.n_post, cfg.n_coarse).ravel()
+    if kw:
+        forced(mg, h, 64)
+    x = torch.full_like(b, float("nan"))
+    mg.vcycle(h, b, x)
+    err = float(np.max(np.abs(x.cpu().numpy() - ref)) / np.max(np.abs(ref)))
+    assert err <= (1e-11 if precision == "fp64" else 1e-6), err
+    h.destroy()
+
+
+def test_choices_are_checked(mg):
+    _, _, h, b = setup(mg, 8, 9, 2, "fp32")
+    for bad in ((32, 0, 0), (64, -1, 0)):
+        with pytest.raises(mg.MGError):
+            mg.mg_apply_choices(h, [(0, 0, 0), bad])
+    with pytest.raises(ValueError):
+        mg.mg_apply_choices(h, [(0, 0, 0)])
+    mg.mg_apply_choices(h, mg.mg_autotune(h))
+    h.destroy()
+
+
+@pytest.mark.parametrize("a", [0.0, 1.0, 1e20, 1e29, 1e31, 1e40, 1e200])
+def test_pivots_of_any_size(mg, a):
+    """One level of C1, whose six cells are alike and whose couplings all equal a: a sweep from zero is
+    omega b / (1 + 4 a).  Seven roundings (weights, sum, reciprocal, products) and the weights' own: 1e-15,
+    below and above the range in which the reciprocal starts from FP32 (1e30)."""
+    h = mg.mg_setup(1, 1, [0.0, 1000.0], np.ones(6), levels=1)
+    coef = torch.zeros((6, 6), dtype=torch.float64, device="cuda")
+    coef[:4] = a
+    mg.mg_set_coefficients(h, coef.ravel())
+    b = torch.from_numpy(syn.normal(5, 0, 6)).cuda()
+    x = torch.empty_like(b)
+    mg.mg_smooth(h, 0, b, None, x, 1)
+    ref = 0.8 * b.cpu().numpy() / (1.0 + 4.0 * a)
+    assert np.max(np.abs(x.cpu().numpy() / ref - 1.0)) <= 1e-15
+    h.destroy()
