@@ -397,8 +397,8 @@ mg_status mg_autotune(mg_handle* h, int32_t* choices, void* stream);
 /* Takes the launch forms that mg_autotune wrote to `choices` for a handle of the same mesh (3 * levels
  * int32 as described there; a sweep form or a number of levels of 0 is the built-in one), so that a
  * tuned program need not tune again.  Changes times only.  Drops the handle's cached GCR graphs.
- * Synchronous.  MG_ERR_ARG for other sweep forms than 0, 64 and 128 or negative numbers of levels, with the
- * handle unchanged. */
+ * Synchronous.  MG_ERR_ARG for other sweep forms than 0, 64 and 128 or numbers of levels outside
+ * 0 .. MG_MAX_NLEV, with the handle unchanged. */
 mg_status mg_apply_choices(mg_handle* h, const int32_t* choices);
 
 /* [u; p] = P_mixed [ru; rp], the Schur-complement preconditioner with one V-cycle. */

@@ -2437,7 +2437,7 @@ mg_status mg_apply_choices(mg_handle* h, const int32_t* choices) {
     if (!h || !choices) return MG_ERR_ARG;
     for (int l = 0; l < h->L; ++l) {
         const int form = choices[3 * l], kc = choices[3 * l + 1];
-        if ((form != 0 && form != 64 && form != 128) || kc < 0) return MG_ERR_ARG;
+        if ((form != 0 && form != 64 && form != 128) || kc < 0 || kc > MG_MAX_NLEV) return MG_ERR_ARG;
     }
     DeviceGuard dg(h->device);
     CK(cudaDeviceSynchronize());

@@ -217,7 +217,7 @@ def test_vcycle_against_the_oracle(mg, n, nlev, levels, precision, kw):
 
 def test_choices_are_checked(mg):
     _, _, h, b = setup(mg, 8, 9, 2, "fp32")
-    for bad in ((32, 0, 0), (64, -1, 0)):
+    for bad in ((32, 0, 0), (64, -1, 0), (64, 129, 0), (0, 2 ** 31 - 1, 0)):
         with pytest.raises(mg.MGError):
             mg.mg_apply_choices(h, [(0, 0, 0), bad])
     with pytest.raises(ValueError):
