@@ -234,7 +234,8 @@ __global__ void __launch_bounds__(tma_threads(K), tma_blocks(MODE, BRAW, sizeof(
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, phase ^= 1) {
         const int row = t / tiles_row, i0 = (t - row * tiles_row) * tile_w;
         const int p = row / n, j = row - p * n, cols = min(tile_w, n - i0);
-        const unsigned c = row * n + i0 + min(lane, cols - 1), cp = (row + 2 * p + 1) * np + of + i0 + lane;
+        // (lanes beyond the tile repeat its last column: rows are too short on small meshes to read on)
+        const unsigned c = row * n + i0 + min(lane, cols - 1), cp = (row + 2 * p + 1) * np + of + i0 + min(lane, cols - 1);
         const float rA = __ldg(L.rA + c);
         // (an edge column is repeated in one rim, a corner column in two)
         int rim0 = -1, rim1 = -1;
