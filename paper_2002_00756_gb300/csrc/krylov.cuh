@@ -443,7 +443,7 @@ __device__ __forceinline__ void gcr_accumulate(double (&v)[J + 2], double we, do
     v[J + 1] += re * we;
 }
 
-// GCR sums for a new direction w (mixed system path, where w comes from other kernels).
+// GCR sums for a new direction w of the 9-cell stencil, whose operator is a kernel of its own.
 template <int J>
 __global__ void __launch_bounds__(RED_THREADS) k_gcr_sums(size_t n, const double* __restrict__ w,
                                                           const double* __restrict__ Wb, size_t ld,

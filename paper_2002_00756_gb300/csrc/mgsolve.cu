@@ -1133,8 +1133,7 @@ mg_status schur_impl(mg_handle* h, const double* ru, const double* rp, double* u
     return launch_mixed<mg::MX_UPDATE, -1>(h, ru, p, u, nullptr, nullptr, s);
 }
 
-// parents of the neighbours E, W, N, S and of the column itself, [5][ncol]
-// the rim cell of the padded fields that repeats each edge column (SLvl::hd), [4][ncol]
+// the rim cell of the padded fields that repeats each edge column (Lvl32::hd), [4][ncol]
 __global__ void k_rims(int n, int ncol, const int32_t* __restrict__ nbr, int32_t* __restrict__ hd) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
     if (c >= ncol) return;
@@ -1155,6 +1154,7 @@ __global__ void k_reciprocal(size_t n, const double* __restrict__ a, double* __r
         r[i] = 1.0 / a[i];
 }
 
+// parents of the neighbours E, W, N, S and of the column itself (Lvl64::par), [5][ncol]
 __global__ void k_parents(int n, int ncol, const int32_t* __restrict__ nbr, int32_t* __restrict__ par) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
     if (c < ncol) par[(size_t)s * ncol + c] = mg::parent_col(s < 4 ? nbr[(size_t)s * ncol + c] : c, n);

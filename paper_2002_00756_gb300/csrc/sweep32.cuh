@@ -346,14 +346,15 @@ __global__ void k_fill_rims(int n, int ncol, const int32_t* __restrict__ hd, T* 
 // Residual and restriction (Algorithm 1): bc[k][C] = sum_q w_q (b - H x)[k][child_q],
 // w = area_child / area_C.  One thread per coarse column (2 x 2 fine columns, whose rows are read 2
 // wide) and kchunk levels.  TREE: the children are summed in pairs (levels of n % 16 == 0), else
-// one after the other.  The loads in flight bound it: the loop stays rolled (two levels at a
+// one after the other: either order is as accurate, both stay because another would move every solve's
+// result within its tolerance (above).  The loads in flight bound it: the loop stays rolled (two levels at a
 // time need more registers, fewer blocks fit: C192L70 72 us instead of 56, C96L70 21 instead of 17; three
 // couplings, x, b and the result at copy speed: 46 and 12).
 template <typename C, bool XZERO, bool TREE>
 __global__ void __launch_bounds__(128) k_restrict32(Lvl32<C, float> L, const float* __restrict__ x,
                                                     const float* __restrict__ b, const float* __restrict__ wq,
                                                     float* __restrict__ bc, int ncol_c, int kchunk) {
-    const unsigned ncol = L.ncol, n = L.n, nc = n >> 1, np = L.np, lx = L.ncolp;
+    const unsigned n = L.n, nc = n >> 1, np = L.np, lx = L.ncolp;
     const unsigned Cc = blockIdx.x * blockDim.x + threadIdx.x;
     if (Cc >= (unsigned)ncol_c) return;
     const Pos at(Cc, nc, pad_row(nc));
@@ -382,7 +383,6 @@ __global__ void __launch_bounds__(128) k_restrict32(Lvl32<C, float> L, const flo
             rA[r][v] = __ldg(L.rA + c0 + r * n + v);
             ww[r][v] = __ldg(wq + (unsigned)(2 * r + v) * ncol_c + Cc);
         }
-    (void)ncol;
     float x0[2][2], xb[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, tb[2][2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {

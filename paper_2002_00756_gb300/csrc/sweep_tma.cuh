@@ -9,15 +9,17 @@
 // box, and the N / S neighbours and south faces are boxes one padded row up / down, at a panel's
 // edges as anywhere else.
 //
-// Blocks are persistent (two per SM where shared memory allows): as soon as a tile's values are in
+// Blocks are persistent (tma_blocks per SM): as soon as a tile's values are in
 // registers the copies of the block's next tile are issued into the same buffers, and run during
 // the recurrences and the stores.
 //
 // Measured (finest level of C192L70, 15.5M cells, us per sweep; two threads per column with the pivot
 // chain in the walk before): plain 86 (121), with prolongation 90 (134), from zero 72 (108); BF16
-// couplings at C90L41 18 (27); FP64 elimination at C96L70 102 (194).  A plain sweep moves 372 MB (24 B
-// per cell), 55 us at the measured copy rate; the same boxes with nothing computed stream in 61 us.
-// Of the rest, 10 us are the stores, the others the time a group's buffers wait for its warps.
+// couplings at C90L41 18 (27); FP64 elimination at C96L70 102 (194).  A plain sweep moves 433 MB (28 B
+// per cell: x, b, three couplings, the reciprocal pivot, the result), 64 us at the measured copy rate; its
+// boxes alone, nothing computed or stored, stream in 61 us.  Of the rest, 10 us are the stores, the others
+// the time a group's buffers wait for its warps.  Columns of more than 80 levels, one block per SM: C128L100,
+// 9.8M cells, 78 us in every mode (the register chunks 103 to 142).
 // With the panel edges fetched by threads instead of kept in rims the plain sweep took 96 us.
 #pragma once
 
