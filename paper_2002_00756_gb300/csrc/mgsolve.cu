@@ -1299,6 +1299,33 @@ mg_status set_coefficients_impl(mg_handle* h, const double* a, cudaStream_t s) {
     return MG_OK;
 }
 
+// x_out = x_in (NULL: zero) after `sweeps` block-Jacobi sweeps in FP64 with one scratch array: they alternate
+// between it and x_out, ordered so that the last one writes x_out.  A sweep never writes the array it
+// reads: where x_in is x_out and that would be the first target, the first sweep goes to the scratch array and
+// the result is copied at the end.  (rec is NULL where no launch may be recorded.)
+mg_status smooth_into(mg_handle* h, mg_handle* rec, int level, const double* b, const double* x_in, double* x_out,
+                      int sweeps, double* scratch, cudaStream_t s) {
+    const size_t n = cells(h, level);
+    if (sweeps == 0) {
+        if (!x_in) CK(cudaMemsetAsync(x_out, 0, n * sizeof(double), s));
+        else if (x_in != x_out) CK(cudaMemcpyAsync(x_out, x_in, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+        return MG_OK;
+    }
+    if (!h->nine) TRY(ready64(h, level, s));
+    const Lvl64 L = lvl64(h, level);
+    bool to_out = sweeps % 2 == 1 && x_in != x_out;
+    const double* cur = x_in;
+    for (int i = 0; i < sweeps; ++i) {
+        double* dst = to_out ? x_out : scratch;
+        if (h->nine) TRY((sweep9<double, double, double>(h, level, cur, b, dst, h->prm.omega, s)));
+        else TRY(launch_sweep64(rec, level, L, cur, nullptr, 0, b, true, nullptr, dst, h->prm.omega, s));
+        cur = dst;
+        to_out = !to_out;
+    }
+    if (cur != x_out) CK(cudaMemcpyAsync(x_out, cur, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    return MG_OK;
+}
+
 mg_status check_level(const mg_handle* h, int level) {
     if (!h || level < 0 || level >= h->L) return MG_ERR_ARG;
     return MG_OK;
@@ -1491,7 +1518,8 @@ mg_status setup_impl(mg_handle* h, const mg_mesh* mesh, const mg_params* prm, co
             }
             if (l + 1 < L && prec == MG_FP64) own.add(&d.par, 5 * (size_t)G.ncol);
         }
-        for (double*& p : d.x64) own.add(&p, Nl);
+        // (mg_smooth's scratch array; the second iterate of an FP64 V-cycle)
+        for (int i = 0; i < (prec == MG_FP64 ? 2 : 1); ++i) own.add(&d.x64[i], Nl);
         // right-hand sides and, below the finest level, the iterate that goes up
         if (prec == MG_FP64) {
             own.add(&d.b64, Nl);
@@ -2297,19 +2325,7 @@ mg_status mg_smooth(mg_handle* h, int32_t level, const double* b, const double* 
     DeviceGuard dg(h->device);
     cudaStream_t s = S(stream);
     DevLevel& d = h->lv[level];
-    if (!h->nine && sweeps > 0) TRY(ready64(h, level, s));
-    const Lvl64 L = lvl64(h, level);
-    const size_t n = cells(h, level);
-    const double* cur = x_in;
-    for (int i = 0; i < sweeps; ++i) {
-        double* dst = (cur == d.x64[0]) ? d.x64[1] : d.x64[0];
-        if (h->nine) TRY((sweep9<double, double, double>(h, level, cur, b, dst, h->prm.omega, s)));
-        else TRY(launch_sweep64(h, level, L, cur, nullptr, 0, b, true, nullptr, dst, h->prm.omega, s));
-        cur = dst;
-    }
-    if (cur == nullptr) CK(cudaMemsetAsync(x_out, 0, n * sizeof(double), s));
-    else if (cur != x_out) CK(cudaMemcpyAsync(x_out, cur, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    return MG_OK;
+    return smooth_into(h, h, level, b, x_in, x_out, sweeps, d.x64[0], s);
 }
 
 mg_status mg_residual_restrict(mg_handle* h, int32_t level, const double* b, const double* x, double* bc,
@@ -2531,27 +2547,5 @@ extern "C" mg_status mg_smooth_noalloc(mg_handle* h, int32_t level, const double
     double* scratch = nullptr;
     TRY(scratch_address(h->device, &scratch));
     cudaStream_t s = S(stream);
-    if (sweeps > 0) TRY(ready64(h, level, s));
-    const Lvl64 L = lvl64(h, level);
-    if (sweeps == 0) {
-        if (!x_in) CK(cudaMemsetAsync(x_out, 0, n * sizeof(double), s));
-        else if (x_in != x_out) CK(cudaMemcpyAsync(x_out, x_in, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-        return MG_OK;
-    }
-    // Sweeps alternate between the scratch array and x_out, ordered so that the last one
-    // writes x_out.  A sweep never writes the array it reads, so when x_in aliases x_out
-    // and x_out would be the first target, the first sweep goes to the scratch array and
-    // the result is copied to x_out at the end.
-    bool to_out = ((sweeps - 1) % 2) == 0;
-    const bool copy_back = to_out && x_in == x_out;
-    if (copy_back) to_out = false;
-    const double* cur = x_in;
-    for (int i = 0; i < sweeps; ++i) {
-        double* dst = to_out ? x_out : scratch;
-        TRY(launch_sweep64(nullptr, level, L, cur, nullptr, 0, b, true, nullptr, dst, h->prm.omega, s));
-        cur = dst;
-        to_out = !to_out;
-    }
-    if (cur != x_out) CK(cudaMemcpyAsync(x_out, cur, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    return MG_OK;
+    return smooth_into(h, nullptr, level, b, x_in, x_out, sweeps, scratch, s);
 }

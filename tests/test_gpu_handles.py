@@ -133,3 +133,37 @@ def test_a_refused_set_of_couplings_leaves_no_trace(mg, precision):
     mg.helmholtz_apply(h, b, x)
     assert torch.equal(x, b)
     h.destroy()
+
+
+def test_one_fp64_scratch_array_is_enough_for_smoothing(mg):
+    """C160L60, restart 1, FP32: 24 + 8 + 56 + 32 bytes per cell and seven FP32 fields padded by 1.215 (9.2M
+    cells; a second scratch array would be 74 MB)."""
+    used, cells = device_bytes(mg, 160, 60, "fp32")
+    assert used <= (24 + 8 + 56 + 32 + 28 * 1.215) * cells + 20 * 2 ** 21, used / cells
+
+
+@pytest.mark.parametrize("gamma2", [0.0, 0.25])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("sweeps", [0, 1, 2, 3, 4])
+def test_smoothing_in_place(mg, sweeps, precision, gamma2):
+    """x_in == x_out, x_in kept, x_in NULL and x_out full of NaN: the same bits as sweep by sweep."""
+    cfg = syn.small_config(10, 9, levels=2, seed=syn.BASE_SEED + 940, gamma2=gamma2)
+    inp = syn.make_inputs(cfg)
+    h = mg.mg_setup_config(cfg, inp, precision=precision)
+    for level in range(2):
+        n = h.level_cells(level)
+        b, x0 = (torch.from_numpy(syn.normal(s, 0, n)).cuda() for s in (3, 4))
+        for start in (None, x0):
+            ref = torch.zeros_like(b) if start is None else start.clone()
+            for i in range(sweeps):
+                y = torch.full_like(b, float("nan"))
+                mg.mg_smooth(h, level, b, None if i == 0 and start is None else ref, y, 1)
+                ref = y
+            x = torch.full_like(b, float("nan"))
+            mg.mg_smooth(h, level, b, start, x, sweeps)
+            assert torch.equal(x, ref)
+            if start is not None:
+                x = start.clone()
+                mg.mg_smooth(h, level, b, x, x, sweeps)
+                assert torch.equal(x, ref)
+    h.destroy()
