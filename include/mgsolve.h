@@ -256,8 +256,8 @@ mg_status mg_level_apply(mg_handle* h, int32_t level, const double* x, double* y
 /* x_out = BlockJacobi(H^(level), b, x_in, omega, sweeps) (Eq. jacobi), x_in == NULL meaning
  * a zero initial guess.  x_in and x_out may be the same array; b must not overlap x_out.
  * A handle whose V-cycle is not MG_FP64 packs the level's FP64 data at the first call of this,
- * mg_smooth_noalloc or mg_residual_restrict for a level; for levels of more than MG_NOALLOC_MAX_CELLS
- * cells that call allocates 40 bytes per cell for it (MG_ERR_NOMEM where there is no room). */
+ * mg_smooth_noalloc or mg_residual_restrict for a level, which waits for that; for levels of more than
+ * MG_NOALLOC_MAX_CELLS cells that call allocates 40 bytes per cell for it (MG_ERR_NOMEM where there is no room). */
 mg_status mg_smooth(mg_handle* h, int32_t level, const double* b, const double* x_in,
                     double* x_out, int32_t sweeps, void* stream);
 

@@ -125,7 +125,8 @@ struct mg_handle {
     // operator with its sums, the orthogonalisation and the read-back of <r, r>, captured on
     // `cap` the first time and replayed on the caller's stream afterwards
     cudaStream_t cap = nullptr;
-    cudaStream_t run = nullptr;   // the handle's stream inside an ensemble solve
+    cudaStream_t run = nullptr;   // the handle's stream inside an ensemble solve, and for ready64 under capture
+    std::mutex pack_mutex;        // ready64
     cudaEvent_t evx = nullptr;    // ordering event (no timing)
     cudaGraphExec_t gexec[3][mg::MAXR] = {};
     bool graphs_off = false;
@@ -1230,24 +1231,30 @@ mg_status pack64(mg_handle* h, int l, cudaStream_t s) {
 
 // A handle whose V-cycle is not in FP64 has FP64 level data for mg_smooth, mg_smooth_noalloc and
 // mg_residual_restrict alone (40 of about 300 bytes per cell, C96L70: 0.12 ms for the finest level).  They are
-// packed when one of these first asks, on its stream, and from then on by mg_set_coefficients; levels that
-// mg_smooth_noalloc takes have their memory from set-up, others from that first call.  A call under stream
-// capture records the packing, which has then not run yet.
+// packed when one of these first asks, and from then on by mg_set_coefficients; levels that mg_smooth_noalloc
+// takes have their memory from set-up, others from that first call.  The first call waits for the packing, so
+// that calls on other streams and from other threads find the data complete.  Under stream capture it runs
+// on the handle's own stream (the couplings are in place: set-up and mg_set_coefficients synchronise), so that a
+// graph does not pack again each time it is replayed; only then, because a process that has run work on
+// several streams launches slower from then on (C64L40 solve 1.57 -> 1.67 ms after seven handles' streams).
 mg_status ready64(mg_handle* h, int l, cudaStream_t s) {
     DevLevel& d = h->lv[l];
+    std::lock_guard<std::mutex> lock(h->pack_mutex);
     if (d.packed64) return MG_OK;
     cudaStreamCaptureStatus cst;
     CK(cudaStreamIsCapturing(s, &cst));
-    if (!d.tv64) {
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // (allocation is no work on the stream)
-        CK(cudaThreadExchangeStreamCaptureMode(&mode));
-        const mg_status st = alloc64(h, l);
-        CK(cudaThreadExchangeStreamCaptureMode(&mode));
-        TRY(st);
-    }
-    TRY(pack64(h, l, s));
-    d.wants64 = true;
-    d.packed64 = cst == cudaStreamCaptureStatusNone;
+    if (cst != cudaStreamCaptureStatusNone) s = h->run;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // (none of this is work of a stream under capture)
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    const mg_status st = [&]() -> mg_status {
+        if (!d.tv64) TRY(alloc64(h, l));
+        TRY(pack64(h, l, s));
+        CK(cudaStreamSynchronize(s));
+        return MG_OK;
+    }();
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    TRY(st);
+    d.wants64 = d.packed64 = true;
     return MG_OK;
 }
 

@@ -1,4 +1,6 @@
 """What a handle holds and what its set-up does."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -167,3 +169,44 @@ def test_smoothing_in_place(mg, sweeps, precision, gamma2):
                 mg.mg_smooth(h, level, b, x, x, sweeps)
                 assert torch.equal(x, ref)
     h.destroy()
+
+
+def test_first_fp64_calls_on_several_streams_and_threads(mg):
+    """Calls on other streams and from other threads than the one that packs an FP32 handle's FP64 data: the
+    first one's stream is busy, so that what it enqueued would come last."""
+    cfg = syn.small_config(128, 30, levels=2, seed=syn.BASE_SEED + 950)
+    inp = syn.make_inputs(cfg)
+    h = [mg.mg_setup_config(cfg, inp, precision=p) for p in ("fp64", "fp32", "fp32")]
+    b, x0 = torch.from_numpy(inp["rhs"]).cuda().ravel(), torch.from_numpy(syn.normal(9, 0, cfg.ncell)).cuda()
+    ref = torch.empty(h[0].level_cells(1), dtype=torch.float64, device="cuda")
+    mg.mg_residual_restrict(h[0], 0, b, x0, ref)
+    torch.cuda.synchronize()
+    busy = torch.empty(4096, 4096, device="cuda")
+    for hd, threads in ((h[1], False), (h[2], True)):
+        streams = [torch.cuda.Stream() for _ in range(4)]
+        out = [torch.empty_like(ref) for _ in streams]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(streams[0]):
+            for _ in range(20):
+                busy = busy @ busy
+        start, status = threading.Barrier(len(streams)), [None] * len(streams)
+
+        def call(i):
+            if threads:
+                start.wait()
+            status[i] = mg.load().mg_residual_restrict(hd.ptr, 0, b.data_ptr(), x0.data_ptr(), out[i].data_ptr(),
+                                                       streams[i].cuda_stream)
+
+        ts = [threading.Thread(target=call, args=(i,)) for i in range(len(streams))]
+        for t in ts:
+            t.start()
+            if not threads:
+                t.join()
+        for t in ts:
+            t.join()
+        torch.cuda.synchronize()
+        assert status == [mg.MG_OK] * len(streams)
+        for o in out:
+            assert torch.equal(o, ref)
+    for hd in h:
+        hd.destroy()
