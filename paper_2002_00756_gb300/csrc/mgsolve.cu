@@ -392,14 +392,15 @@ inline int sweep_mode(const void* x, const void* xc) {
     return xc ? (x ? mg::XM_PROLONG : mg::XM_PROLONG0) : (x ? mg::XM_PLAIN : mg::XM_ZERO);
 }
 
-// levels per thread of the residual + restriction: long chunks (fewer prologues) where the level
-// fills the GPU several times over (C192L70 60 us with 35, 62 with 8, events included; C96L70 21 with 2 or
-// 6, 22 with 12); the small levels need every thread (one level per thread at C48L30: 6.5 us a launch
-// against 13 with eight)
+// levels per thread of the residual + restriction: a few (fewer prologues) where the level fills the GPU
+// several times over, one on small levels, which need every thread (C48L30: 6.5 us a launch against 13 with
+// eight).  V-cycle on two levels with 1 / 2 / 4 / 8 / 35 a thread: C192L70 482/478/477/480/480 us (FP64
+// 2218/2191/2179/2178/2221), C144L36 FP64 763/756/754/756/783, C160L20 162/162/161/162/176, C130L128
+// 674/669/670/672/672; C96L70's restriction 21 us with 2 or 6, 22 with 12.
 inline int restrict_chunk(const mg_handle* h, int lev) {
     const DevLevel& d = h->lv[lev];
     if (d.restrict_kc > 0) return d.restrict_kc;
-    return d.ncol >= 100000 ? 35 : (double)h->nlev * d.ncol >= 2e6 ? 2 : 1;
+    return d.ncol >= 100000 ? 4 : (double)h->nlev * d.ncol >= 2e6 ? 2 : 1;
 }
 
 // One FP64 block-Jacobi sweep on level `lev`.  The iterate it starts from is x (NULL: zero) plus,
